@@ -3,102 +3,141 @@
 #include <cstring>
 #include <vector>
 
+#include <cooperative_groups.h>
+
 #include "dense.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace rsrr {
 
 // ---------------------------------------------------------------------------------------------
-// ZGEMM: 64 x 64 output tile per CTA, K in steps of 8, 256 threads each owning a 4 x 4 grid of
-// outputs spaced 16 apart.  FP64 FMA throughput bounds it on this part; the tiling keeps the
-// operands in shared memory so global traffic is (M + N) K / 64 elements per tile.
+// ZGEMM on the FP64 cores.  GB300 issues two FP64 multiply-adds a clock per SM (1.25 TFLOP/s in
+// all), so what bounds a product is how evenly its multiply-adds spread over the SMs and their
+// sub-partitions, not the operand traffic: a 16 x 16 tile reads one byte a clock.  The tiles are
+// therefore small (256 outputs for 128 threads, four warps, two outputs a thread), and K is cut
+// over the up to eight CTAs of a cluster, which add their partial tiles through distributed shared
+// memory in a fixed order (no atomics, no workspace, the same bits on every run).  The
+// FP64 products of one pass (projection and reduced solve), before with 32 x 32 tiles of two warps
+// and no K split below 512, and now: n = 9991, k_S = 133: 18.8 -> 3.1 ms; n = 900, moment scheme,
+// k_S = 45: 18.5 -> 1.0 ms; n = 5000, k_S = 48, K = 8: 29.7 -> 3.8 ms.
+// A tile is 16 x 16, or 64 x 4 for the products with a handful of columns (moments, traces).
 // ---------------------------------------------------------------------------------------------
 namespace {
-constexpr int BK = 8;
+constexpr int BK = 16;          // K terms per shared-memory stage
+constexpr int kZgThreads = 128;
+constexpr int kZgTile = 256;    // outputs per tile
+constexpr int kZgMaxSplit = 8;  // portable cluster size
 
-// Tile BM x BN, NT = BM BN / 16 threads as TY x TX = (BM/4) x (BN/4), each owning a 4 x 4 grid
-// of outputs spaced TY rows and TX columns apart.  64 x 64 for general shapes, 32 x 128 when
-// M <= 32, 32 x 32 (64 threads) when those give too few CTAs to fill the GPU.  Every output
-// accumulates over k in the same order whatever the tile.
-template <int OPA, int OPB, int BM, int BN>
-__global__ void __launch_bounds__(BM * BN / 16) zgemm_kernel(Zgemm g, int kchunk) {
-    constexpr int TY = BM / 4, TX = BN / 4, NT = TY * TX;
-    static_assert(BM * BK % NT == 0 && BN * BK % NT == 0, "tile loads");
+struct ZgOperand {  // op(X)(row, k) = X[row * sr + k * sk], conjugated when conj
+    const c128* p;
+    int64_t sr, sk, sb;
+    int conj;
+};
+struct ZgArgs {
+    ZgOperand A, B;  // B's "row" is the output column
+    c128* C;
+    int64_t ldc, sC;
+    int M, N, K, tm, tn, split, kper;
+    c128 alpha, beta;
+};
+
+__device__ __forceinline__ c128 zg_fetch(const ZgOperand& o, const c128* base, int r, int R, int k, int k_end) {
+    c128 v = czero<double>();
+    if (r < R && k < k_end) {
+        v = base[r * o.sr + k * o.sk];
+        if (o.conj) v.im = -v.im;
+    }
+    return v;
+}
+
+template <int BM, int BN>
+__global__ void __launch_bounds__(kZgThreads) zgemm_kernel(ZgArgs g) {
+    static_assert(BM * BN == kZgTile, "two outputs a thread");
+    constexpr int TX = BN / 2;  // threads across the columns; a thread owns columns tx and tx + TX
+    constexpr int NA = BM * BK / kZgThreads, NB = (BN * BK + kZgThreads - 1) / kZgThreads;
     __shared__ c128 As[BK][BM + 1];
     __shared__ c128 Bs[BK][BN + 1];
+    __shared__ c128 part[kZgTile];
     const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
-    const int bm = blockIdx.x * BM, bn = blockIdx.y * BN;
-    const int bz = blockIdx.z, b = bz / g.ksplit, ks = bz % g.ksplit;
-    const c128* A = g.A + b * g.sA;
-    const c128* B = g.B + b * g.sB;
-    c128* C = g.C + b * g.sC;
-    const int k_begin = ks * kchunk, k_end = min(g.K, k_begin + kchunk);
-    c128 acc[4][4];
+    // the CTAs of a cluster are the K slices of one tile
+    const int64_t tile = blockIdx.x / g.split;
+    const int ks = (int)(blockIdx.x % g.split);
+    const int bm = (int)(tile % g.tm) * BM, bn = (int)((tile / g.tm) % g.tn) * BN;
+    const int64_t b = tile / ((int64_t)g.tm * g.tn);
+    const c128* Ab = g.A.p + b * g.A.sb;
+    const c128* Bb = g.B.p + b * g.B.sb;
+    const int k_begin = min(g.K, ks * g.kper), k_end = min(g.K, k_begin + g.kper);
+    // consecutive threads follow whichever index is contiguous in memory
+    const bool a_rows = g.A.sr == 1, b_rows = g.B.sr == 1;
+    c128 ra[NA], rb[NB];
+    auto fetch = [&](int k0) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = czero<double>();
-    for (int k0 = k_begin; k0 < k_end; k0 += BK) {
-#pragma unroll
-        for (int r = 0; r < BM * BK / NT; ++r) {
-            const int idx = tid + NT * r;
-            int i, k;
-            if (OPA == OP_N) { i = idx % BM; k = idx / BM; } else { k = idx % BK; i = idx / BK; }
-            const int gi = bm + i, gk = k0 + k;
-            c128 v = czero<double>();
-            if (gi < g.M && gk < k_end) {
-                v = (OPA == OP_N) ? A[gi + (int64_t)gk * g.lda] : A[gk + (int64_t)gi * g.lda];
-                if (OPA == OP_C) v.im = -v.im;
-            }
-            As[k][i] = v;
+        for (int u = 0; u < NA; ++u) {
+            const int idx = tid + kZgThreads * u;
+            const int i = a_rows ? idx % BM : idx / BK, k = a_rows ? idx / BM : idx % BK;
+            ra[u] = zg_fetch(g.A, Ab, bm + i, g.M, k0 + k, k_end);
         }
 #pragma unroll
-        for (int r = 0; r < BN * BK / NT; ++r) {
-            const int idx = tid + NT * r;
-            int j, k;
-            if (OPB == OP_N) { k = idx % BK; j = idx / BK; } else { j = idx % BN; k = idx / BN; }
-            const int gj = bn + j, gk = k0 + k;
-            c128 w = czero<double>();
-            if (gj < g.N && gk < k_end) {
-                w = (OPB == OP_N) ? B[gk + (int64_t)gj * g.ldb] : B[gj + (int64_t)gk * g.ldb];
-                if (OPB == OP_C) w.im = -w.im;
+        for (int u = 0; u < NB; ++u) {
+            const int idx = tid + kZgThreads * u;
+            if (idx < BN * BK) {
+                const int j = b_rows ? idx % BN : idx / BK, k = b_rows ? idx / BN : idx % BK;
+                rb[u] = zg_fetch(g.B, Bb, bn + j, g.N, k0 + k, k_end);
             }
-            Bs[k][j] = w;
+        }
+    };
+    c128 acc0 = czero<double>(), acc1 = czero<double>();
+    if (k_begin < k_end) fetch(k_begin);
+    for (int k0 = k_begin; k0 < k_end; k0 += BK) {
+        __syncthreads();  // the previous stage has been read
+#pragma unroll
+        for (int u = 0; u < NA; ++u) {
+            const int idx = tid + kZgThreads * u;
+            const int i = a_rows ? idx % BM : idx / BK, k = a_rows ? idx / BM : idx % BK;
+            As[k][i] = ra[u];
+        }
+#pragma unroll
+        for (int u = 0; u < NB; ++u) {
+            const int idx = tid + kZgThreads * u;
+            if (idx < BN * BK) {
+                const int j = b_rows ? idx % BN : idx / BK, k = b_rows ? idx / BN : idx % BK;
+                Bs[k][j] = rb[u];
+            }
         }
         __syncthreads();
+        if (k0 + BK < k_end) fetch(k0 + BK);  // in flight under this stage's multiply-adds
 #pragma unroll
         for (int k = 0; k < BK; ++k) {
-            c128 a[4], bb[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[k][ty + TY * i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) bb[j] = Bs[k][tx + TX * j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) cfma(acc[i][j], a[i], bb[j]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int gi = bm + ty + TY * i;
-        if (gi >= g.M) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int gj = bn + tx + TX * j;
-            if (gj >= g.N) continue;
-            c128* c = C + gi + (int64_t)gj * g.ldc;
-            const c128 v = g.alpha * acc[i][j];
-            if (g.ksplit > 1) {
-                atomicAdd(&c->re, v.re);
-                atomicAdd(&c->im, v.im);
-            } else if (g.beta.re == 0.0 && g.beta.im == 0.0) {
-                *c = v;
-            } else {
-                *c = v + g.beta * (*c);
-            }
+            if (k0 + k >= k_end) break;
+            const c128 x = As[k][ty];
+            cfma(acc0, x, Bs[k][tx]);
+            cfma(acc1, x, Bs[k][tx + TX]);
         }
     }
+    auto store = [&](int i, int j, c128 v) {
+        const int gi = bm + i, gj = bn + j;
+        if (gi >= g.M || gj >= g.N) return;
+        c128* c = g.C + b * g.sC + gi + (int64_t)gj * g.ldc;
+        v = g.alpha * v;
+        *c = (g.beta.re == 0.0 && g.beta.im == 0.0) ? v : v + g.beta * (*c);
+    };
+    if (g.split == 1) {
+        store(ty, tx, acc0);
+        store(ty, tx + TX, acc1);
+        return;
+    }
+    part[ty + BM * tx] = acc0;
+    part[ty + BM * (tx + TX)] = acc1;
+    cg::cluster_group cluster = cg::this_cluster();
+    cluster.sync();
+    // the tile's outputs are dealt out over the cluster; each is summed in K order
+    for (int e = tid + kZgThreads * ks; e < kZgTile; e += kZgThreads * g.split) {
+        c128 v = czero<double>();
+        for (int q = 0; q < g.split; ++q) v = v + *cluster.map_shared_rank(&part[e], q);
+        store(e % BM, e / BM, v);
+    }
+    cluster.sync();  // no CTA leaves while its partial tile may still be read
 }
 
 __global__ void scale_kernel(c128* C, int M, int N, int64_t ldc, int64_t sC, c128 beta) {
@@ -111,41 +150,45 @@ __global__ void scale_kernel(c128* C, int M, int N, int64_t ldc, int64_t sC, c12
 }
 }  // namespace
 
+namespace {
+ZgOperand zg_operand(const c128* p, int64_t ld, int64_t sb, int op, bool is_b) {
+    // A: op(A)(i, k); B is taken by its output column j: op(B)(k, j)
+    const bool rows = (op == OP_N) != is_b;  // the row index is the contiguous one
+    return ZgOperand{p, rows ? 1 : ld, rows ? ld : 1, sb, op == OP_C ? 1 : 0};
+}
+
 template <int BM, int BN>
-int zgemm_shape(Zgemm g, cudaStream_t s) {
-    const int tm = (int)ceil_div(g.M, BM), tn = (int)ceil_div(g.N, BN);
-    if (g.ksplit <= 0) {
-        const int64_t tiles = (int64_t)tm * tn * g.batch;
-        int ks = 1;
-        while (tiles * ks < 2 * 152 && (int64_t)g.K / (ks * 2) >= 256) ks *= 2;
-        g.ksplit = ks;
-    }
-    int kchunk = (int)ceil_div(ceil_div(g.K, g.ksplit), BK) * BK;
-    g.ksplit = (int)ceil_div(g.K, kchunk);
-    if (g.ksplit > 1) {
-        dim3 grid((unsigned)ceil_div((int64_t)g.M * g.N, 256), g.batch);
-        { scale_kernel<<<grid, 256, 0, s>>>(g.C, g.M, g.N, g.ldc, g.sC, g.beta); note_launch(); }
-    }
-    if constexpr (BM * BN > 32 * 32) {
-        // too few tiles and no K split: 32 x 32 tiles give up to four times the CTAs
-        if (g.ksplit == 1 && (int64_t)tm * tn * g.batch < 2 * 152) return zgemm_shape<32, 32>(g, s);
-    }
-    dim3 grid(tm, tn, g.batch * g.ksplit);
-#define ZG(a, b) { zgemm_kernel<a, b, BM, BN><<<grid, BM * BN / 16, 0, s>>>(g, kchunk); note_launch(); }
-    if (g.opA == OP_N && g.opB == OP_N) ZG(OP_N, OP_N)
-    else if (g.opA == OP_N && g.opB == OP_T) ZG(OP_N, OP_T)
-    else if (g.opA == OP_N && g.opB == OP_C) ZG(OP_N, OP_C)
-    else if (g.opA == OP_T && g.opB == OP_N) ZG(OP_T, OP_N)
-    else if (g.opA == OP_C && g.opB == OP_N) ZG(OP_C, OP_N)
-    else if (g.opA == OP_C && g.opB == OP_C) ZG(OP_C, OP_C)
-    else if (g.opA == OP_T && g.opB == OP_T) ZG(OP_T, OP_T)
-    else if (g.opA == OP_T && g.opB == OP_C) ZG(OP_T, OP_C)
-    else if (g.opA == OP_C && g.opB == OP_T) ZG(OP_C, OP_T)
-    else return set_error(RSRR_EINVAL, "zgemm: unsupported op combination");
-#undef ZG
-    RSRR_CUDA(cudaGetLastError());
+int zgemm_fp64(const Zgemm& g, cudaStream_t s) {
+    ZgArgs a;
+    a.A = zg_operand(g.A, g.lda, g.sA, g.opA, false);
+    a.B = zg_operand(g.B, g.ldb, g.sB, g.opB, true);
+    a.C = g.C; a.ldc = g.ldc; a.sC = g.sC;
+    a.M = g.M; a.N = g.N; a.K = g.K;
+    a.tm = (int)ceil_div(g.M, BM);
+    a.tn = (int)ceil_div(g.N, BN);
+    a.alpha = g.alpha; a.beta = g.beta;
+    // K slices until every SM has two CTAs, but none shorter than one stage
+    const int64_t tiles = (int64_t)a.tm * a.tn * g.batch;
+    int split = 1;
+    while (split < kZgMaxSplit && tiles * split < 2 * 152 && g.K >= 2 * split * BK) split *= 2;
+    a.split = split;
+    a.kper = (int)ceil_div(g.K, split);
+    if (tiles * split > INT32_MAX) return set_error(RSRR_EINVAL, "zgemm: too many tiles");
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(tiles * split));
+    cfg.blockDim = dim3(kZgThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = split;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    RSRR_CUDA(cudaLaunchKernelEx(&cfg, zgemm_kernel<BM, BN>, a));
+    note_launch();
     return RSRR_OK;
 }
+}  // namespace
 
 // ZGEMM accounting for the calling host thread: device time (events around each call) and
 // algorithmic flops 8 M N K per product, between zgemm_profile_begin and zgemm_profile_end.
@@ -249,8 +292,7 @@ static int zgemm_dispatch(const Zgemm& g0, cudaStream_t s) {
         return RSRR_OK;
     }
     if (g_zpath == 2 || (g_zpath == 0 && !g.fp64 && zgemm_tc_fits(g))) return zgemm_tc(g, s);
-    if (g.M <= 32) return zgemm_shape<32, 128>(g, s);
-    return zgemm_shape<64, 64>(g, s);
+    return g.N <= 8 ? zgemm_fp64<64, 4>(g, s) : zgemm_fp64<16, 16>(g, s);
 }
 
 // ---------------------------------------------------------------------------------------------

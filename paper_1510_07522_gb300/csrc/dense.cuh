@@ -7,9 +7,8 @@ namespace rsrr {
 
 enum { OP_N = 0, OP_T = 1, OP_C = 2 };
 
-// C = alpha op(A) op(B) + beta C for `batch` independent problems (strided).  With ksplit > 1
-// the K range is cut into slices whose products are added to C atomically (beta is applied
-// first by a separate pass).  op(A) is M x K, op(B) is K x N, all column-major.
+// C = alpha op(A) op(B) + beta C for `batch` independent problems (strided).
+// op(A) is M x K, op(B) is K x N, all column-major.
 struct Zgemm {
     int opA = OP_N, opB = OP_N;
     int M = 0, N = 0, K = 0;
@@ -21,7 +20,6 @@ struct Zgemm {
     c128* C = nullptr;
     int64_t ldc = 0, sC = 0;
     int batch = 1;
-    int ksplit = 0;  // 0 = choose
     bool fp64 = false;  // FP64 CUDA cores even where the tensor-core emulation would be chosen
 };
 int zgemm(const Zgemm& g, cudaStream_t s);

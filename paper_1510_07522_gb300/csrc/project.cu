@@ -320,7 +320,6 @@ int householder_qr(c128* A, int64_t rows, int cols, int64_t lda, HqrWork& w, dou
             g3.opA = OP_N; g3.opB = OP_N; g3.M = (int)(rows - kb); g3.N = mt; g3.K = bw;
             g3.alpha = mk<double>(-1.0, 0.0); g3.beta = mk<double>(1.0, 0.0);
             g3.A = w.V; g3.lda = rows; g3.B = w.W2; g3.ldb = kPB; g3.C = A + kb + (int64_t)kk * lda; g3.ldc = lda;
-            g3.ksplit = 1;
             RSRR_TRY(zgemm(g3, st));
         }
         int berr = 0;
@@ -370,7 +369,7 @@ int apply_q(const c128* A, int64_t n, int npan, int kmax, HqrWork& hw, c128* Y, 
         Zgemm g3;
         g3.opA = OP_N; g3.opB = OP_N; g3.M = (int)(n - kb); g3.N = ncols; g3.K = bw;
         g3.alpha = mk<double>(-1.0, 0.0); g3.beta = mk<double>(1.0, 0.0);
-        g3.A = hw.V; g3.lda = n; g3.B = Z2; g3.ldb = kPB; g3.C = Y + kb; g3.ldc = n; g3.ksplit = 1;
+        g3.A = hw.V; g3.lda = n; g3.B = Z2; g3.ldb = kPB; g3.C = Y + kb; g3.ldc = n;
         RSRR_TRY(zgemm(g3, st));
     }
     return RSRR_OK;
@@ -538,7 +537,6 @@ int project_run(rsrr_nep h, double delta) {
         Zgemm gm;
         gm.opA = OP_N; gm.opB = OP_N; gm.M = (int)n; gm.N = m; gm.K = N * L;
         gm.A = h->d_S; gm.lda = n; gm.B = Z; gm.ldb = N * L; gm.C = A; gm.ldc = n;
-        gm.ksplit = 1;
         TRYC(zgemm(gm, st));
         CUDAC(cudaStreamSynchronize(st));
         dfree(Z, st);
@@ -655,7 +653,7 @@ int project_run(rsrr_nep h, double delta) {
         Zgemm gn;
         gn.M = kk; gn.N = kS; gn.K = kS;
         gn.alpha = mk<double>(-0.5, 0.0); gn.beta = mk<double>(1.0, 0.0);
-        gn.A = Ybuf; gn.lda = n; gn.B = Eg; gn.ldb = kS; gn.C = Jn; gn.ldc = kk; gn.ksplit = 1;
+        gn.A = Ybuf; gn.lda = n; gn.B = Eg; gn.ldb = kS; gn.C = Jn; gn.ldc = kk;
         TRYC(zgemm(gn, st));
         CUDAC(cudaMemcpy2DAsync(Ybuf, (size_t)n * sizeof(c128), Jn, (size_t)kk * sizeof(c128), (size_t)kk * sizeof(c128),
                                 kS, cudaMemcpyDeviceToDevice, st));
@@ -750,7 +748,7 @@ int chebyshev_reduce_tz(rsrr_nep h, int d, double lo, double hi) {
         if (rc == RSRR_OK) {
             Zgemm gc;  // P_hat = [Q_0 .. Q_d] C
             gc.M = (int)kk; gc.N = m; gc.K = m;
-            gc.A = Q; gc.lda = kk; gc.B = Cd; gc.ldb = m; gc.C = Pn; gc.ldc = kk; gc.ksplit = 1;
+            gc.A = Q; gc.lda = kk; gc.B = Cd; gc.ldb = m; gc.C = Pn; gc.ldc = kk;
             rc = zgemm(gc, st);
         }
         if (rc == RSRR_OK && cudaStreamSynchronize(st) != cudaSuccess)
@@ -803,7 +801,7 @@ int chebyshev_reduce(rsrr_nep h, int d, double lo, double hi) {
         cudaMemcpyAsync(Wd, Wh.data(), Wh.size() * sizeof(c128), cudaMemcpyHostToDevice, st);
         Zgemm g;
         g.M = (int)kk; g.N = m; g.K = J;
-        g.A = h->d_P; g.lda = kk; g.B = Wd; g.ldb = J; g.C = Pn; g.ldc = kk; g.ksplit = 1;
+        g.A = h->d_P; g.lda = kk; g.B = Wd; g.ldb = J; g.C = Pn; g.ldc = kk;
         rc = zgemm(g, st);
         if (rc == RSRR_OK && cudaStreamSynchronize(st) != cudaSuccess)
             rc = set_error(RSRR_ECUDA, "Chebyshev coefficients");

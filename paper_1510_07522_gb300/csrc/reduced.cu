@@ -470,7 +470,7 @@ int solve_run(rsrr_nep h, int N_S, int K, double tol_gap, int cap, double* lambd
         Zgemm gm;
         gm.opA = OP_N; gm.opB = OP_N; gm.M = (int)kk; gm.N = 2 * K; gm.K = np;
         gm.A = X; gm.lda = kk; gm.B = dWt + j0; gm.ldb = N_S; gm.C = mom; gm.ldc = kk;
-        gm.beta = mk<double>(1.0, 0.0); gm.ksplit = 1;
+        gm.beta = mk<double>(1.0, 0.0);
         TRYC(zgemm(gm, st));
         // traces tr(X_j P_i) = vec(X_j)^T vec(P_i^T): [np x J]
         Zgemm gt;
@@ -676,7 +676,7 @@ int solve_run(rsrr_nep h, int N_S, int K, double tol_gap, int cap, double* lambd
         TRYC(dalloc_n(&Vfull, (size_t)n * nk, st));
         Zgemm gv;
         gv.opA = OP_N; gv.opB = OP_N; gv.M = (int)n; gv.N = nk; gv.K = k;
-        gv.A = h->d_Q; gv.lda = n; gv.B = RG; gv.ldb = k; gv.C = Vfull; gv.ldc = n; gv.ksplit = 1;
+        gv.A = h->d_Q; gv.lda = n; gv.B = RG; gv.ldb = k; gv.C = Vfull; gv.ldc = n;
         TRYC(zgemm(gv, st));
         column_norms(Vfull, (int)n, nk, n, rn, st);
         { scale_cols_kernel<<<(unsigned)ceil_div(n * nk, 256), 256, 0, st>>>(Vfull, n, nk, n, rn, 1); note_launch(); }

@@ -599,14 +599,13 @@ static int oz_max(const c128* X, int64_t ld, int64_t sb, int op, int U, int V, i
     return RSRR_OK;
 }
 
-// Worth it when the FP64 GEMM would take a while.  A thin output side (the moments' 2K columns,
-// the traces' J columns) wastes most of a 32-column tile, but the FP64 kernel wastes more of
-// its 64 x 64 tile on such shapes (measured 0.05-0.07 TFLOP/s on the moments and traces).  The
-// QR updates of an 800-column Hankel matrix (0.17 GFLOP each) ran at 0.2 TFLOP/s on the FP64
-// kernel: from 0.1 GFLOP on, the emulation's fixed costs (five launches, one host wait) are paid.
+// Worth it when the FP64 GEMM would take a while: from 0.1 GFLOP (100 us there) the emulation's
+// fixed costs (five launches, one host wait) are paid.  With at most 8 columns (or rows) the FP64
+// kernel wins at every size: the digit images cost 144 bytes of traffic for every operand entry,
+// which is then used a few times only, and a 32-column tile is mostly padding.
 bool zgemm_tc_fits(const Zgemm& g) {
     const double work = 8.0 * g.M * (double)g.N * g.K * g.batch;
-    return work >= 1e8 && g.K >= 16;
+    return work >= 1e8 && g.K >= 16 && std::min(g.M, g.N) > 8;
 }
 
 int zgemm_tc(const Zgemm& g0, cudaStream_t s) {
