@@ -3,7 +3,7 @@
 //
 //   1. Householder QR of S_hat (n x m, m = N L) in panels of 32 columns.  The point blocks are
 //      taken in bit-reversed order (0, N/2, N/4, 3N/4, ...) so early columns sample the whole
-//      contour.  Each panel is factored by one cooperative kernel (two grid barriers per
+//      contour.  Each panel is factored by one cooperative kernel (one grid barrier per
 //      column); the trailing matrix is updated with the compact WY form by three ZGEMMs.
 //      After every panel the remaining trailing block is measured (Frobenius norm, then a
 //      power-iteration estimate of its 2-norm with a safety factor of 3); once its 2-norm is
@@ -35,139 +35,180 @@ constexpr int kPB = 32;  // panel width
 struct PanelArgs {
     c128* A;
     int64_t lda;
-    int n, kb, bw;
+    int n, kb, bw, per;  // per: rows of a CTA
     c128* tau;
-    c128* T;       // bw x bw, column-major
-    double* part;  // [G]
-    c128* alpha;   // [1]
-    c128* part2;   // [G][kPB]
-    c128* part3;   // [G][kPB*kPB]
-    c128* Y;       // [kPB*kPB]
+    c128* T;             // bw x bw, column-major
+    c128* V;             // rows kb..n-1 of the reflectors, unit diagonal, zeros above
+    int64_t ldv;
+    double* part;        // [2][G][2 kPB] partial inner products
+    c128* row;           // [2][kPB] the pivot row
+    int resident;        // the CTA's rows of the panel stay in shared memory
     GridBar gb;
 };
 
+// One panel of the Householder QR (LAPACK zlarfg convention), a cooperative kernel.  What bounds it
+// is the FP64 rate (two multiply-adds a clock per SM: 0.4 ms for 40000 rows) and, below some
+// thousand rows, the chain of 32 columns.  A column costs one grid barrier: the inner products of
+// the unscaled column x with every column of the panel (its own norm, v^H A for the columns right
+// of it, V^H v for T on its left) are summed before the barrier, v = [1; scal x] and
+// w_c = conj(scal) x^H a_c + a_dc follow from them and from the pivot row, and every CTA forms the
+// reflector for itself.  A CTA keeps its rows (a multiple of 32, lane = row) in shared memory for
+// the whole panel; more than that fit (about 63000 rows) stay in global memory.  A full-warp FP64
+// addition occupies its sub-partition for 64 clocks, so the warps' sums are reduce-scattered
+// (9 additions for 8 values, not 40).  With two barriers a column, panels in global memory and V, T
+// and the sums in passes of their own, the 48 panels of a pass at n = 40000 took 47.4 ms, now 21.7
+// (23 panels at n = 9991: 18.0, now 7.3).
 __global__ void __launch_bounds__(256) hqr_panel_kernel(PanelArgs a) {
-    const int G = gridDim.x, g = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int NW = 8;
-    const int rows = a.n - a.kb;
-    const int per = (rows + G - 1) / G;
-    const int r0 = min(a.n, a.kb + g * per), r1 = min(a.n, r0 + per);
-    __shared__ c128 s_w[kPB];
-    __shared__ c128 s_tau, s_scal;
+    extern __shared__ __align__(16) unsigned char hqr_dyn[];
+    constexpr int NW = 8, NV = 2 * kPB;  // warps; doubles of one CTA's inner products
+    __shared__ double s_red[4][NV];
+    __shared__ double s_D[NV];
+    __shared__ c128 s_row[kPB], s_g[kPB], s_tau[kPB];
+    __shared__ c128 s_Y[kPB * (kPB - 1) / 2];  // V^H V above the diagonal, packed by columns
+    __shared__ c128 s_scal;
+    __shared__ double s_beta;
     __shared__ int s_ident;
-    const int cend = a.kb + a.bw;
-    for (int j = 0; j < a.bw; ++j) {
-        const int c = a.kb + j, d = c;
-        c128* col = a.A + (int64_t)c * a.lda;
-        // phase 1: partial squared norm below the diagonal, and alpha
-        double ss = 0.0;
-        for (int i = max(r0, d + 1) + tid; i < r1; i += 256) ss += cnorm2(col[i]);
-        ss = block_sum_all(ss);
-        if (tid == 0) {
-            a.part[g] = ss;
-            if (d >= r0 && d < r1) *a.alpha = col[d];
-        }
-        if (!grid_sync(a.gb)) return;
-        // phase 2: reflector (LAPACK zlarfg convention: real beta), scale own rows, partial dots
-        double xs = 0.0;
-        for (int t = tid; t < G; t += 256) xs += a.part[t];
-        xs = block_sum_all(xs);
-        if (tid == 0) {
-            const c128 al = *a.alpha;
-            if (xs == 0.0 && al.im == 0.0) {
-                s_ident = 1;
-                s_tau = czero<double>();
-                s_scal = mk<double>(1.0, 0.0);
-            } else {
-                const double beta = -copysign(sqrt(al.re * al.re + al.im * al.im + xs), al.re);
-                s_ident = 0;
-                s_tau = mk<double>((beta - al.re) / beta, -al.im / beta);
-                s_scal = crecip(mk<double>(al.re - beta, al.im));
-                if (d >= r0 && d < r1) col[d] = mk<double>(beta, 0.0);
-            }
-            if (g == 0) a.tau[c] = s_tau;
-        }
-        __syncthreads();
-        const bool ident = s_ident != 0;
-        if (!ident) {
-            const c128 sc = s_scal;
-            for (int i = max(r0, d + 1) + tid; i < r1; i += 256) col[i] = col[i] * sc;
-        }
-        __syncthreads();
-        for (int cc = c + 1 + warp; cc < cend; cc += NW) {
-            const c128* x = a.A + (int64_t)cc * a.lda;
-            c128 w = czero<double>();
-            for (int i = max(r0, d) + lane; i < r1; i += 32) {
-                const c128 v = (i == d) ? mk<double>(1.0, 0.0) : col[i];
-                cfma_conj(w, v, x[i]);
-            }
-            for (int off = 16; off; off >>= 1) {
-                w.re += __shfl_down_sync(0xffffffffu, w.re, off);
-                w.im += __shfl_down_sync(0xffffffffu, w.im, off);
-            }
-            if (lane == 0) a.part2[(int64_t)g * kPB + (cc - a.kb)] = w;
-        }
-        if (!grid_sync(a.gb)) return;
-        // phase 3: A[i, cc] -= conj(tau) v_i w_cc on own rows
-        for (int cc = c + 1 + warp; cc < cend; cc += NW) {
-            c128 w = czero<double>();
-            for (int t = lane; t < G; t += 32) w = w + a.part2[(int64_t)t * kPB + (cc - a.kb)];
-            for (int off = 16; off; off >>= 1) {
-                w.re += __shfl_down_sync(0xffffffffu, w.re, off);
-                w.im += __shfl_down_sync(0xffffffffu, w.im, off);
-            }
-            if (lane == 0) s_w[cc - a.kb] = w;
-        }
-        __syncthreads();
-        if (!ident) {
-            const c128 ct = cconj(s_tau);
-            const int nc = cend - (c + 1);
-            const int lo = max(r0, d);
-            const int nr = max(0, r1 - lo);
-            for (int idx = tid; idx < nr * nc; idx += 256) {
-                const int i = lo + idx % nr, cc = c + 1 + idx / nr;
-                const c128 v = (i == d) ? mk<double>(1.0, 0.0) : col[i];
-                cfms(a.A[i + (int64_t)cc * a.lda], ct * v, s_w[cc - a.kb]);
-            }
-        }
-        __syncthreads();
-    }
-    // compact WY factor: T upper triangular with I - V T V^H = H_0 ... H_{bw-1}
+    const int G = gridDim.x, g = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int bw = a.bw;
-    for (int e = tid; e < bw * bw; e += 256) {
-        const int p = e % bw, q = e / bw;
-        c128 s = czero<double>();
-        if (p < q) {
-            for (int i = max(r0, a.kb + q); i < r1; ++i) {
-                const c128 vp = (i == a.kb + p) ? mk<double>(1.0, 0.0) : a.A[i + (int64_t)(a.kb + p) * a.lda];
-                const c128 vq = (i == a.kb + q) ? mk<double>(1.0, 0.0) : a.A[i + (int64_t)(a.kb + q) * a.lda];
-                cfma_conj(s, vp, vq);
+    const int r0 = min(a.n, a.kb + g * a.per), r1 = min(a.n, r0 + a.per), nr = r1 - r0;
+    c128* Ag = a.A + r0 + (int64_t)a.kb * a.lda;
+    c128* P = a.resident ? reinterpret_cast<c128*>(hqr_dyn) : Ag;  // element (local row i, column c) at P[i + c ld]
+    const int64_t ld = a.resident ? a.per + 1 : a.lda;
+    if (a.resident)
+        for (int c = warp; c < bw; c += NW)
+            for (int i = lane; i < nr; i += 32) P[i + c * ld] = Ag[i + (int64_t)c * a.lda];
+    __syncthreads();
+
+    // partial x^H a_c over the own rows below the diagonal of column j, for every c; the pivot row
+    auto publish = [&](int j) {
+        const int d = a.kb + j, lo = max(0, d + 1 - r0);
+        const c128* x = P + j * ld;
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int c = warp + NW * u;
+            c128 acc = czero<double>();
+            if (c < bw)
+                for (int i = lo + lane; i < nr; i += 32) cfma_conj(acc, x[i], P[i + c * ld]);
+            v[2 * u] = acc.re;
+            v[2 * u + 1] = acc.im;
+        }
+#pragma unroll
+        for (int off = 16, m = 4; off >= 4; off >>= 1, m >>= 1)
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                if (t >= m) break;
+                const bool up = (lane & off) != 0;
+                const double send = up ? v[t] : v[t + m], keep = up ? v[t + m] : v[t];
+                v[t] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+            }
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+        const int id = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+        if ((lane & 3) == 0) a.part[((int64_t)(j & 1) * G + g) * NV + 2 * (warp + NW * (id >> 1)) + (id & 1)] = v[0];
+        if (d >= r0 && d < r1 && tid < bw) a.row[(j & 1) * kPB + tid] = P[d - r0 + tid * ld];
+    };
+
+    publish(0);
+    for (int j = 0; j < bw; ++j) {
+        const int d = a.kb + j, lo = max(0, d + 1 - r0);
+        c128* x = P + j * ld;
+        if (!grid_sync(a.gb)) return;
+        {  // the sums over all CTAs, in the same order everywhere
+            const int id = tid & (NV - 1), seg = tid / NV;
+            const double* p = a.part + (int64_t)(j & 1) * G * NV + id;
+            double s = 0.0;
+#pragma unroll 4
+            for (int t = seg; t < G; t += 4) s += __ldcg(p + (int64_t)t * NV);
+            s_red[seg][id] = s;
+            if (tid < bw) {
+                const double2 rv = __ldcg(reinterpret_cast<const double2*>(a.row + (j & 1) * kPB + tid));
+                s_row[tid] = mk<double>(rv.x, rv.y);
             }
         }
-        a.part3[(int64_t)g * kPB * kPB + e] = s;
-    }
-    if (!grid_sync(a.gb)) return;
-    if (tid == 0) {
-        for (int e = g; e < bw * bw; e += G) {
-            c128 s = czero<double>();
-            for (int t = 0; t < G; ++t) s = s + a.part3[(int64_t)t * kPB * kPB + e];
-            a.Y[e] = s;
-        }
-    }
-    if (!grid_sync(a.gb)) return;
-    if (g == 0) {
-        for (int q = 0; q < bw; ++q) {
-            const c128 tq = a.tau[a.kb + q];
-            if (tid < q) {
-                c128 s = czero<double>();
-                for (int l = tid; l < q; ++l) cfma(s, a.T[tid + l * bw], a.Y[l + q * bw]);
-                a.T[tid + q * bw] = czero<double>() - tq * s;
+        __syncthreads();
+        if (tid < NV) s_D[tid] = (s_red[0][tid] + s_red[1][tid]) + (s_red[2][tid] + s_red[3][tid]);
+        __syncthreads();
+        if (warp == 0) {
+            const c128 al = s_row[j];
+            const double xs = s_D[2 * j];
+            c128 tau = czero<double>(), scal = mk<double>(1.0, 0.0);
+            double beta = al.re;
+            const bool ident = xs == 0.0 && al.im == 0.0;
+            if (!ident) {
+                beta = -copysign(sqrt(al.re * al.re + al.im * al.im + xs), al.re);
+                const double dre = al.re - beta;
+                // 1 / beta and 1 / |alpha - beta|^2 in two lanes of one division
+                const double q = 1.0 / (lane == 0 ? beta : dre * dre + al.im * al.im);
+                const double qb = __shfl_sync(0xffffffffu, q, 0), qd = __shfl_sync(0xffffffffu, q, 1);
+                tau = mk<double>(-dre * qb, -al.im * qb);
+                scal = mk<double>(dre * qd, -al.im * qd);
             }
-            if (tid == 0) a.T[q + q * bw] = tq;
-            for (int i = q + 1 + tid; i < bw; i += 256) a.T[i + q * bw] = czero<double>();
+            if (lane < bw) {
+                const c128 D = mk<double>(s_D[2 * lane], s_D[2 * lane + 1]);
+                if (lane > j) s_g[lane] = cconj(tau) * (cconj(scal) * D + s_row[lane]);
+                if (lane < j) s_Y[j * (j - 1) / 2 + lane] = scal * cconj(D) + cconj(s_row[lane]);
+            }
+            if (lane == 0) {
+                s_scal = scal;
+                s_beta = beta;
+                s_ident = ident;
+                s_tau[j] = tau;
+                if (g == 0) a.tau[d] = tau;
+            }
+        }
+        __syncthreads();
+        if (!s_ident) {
+            const c128 sc = s_scal;
+            for (int i = lo + tid; i < nr; i += 256) x[i] = x[i] * sc;
+            if (d >= r0 && d < r1 && tid >= j && tid < bw) {
+                c128* e = P + (d - r0) + tid * ld;
+                *e = tid == j ? mk<double>(s_beta, 0.0) : *e - s_g[tid];
+            }
             __syncthreads();
+            for (int c = j + 1 + ((warp - j - 1) & (NW - 1)); c < bw; c += NW) {
+                const c128 gc = s_g[c];
+                for (int i = lo + lane; i < nr; i += 32) cfms(P[i + c * ld], x[i], gc);
+            }
         }
+        __syncthreads();
+        if (j + 1 < bw) publish(j + 1);
     }
+    for (int c = warp; c < bw; c += NW)
+        for (int i = lane; i < nr; i += 32) {
+            const c128 v = P[i + c * ld];
+            const int gi = r0 + i - a.kb;
+            if (a.resident) Ag[i + (int64_t)c * a.lda] = v;
+            a.V[gi + (int64_t)c * a.ldv] = gi == c ? mk<double>(1.0, 0.0) : gi > c ? v : czero<double>();
+        }
+    if (g != G - 1) return;
+    // compact WY factor, I - V T V^H = H_0 ... H_{bw-1}: merged from blocks of one column by
+    // T = [T1, -T1 Y12 T2; 0, T2] with Y = V^H V
+    c128(*s_T)[kPB + 1] = reinterpret_cast<c128(*)[kPB + 1]>(hqr_dyn);  // [column][row], over the panel
+    __syncthreads();
+    for (int e = tid; e < kPB * kPB; e += 256) {
+        const int r = e % kPB, c = e / kPB;
+        s_T[c][r] = (r == c && c < bw) ? s_tau[c] : czero<double>();
+    }
+    __syncthreads();
+    for (int w = 1; w < kPB; w *= 2) {  // 16 w entries of the off-diagonal blocks, at most one a thread
+        const int b0 = 2 * w * (tid / (w * w)), r = b0 + tid % w, c = b0 + w + (tid % (w * w)) / w;
+        const bool on = tid < 16 * w && c < bw;
+        c128* y = s_Y + c * (c - 1) / 2;
+        c128 s = czero<double>();
+        if (on)
+            for (int l = r; l < b0 + w; ++l) cfma(s, s_T[l][r], y[l]);  // Y12 <- T1 Y12
+        __syncthreads();
+        if (on) y[r] = s;
+        __syncthreads();
+        s = czero<double>();
+        if (on)
+            for (int l = b0 + w; l <= c; ++l) cfms(s, s_Y[l * (l - 1) / 2 + r], s_T[c][l]);  // T12 = -Y12 T2
+        __syncthreads();
+        if (on) s_T[c][r] = s;
+        __syncthreads();
+    }
+    for (int e = tid; e < bw * bw; e += 256) a.T[e] = s_T[e / bw][e % bw];
 }
 
 // explicit V block: rows kb..n-1 of the panel, unit diagonal, zeros above
@@ -244,32 +285,30 @@ std::vector<int> bit_reversed_order(int N) {
 // stops after the first panel whose remaining trailing block has squared Frobenius norm
 // <= stop2.  Returns the number of rows of R produced in *kk and panels in *npan.
 struct HqrWork {
-    c128 *V = nullptr, *W = nullptr, *W2 = nullptr, *tau = nullptr, *Tall = nullptr, *alpha = nullptr,
-         *part2 = nullptr, *part3 = nullptr, *Yb = nullptr;
+    c128 *V = nullptr, *W = nullptr, *W2 = nullptr, *tau = nullptr, *Tall = nullptr, *row = nullptr;
     double *part = nullptr, *dnorm = nullptr;
     c128 *px = nullptr, *py = nullptr;
     unsigned* bar = nullptr;
-    int G = 0;
+    int nsm = 0, smem_max = 0;
     cudaStream_t st = nullptr;
     int alloc(int64_t rows, int cols, int kmax, cudaStream_t s) {
         st = s;
-        int dev = 0, nsm = 0, occ = 0;
+        int dev = 0;
         RSRR_CUDA(cudaGetDevice(&dev));
         RSRR_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-        RSRR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, hqr_panel_kernel, 256, 0));
-        if (occ < 1) return set_error(RSRR_ECUDA, "panel kernel cannot be resident");
-        G = nsm;
+        cudaFuncAttributes fa;
+        RSRR_CUDA(cudaFuncGetAttributes(&fa, hqr_panel_kernel));
+        RSRR_CUDA(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+        smem_max -= (int)fa.sharedSizeBytes;
+        RSRR_CUDA(cudaFuncSetAttribute(hqr_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
         const int np = (int)ceil_div(kmax, kPB);
         RSRR_TRY(dalloc_n(&V, (size_t)rows * kPB, s));
         RSRR_TRY(dalloc_n(&W, (size_t)kPB * cols, s));
         RSRR_TRY(dalloc_n(&W2, (size_t)kPB * cols, s));
         RSRR_TRY(dalloc_n(&tau, (size_t)kmax, s));
         RSRR_TRY(dalloc_n(&Tall, (size_t)np * kPB * kPB, s));
-        RSRR_TRY(dalloc_n(&alpha, 1, s));
-        RSRR_TRY(dalloc_n(&part, (size_t)G, s));
-        RSRR_TRY(dalloc_n(&part2, (size_t)G * kPB, s));
-        RSRR_TRY(dalloc_n(&part3, (size_t)G * kPB * kPB, s));
-        RSRR_TRY(dalloc_n(&Yb, (size_t)kPB * kPB, s));
+        RSRR_TRY(dalloc_n(&row, (size_t)2 * kPB, s));
+        RSRR_TRY(dalloc_n(&part, (size_t)4 * kPB * nsm, s));
         RSRR_TRY(dalloc_n(&bar, kGridBarWords, s));
         RSRR_TRY(dalloc_n(&dnorm, 1, s));
         RSRR_TRY(dalloc_n(&px, (size_t)cols, s));
@@ -278,8 +317,8 @@ struct HqrWork {
         return RSRR_OK;
     }
     ~HqrWork() {
-        for (void* p : {(void*)V, (void*)W, (void*)W2, (void*)tau, (void*)Tall, (void*)alpha, (void*)part2,
-                        (void*)part3, (void*)Yb, (void*)part, (void*)dnorm, (void*)bar, (void*)px, (void*)py})
+        for (void* p : {(void*)V, (void*)W, (void*)W2, (void*)tau, (void*)Tall, (void*)row, (void*)part, (void*)dnorm,
+                        (void*)bar, (void*)px, (void*)py})
             dfree(p, st);
     }
 };
@@ -297,16 +336,22 @@ int householder_qr(c128* A, int64_t rows, int cols, int64_t lda, HqrWork& w, dou
     int kk = 0, npan = 0;
     for (int kb = 0; kb < kmax; kb += kPB) {
         const int bw = std::min(kPB, kmax - kb);
-        PanelArgs pa{A, lda, (int)rows, kb, bw, w.tau, w.Tall + (int64_t)npan * kPB * kPB, w.part, w.alpha,
-                     w.part2, w.part3, w.Yb, grid_bar_at(w.bar)};
+        // rows per CTA: a multiple of 32 (lane = row), the fewest that use every SM.  Fewer than 32
+        // rows cost as much as 32, and every further CTA adds its share to each column's sums.
+        const int per = (int)ceil_div(ceil_div(rows - kb, w.nsm), 32) * 32;
+        const size_t sm = (size_t)(per + 1) * bw * sizeof(c128);
+        const int resident = sm <= (size_t)w.smem_max;
+        const size_t smt = (size_t)kPB * (kPB + 1) * sizeof(c128);  // T is formed over the panel's rows
+        PanelArgs pa{A, lda, (int)rows, kb, bw, per, w.tau, w.Tall + (int64_t)npan * kPB * kPB, w.V, rows,
+                     w.part, w.row, resident, grid_bar_at(w.bar)};
         void* args[] = {&pa};
-        RSRR_CUDA(cudaLaunchCooperativeKernel((void*)hqr_panel_kernel, w.G, 256, args, 0, st));
+        RSRR_CUDA(cudaLaunchCooperativeKernel((void*)hqr_panel_kernel, (unsigned)ceil_div(rows - kb, per), 256, args,
+                                              resident ? std::max(sm, smt) : smt, st));
         note_launch();
         ++npan;
         kk = kb + bw;
         const int mt = cols - kk;
         if (mt > 0) {
-            { extract_v_kernel<<<(unsigned)ceil_div((rows - kb) * bw, 256), 256, 0, st>>>(A, lda, (int)rows, kb, bw, w.V, rows); note_launch(); }
             Zgemm g1;
             g1.opA = OP_C; g1.opB = OP_N; g1.M = bw; g1.N = mt; g1.K = (int)(rows - kb);
             g1.A = w.V; g1.lda = rows; g1.B = A + kb + (int64_t)kk * lda; g1.ldb = lda; g1.C = w.W; g1.ldc = kPB;
@@ -487,31 +532,21 @@ int project_run(rsrr_nep h, double delta) {
     h->red_fns = h->fns;  // the reduced NEP keeps T's own functions: P_i = S^H A_i S
     h->red_J = h->tz ? 0 : J;  // a tz handle has no A_i: its reduced NEP comes from chebyshev_reduce
 
-    c128 *A = nullptr, *V = nullptr, *W = nullptr, *W2 = nullptr, *tau = nullptr, *Tall = nullptr,
-         *alpha = nullptr, *part2 = nullptr, *part3 = nullptr, *Yb = nullptr, *B = nullptr, *Jm = nullptr,
-         *Ybuf = nullptr, *Z = nullptr, *Z2 = nullptr, *AY = nullptr, *Eg = nullptr, *Jn = nullptr;
-    double *part = nullptr, *dnorm = nullptr, *colnrm = nullptr;
-    unsigned* bar = nullptr;
+    c128 *A = nullptr, *B = nullptr, *Jm = nullptr, *Ybuf = nullptr, *Z = nullptr, *Z2 = nullptr, *AY = nullptr,
+         *Eg = nullptr, *Jn = nullptr;
+    double* colnrm = nullptr;
     int *order_d = nullptr, *cols_d = nullptr;
     int rc = RSRR_OK;
     auto cleanup = [&]() {
         double zm, zf;
         zgemm_profile_end(&zm, &zf);
         jacobi_profile_end(&zm, &zf);
-        for (void* p : {(void*)A, (void*)V, (void*)W, (void*)W2, (void*)tau, (void*)Tall, (void*)alpha,
-                        (void*)part2, (void*)part3, (void*)Yb, (void*)B, (void*)Jm, (void*)Ybuf, (void*)Z,
-                        (void*)Z2, (void*)AY, (void*)Eg, (void*)Jn, (void*)part, (void*)dnorm, (void*)colnrm, (void*)bar,
-                        (void*)order_d, (void*)cols_d})
+        for (void* p : {(void*)A, (void*)B, (void*)Jm, (void*)Ybuf, (void*)Z, (void*)Z2, (void*)AY, (void*)Eg, (void*)Jn,
+                        (void*)colnrm, (void*)order_d, (void*)cols_d})
             dfree(p, st);
     };
 #define TRYC(expr) do { rc = (expr); if (rc != RSRR_OK) { cleanup(); return rc; } } while (0)
 #define CUDAC(call) do { cudaError_t e_ = (call); if (e_ != cudaSuccess) { cleanup(); return set_error(RSRR_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); } } while (0)
-
-    int dev = 0, nsm = 0, occ = 0;
-    CUDAC(cudaGetDevice(&dev));
-    CUDAC(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    CUDAC(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, hqr_panel_kernel, 256, 0));
-    if (occ < 1) { cleanup(); return set_error(RSRR_ECUDA, "panel kernel cannot be resident"); }
 
     TRYC(dalloc_n(&A, (size_t)n * m, st));
     if (Kp > 0) {
