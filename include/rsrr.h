@@ -415,10 +415,10 @@ int rsrr_band_solve_noalloc(int64_t n, int32_t kl, int32_t ku, double* ab_reim, 
  * reports RSRR_ETIMEOUT.  This call runs one such wait with a short poll limit (well under a
  * second) on a condition the host arranged, so that a test can check that chain without faulting
  * or hanging the device:
- *   kind 0  a grid barrier (2 CTAs, cooperative launch) whose arrival count starts where no CTA
- *           can complete it: returns RSRR_ETIMEOUT
+ *   kind 0  a grid barrier (2 CTAs, cooperative launch) that waits for one CTA more than there
+ *           are: returns RSRR_ETIMEOUT
  *   kind 1  an mbarrier wait on a phase that nothing arrives at: returns RSRR_ETIMEOUT
- *   kind 2  the same grid barrier from a zero count: returns RSRR_OK
+ *   kind 2  the same grid barrier over the CTAs there are: returns RSRR_OK
  *   kind 3  the same mbarrier wait after its one expected arrival: returns RSRR_OK
  *   stream  cudaStream_t for the work (NULL = default); returns after it completes.
  * The device context stays usable after every kind.  Errors: EINVAL (kind), ENOMEM, ECUDA. */

@@ -353,260 +353,242 @@ void block_norm2(const c128* A, int64_t lda, int r0, int r1, int c0, int c1, dou
 // columns are above an absolute floor: columns below the floor are rounding noise, and rotating
 // them against anything changes no column above the floor by more than the floor itself.
 //
-// The squared column norms live in a small array: computed once at the start of the sweep and
-// recomputed from the rotated entries by the CTA that rotates a pair, so they are always the sums
-// a fresh pass over the stored columns would give.  A pair then costs one complex inner product
-// (4 FP64 fused multiply-adds a row) when it is not rotated, nothing when a column is below the
-// floor, and the columns it rotates are held in registers between the two passes.
+// The rounds of a sweep are a chain, so a pair's latency is what counts, and on this part a
+// dependent FP64 operation takes 70-85 ns, a division 260 ns, a square root 350 ns.  A pair is
+// therefore one pass: both columns are loaded into registers with the first reads, one reduction
+// gives the inner product and both norms, the tangent T = t e^{i phi} of the rotation is formed in
+// FP32, and only what unitarity needs is FP64: c = (1 + |T|^2)^(-1/2), s e^{i phi} = c T.  The
+// rotation is unitary to FP64 for any T; an angle off by 2^-23 leaves that share of the pair's
+// inner product, which the next sweep sees (sweeps already converge quadratically to 1e-10).
+// One round then takes 3.0 us at 212 columns, from 6.1 us; a whole pass's sweeps: n = 900, k_S = 233:
+// 50.7 -> 23 ms, n = 40000: 88.9 -> 43.5 ms (there also without J in the projection, see project.cu).
+// The norms that decide about the floor are al - Re(conj(T) g) and be + Re(conj(T) g), exact to
+// rounding in the smaller one; every pair forms its own from the columns.
 // ---------------------------------------------------------------------------------------------
 namespace {
 __device__ __forceinline__ int rr_pos(int k, int r, int n) {  // player at seat k in round r
     return k == 0 ? 0 : ((k - 1 + r) % (n - 1)) + 1;
 }
 
+struct JacobiCtl {  // cleared before each sweep
+    unsigned long long max_off;
+    int rotations, formed;  // pairs rotated, pairs whose inner product was formed
+    int err, pad[3];
+};
 struct JacobiArgs {
     c128* B;
     int mb, kk, npad;
     c128* J;
-    double tol, floor2, abs_g;
-    double* nrm2;  // squared column norms of B (kk entries)
-    int* ver;      // rounds each column has finished in this sweep (kk entries, zero at launch)
-    int* jver;     // rounds whose rotation of J's column is done (kk entries, zero at launch)
-    unsigned long long* max_off;
-    int* rotations;  // [0] pairs rotated, [1] pairs whose inner product was formed
-    GridBar gb;      // the barrier after the norms; its error word also records a wait that gave up
+    double tol2, floor2;
+    double* nrm2;    // squared column norms of B (kk entries)
+    // rounds each column has finished in this sweep, rounds whose rotation of J's column is done (zero
+    // at launch); one entry every kJacVer words, so that the polls of a round spread over L2
+    unsigned *ver, *jver;
+    JacobiCtl* ctl;
 };
 
-// Two block-wide sums; every thread gets both, summed in the same order (two CTA barriers).  The
-// per-warp partials are combined by a shuffle tree in every warp (log2 of the warp count FP64
-// additions a thread), not by a loop over them: FP64 issue slots are the scarce resource here.
-__device__ __forceinline__ void block_sum2(double& a, double& b) {
-    __shared__ double red2_[2][32];
-    for (int off = 16; off; off >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, off);
-        b += __shfl_down_sync(0xffffffffu, b, off);
-    }
-    __syncthreads();
-    const int w = threadIdx.x >> 5, nw = blockDim.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) { red2_[0][w] = a; red2_[1][w] = b; }
-    __syncthreads();
-    double s0 = lane < nw ? red2_[0][lane] : 0.0, s1 = lane < nw ? red2_[1][lane] : 0.0;
-    for (int off = nw >> 1; off; off >>= 1) {  // nw is a power of two
-        s0 += __shfl_xor_sync(0xffffffffu, s0, off);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, off);
-    }
-    a = __shfl_sync(0xffffffffu, s0, 0);
-    b = __shfl_sync(0xffffffffu, s1, 0);
-}
-
-constexpr int kJacThreads = 256;
 // Columns are read past L1: between rounds they are rewritten by CTAs on other SMs.
 __device__ __forceinline__ c128 ldcg_c(const c128* p) {
     const double2 v = __ldcg(reinterpret_cast<const double2*>(p));
     return mk<double>(v.x, v.y);
 }
-constexpr int kJacCache = 3;  // rows per thread kept in registers (columns up to 768 rows)
+constexpr int kJacCache = 3;  // rows per thread kept in registers
+constexpr int kJacVer = 8;
 
-__device__ __forceinline__ void jac_norm_acc(double& acc, c128 x) { acc = fma(x.re, x.re, fma(x.im, x.im, acc)); }
-// conj(x) y accumulated into (gr, gi)
-__device__ __forceinline__ void jac_dot_acc(double& gr, double& gi, c128 x, c128 y) {
-    gr = fma(x.re, y.re, fma(x.im, y.im, gr));
-    gi = fma(x.re, y.im, fma(-x.im, y.re, gi));
+struct JacSums { double gr, gi, al, be; };
+__device__ __forceinline__ void jac_acc(JacSums& t, c128 x, c128 y) {
+    t.gr = fma(x.re, y.re, fma(x.im, y.im, t.gr));  // conj(x) y
+    t.gi = fma(x.re, y.im, fma(-x.im, y.re, t.gi));
+    t.al = fma(x.re, x.re, fma(x.im, x.im, t.al));
+    t.be = fma(y.re, y.re, fma(y.im, y.im, t.be));
 }
-// (x, y) <- (c x - sp y, s x + cp y): the rotation with the phase folded into the two complex
-// coefficients (12 FP64 operations a row)
-__device__ __forceinline__ void jac_rotate(c128& x, c128& y, double c, double s, c128 sp, c128 cp) {
-    const c128 nx = mk<double>(fma(-sp.re, y.re, fma(sp.im, y.im, c * x.re)),
-                               fma(-sp.re, y.im, fma(-sp.im, y.re, c * x.im)));
-    const c128 ny = mk<double>(fma(cp.re, y.re, fma(-cp.im, y.im, s * x.re)),
-                               fma(cp.re, y.im, fma(cp.im, y.re, s * x.im)));
+// (x, y) <- (c x - conj(S) y, S x + c y): 12 FP64 operations a row
+__device__ __forceinline__ void jac_rotate(c128& x, c128& y, double c, c128 S) {
+    const c128 nx = mk<double>(fma(-S.re, y.re, fma(-S.im, y.im, c * x.re)),
+                               fma(-S.re, y.im, fma(S.im, y.re, c * x.im)));
+    const c128 ny = mk<double>(fma(S.re, x.re, fma(-S.im, x.im, c * y.re)),
+                               fma(S.re, x.im, fma(S.im, x.re, c * y.im)));
     x = nx;
     y = ny;
 }
 
-// One column pair (p, q) of a round, p < q < kk; every thread of the CTA takes the same branches.
-// Rotates the pair's columns of B and stores their norms; returns whether it rotated, with the
-// rotation in (c, s, sp, cp) for J's columns, which the caller rotates after releasing B's.
-// The rotation of the CTA's current pair (c, s, s e^{-i phi}, c e^{-i phi}): written by thread 0,
-// read by every thread for B's columns and, after B's release, for J's.
-__shared__ double jac_spar[6];
-
-__device__ __forceinline__ bool jac_pair(const JacobiArgs& a, int p, int q) {
-    const int tid = threadIdx.x;
-    const double al = __ldcg(a.nrm2 + p), be = __ldcg(a.nrm2 + q);
-    if (fmin(al, be) <= a.floor2) return false;
-    c128* bp = a.B + (int64_t)p * a.mb;
-    c128* bq = a.B + (int64_t)q * a.mb;
-    c128 xc[kJacCache], yc[kJacCache];
-    double gr = 0.0, gi = 0.0;
-#pragma unroll
-    for (int u = 0; u < kJacCache; ++u) {
-        const int r = tid + kJacThreads * u;
-        xc[u] = yc[u] = czero<double>();
-        if (r < a.mb) {
-            xc[u] = ldcg_c(bp + r);
-            yc[u] = ldcg_c(bq + r);
-            jac_dot_acc(gr, gi, xc[u], yc[u]);
-        }
-    }
-    for (int r = tid + kJacThreads * kJacCache; r < a.mb; r += kJacThreads)
-        jac_dot_acc(gr, gi, ldcg_c(bp + r), ldcg_c(bq + r));
-    block_sum2(gr, gi);
-    // the decision and the rotation are computed once, by thread 0, and shared
-    __shared__ int s_act;
-    if (tid == 0) {
-        atomicAdd(a.rotations + 1, 1);
-        int act = 0;
-        const double g = sqrt(gr * gr + gi * gi);
-        if (g > a.abs_g) {
-            const double off = g / sqrt(al * be);
-            atomicMax(a.max_off, (unsigned long long)__double_as_longlong(off));
-            if (off > a.tol) {
-                const double ig = 1.0 / g;
-                const c128 ph = mk<double>(gr * ig, -gi * ig);  // e^{-i phi}, phi = arg(conj(b_p) b_q)
-                const double zeta = (be - al) * (0.5 * ig);
-                const double t = (zeta >= 0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-                const double c = 1.0 / sqrt(1.0 + t * t), sn = c * t;
-                jac_spar[0] = c;
-                jac_spar[1] = sn;
-                jac_spar[2] = ph.re * sn;
-                jac_spar[3] = ph.im * sn;
-                jac_spar[4] = ph.re * c;
-                jac_spar[5] = ph.im * c;
-                act = 1;
-            }
-        }
-        s_act = act;
-    }
+// The sums of the four values over the CTA, in every lane of warp 0 (lane l holds value l & 3).  A
+// full-warp FP64 addition takes 64 clocks of its sub-partition, so the values are reduce-scattered.
+template <int NT>
+__device__ __forceinline__ double jac_reduce(JacSums t) {
+    constexpr int NW = NT / 32;
+    __shared__ double red[NW * 4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool h1 = lane & 1, h2 = lane & 2;
+    double a = (h1 ? t.gi : t.gr) + __shfl_xor_sync(0xffffffffu, h1 ? t.gr : t.gi, 1);
+    double b = (h1 ? t.be : t.al) + __shfl_xor_sync(0xffffffffu, h1 ? t.al : t.be, 1);
+    double v = (h2 ? b : a) + __shfl_xor_sync(0xffffffffu, h2 ? a : b, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 4);
+    v += __shfl_xor_sync(0xffffffffu, v, 8);
+    v += __shfl_xor_sync(0xffffffffu, v, 16);
+    if (lane < 4) red[warp * 4 + lane] = v;
     __syncthreads();
-    if (!s_act) return false;
-    // (b_p, b_q) <- (c b_p - s e^{-i phi} b_q, s b_p + c e^{-i phi} b_q)
-    const double c = jac_spar[0], s = jac_spar[1];
-    const c128 sp = mk<double>(jac_spar[2], jac_spar[3]), cp = mk<double>(jac_spar[4], jac_spar[5]);
-    double an = 0.0, bn = 0.0;
-#pragma unroll
-    for (int u = 0; u < kJacCache; ++u) {
-        const int r = tid + kJacThreads * u;
-        if (r < a.mb) {
-            jac_rotate(xc[u], yc[u], c, s, sp, cp);
-            bp[r] = xc[u];
-            bq[r] = yc[u];
-            jac_norm_acc(an, xc[u]);
-            jac_norm_acc(bn, yc[u]);
-        }
+    if (warp == 0) {
+        v = red[lane % (NW * 4)];
+        for (int off = 4; off < 4 * NW; off <<= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
     }
-    for (int r = tid + kJacThreads * kJacCache; r < a.mb; r += kJacThreads) {
-        c128 x = ldcg_c(bp + r), y = ldcg_c(bq + r);
-        jac_rotate(x, y, c, s, sp, cp);
-        bp[r] = x;
-        bq[r] = y;
-        jac_norm_acc(an, x);
-        jac_norm_acc(bn, y);
-    }
-    block_sum2(an, bn);
-    if (tid == 0) {
-        a.nrm2[p] = an;
-        a.nrm2[q] = bn;
-        atomicAdd(a.rotations, 1);
-    }
-    return true;
+    return v;
 }
 
-// Thread 0 waits until column c has finished `target` rounds.  Bounded: after the spin limit, or
-// once another CTA has reported a timeout, it records the failure and returns false.
-__device__ __forceinline__ bool jac_wait(const int* ver, int c, int target, int* err) {
-    const volatile int* v = ver + c;
+// Waits until column c has finished `target` rounds.  Bounded: after the spin limit, or once
+// another CTA has reported a timeout, it records the failure and returns false.
+__device__ __forceinline__ bool jac_wait(const unsigned* ver, int c, unsigned target, int* err) {
     long long spins = 0;
-    unsigned backoff = 16;
-    while (*v < target) {
-        if (++spins > (1LL << 24) || *(volatile int*)err != 0) {
+    while (ld_acquire_gpu(ver + (int64_t)c * kJacVer) < target) {
+        if (++spins > (1LL << 22) || ((spins & 255) == 0 && *(volatile int*)err != 0)) {
             atomicExch(err, 1);
             return false;
         }
-        __nanosleep(backoff);
-        if (backoff < 256) backoff <<= 1;
     }
     return true;
 }
 
-__global__ void __launch_bounds__(kJacThreads, 3) jacobi_sweep_kernel(JacobiArgs a) {
-    // One CTA per column pair (CTAs take the pairs in order, see below), so every round spreads its
-    // FP64 work over all SMs.  The rounds are not separated by grid barriers: a pair of round r
-    // starts as soon as both of its columns have come out of round r - 1 (a per-column count of
-    // finished rounds), so a slow pair holds up only the pairs that need its columns.  The pairs,
-    // their order and every value are those of the barrier-separated sweep.
-    const int tid = threadIdx.x;
-    __shared__ int s_ok;
-    for (int c = blockIdx.x; c < a.kk; c += gridDim.x) {
-        const c128* bc = a.B + (int64_t)c * a.mb;
-        double s = 0.0, unused = 0.0;
-        for (int r = tid; r < a.mb; r += kJacThreads) jac_norm_acc(s, ldcg_c(bc + r));
-        block_sum2(s, unused);
-        if (tid == 0) a.nrm2[c] = s;
-    }
-    if (!grid_sync(a.gb)) return;
-    // The pairs of all rounds are numbered g = round * (npad / 2) + i and dealt out in that order.
-    // A pair releases its columns of B (and their norms) to the next round as soon as they are
+template <int NT>
+__global__ void __launch_bounds__(NT, 768 / NT) jacobi_sweep_kernel(JacobiArgs a) {
+    // One CTA per column pair, so every round spreads its FP64 work over all SMs.  The rounds are not
+    // separated by grid barriers: a pair of round r starts as soon as both of its columns have come out
+    // of round r - 1 (a per-column count of finished rounds), so a slow pair holds up only the pairs
+    // that need its columns.  The pairs of all rounds are numbered g = round * (npad / 2) + i and
+    // dealt out in that order.  A pair releases its columns of B to the next round as soon as they are
     // rotated; it then rotates its columns of J, once the previous round's rotation of them is done
     // (jver), and releases those.  With more CTAs than pairs in a round, CTAs start pairs of the next
-    // round while J's rotations of this one run.  Every wait is on a smaller g (or the same g's B
-    // part), every CTA takes its pairs in increasing g and all are resident (cooperative launch), so
-    // the smallest unfinished step can always proceed.  The arithmetic is that of the sweep with a
-    // grid barrier between rounds.
+    // round meanwhile.  Every wait is on a smaller g (or the same g's B part), every CTA takes its pairs
+    // in increasing g and all are resident (cooperative launch), so the smallest unfinished step can
+    // always proceed.
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ int s_ok, s_act;
+    __shared__ double s_c;
+    __shared__ c128 s_S;
     const int ppr = a.npad / 2;
     const int64_t npairs = (int64_t)(a.npad - 1) * ppr;
-    for (int64_t gi = blockIdx.x; gi < npairs; gi += gridDim.x) {
-        const int round = (int)(gi / ppr), i = (int)(gi % ppr);
-        int p = rr_pos(i, round, a.npad), q = rr_pos(a.npad - 1 - i, round, a.npad);
+    for (int64_t g = blockIdx.x; g < npairs; g += gridDim.x) {
+        const unsigned round = (unsigned)(g / ppr);
+        const int i = (int)(g % ppr);
+        int p = rr_pos(i, (int)round, a.npad), q = rr_pos(a.npad - 1 - i, (int)round, a.npad);
         if (p > q) { const int t = p; p = q; q = t; }
         const bool real_pair = q < a.kk;  // q == kk is the padding column of an odd count
-        if (tid == 0) {
-            const bool ok = jac_wait(a.ver, p, round, a.gb.err) && (!real_pair || jac_wait(a.ver, q, round, a.gb.err));
-            __threadfence();
-            s_ok = ok;
-        }
-        __syncthreads();
-        if (!s_ok) return;
-        const bool rot = real_pair && jac_pair(a, p, q);
-        __syncthreads();  // every store of B and of the norms issued
-        if (tid == 0) {
-            __threadfence();
-            atomicExch(a.ver + p, round + 1);
-            if (real_pair) atomicExch(a.ver + q, round + 1);
-        }
-        if (a.J) {
-            if (tid == 0) {
-                const bool ok = jac_wait(a.jver, p, round, a.gb.err) &&
-                                (!real_pair || jac_wait(a.jver, q, round, a.gb.err));
-                __threadfence();
-                s_ok = ok;
+        auto wait_both = [&](const unsigned* ver) {  // lanes 0 and 1 of warp 0 poll one column each
+            if (warp == 0) {
+                bool ok = true;
+                if (lane < (real_pair ? 2 : 1)) ok = jac_wait(ver, lane ? q : p, round, &a.ctl->err);
+                ok = __all_sync(0xffffffffu, ok);
+                if (lane == 0) s_ok = ok;
             }
             __syncthreads();
-            if (!s_ok) return;
+            return s_ok != 0;
+        };
+        auto release_both = [&](unsigned* ver) {  // after a barrier: every store of the columns is issued
+            if (tid < (real_pair ? 2 : 1)) st_release_gpu(ver + (int64_t)(tid ? q : p) * kJacVer, round + 1);
+        };
+        if (!wait_both(a.ver)) return;
+        bool rot = false;
+        if (real_pair) {
+            c128* bp = a.B + (int64_t)p * a.mb;
+            c128* bq = a.B + (int64_t)q * a.mb;
+            const double np = __ldcg(a.nrm2 + p), nq = __ldcg(a.nrm2 + q);
+            c128 xc[kJacCache], yc[kJacCache];
+#pragma unroll
+            for (int u = 0; u < kJacCache; ++u) {
+                const int r = tid + NT * u;
+                xc[u] = yc[u] = czero<double>();
+                if (r < a.mb) {
+                    xc[u] = ldcg_c(bp + r);
+                    yc[u] = ldcg_c(bq + r);
+                }
+            }
+            if (fmin(np, nq) > a.floor2) {  // the same for the whole CTA
+                JacSums t{0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+                for (int u = 0; u < kJacCache; ++u)
+                    if (tid + NT * u < a.mb) jac_acc(t, xc[u], yc[u]);
+                for (int r = tid + NT * kJacCache; r < a.mb; r += NT) jac_acc(t, ldcg_c(bp + r), ldcg_c(bq + r));
+                const double v = jac_reduce<NT>(t);
+                if (warp == 0) {
+                    const double gr = __shfl_sync(0xffffffffu, v, 0), gi = __shfl_sync(0xffffffffu, v, 1);
+                    const double al = __shfl_sync(0xffffffffu, v, 2), be = __shfl_sync(0xffffffffu, v, 3);
+                    const double g2 = fma(gr, gr, gi * gi), ab = al * be;
+                    const bool act = g2 > 0.0 && g2 > a.tol2 * ab;
+                    double dn = 0.0;
+                    if (act) {
+                        // T = 2 g sign(d) / (|d| + sqrt(d^2 + 4 |g|^2)), d = be - al, scaled by a power of two
+                        const int e = min(2045, (__double2hiint(fmax(al, be)) >> 20) & 0x7ff);
+                        const double sf = __hiloint2double((2046 - e) << 20, 0);
+                        const float fr = (float)(gr * sf), fi = (float)(gi * sf), fd = (float)((be - al) * sf);
+                        const float h = sqrtf(fmaf(fd, fd, 4.f * fmaf(fr, fr, fi * fi)));
+                        const float w = copysignf(2.f / (fabsf(fd) + h), fd);
+                        const double Tr = (double)(fr * w), Ti = (double)(fi * w);
+                        // (1 + |T|^2)^(-1/2): FP32 seed, one third-order step
+                        const double x = fma(Tr, Tr, fma(Ti, Ti, 1.0)), y0 = (double)rsqrtf((float)x);
+                        const double r1 = fma(-(x * y0), y0, 1.0);
+                        const double c = fma(fma(0.375, r1, 0.5), y0 * r1, y0);
+                        dn = fma(Tr, gr, Ti * gi);
+                        if (lane == 0) {
+                            s_c = c;
+                            s_S = mk<double>(Tr * c, Ti * c);
+                        }
+                    }
+                    if (lane == 0) {
+                        s_act = act;
+                        atomicAdd(&a.ctl->formed, 1);
+                        if (act) {
+                            a.nrm2[p] = al - dn;
+                            a.nrm2[q] = be + dn;
+                            atomicAdd(&a.ctl->rotations, 1);
+                        }
+                    } else if (lane == 1 && g2 > 0.0) {
+                        atomicMax(&a.ctl->max_off, (unsigned long long)__double_as_longlong(sqrt(g2 / ab)));
+                    }
+                }
+                __syncthreads();
+                rot = s_act != 0;
+                if (rot) {
+                    const double c = s_c;
+                    const c128 S = s_S;
+#pragma unroll
+                    for (int u = 0; u < kJacCache; ++u) {
+                        const int r = tid + NT * u;
+                        if (r < a.mb) {
+                            jac_rotate(xc[u], yc[u], c, S);
+                            bp[r] = xc[u];
+                            bq[r] = yc[u];
+                        }
+                    }
+                    for (int r = tid + NT * kJacCache; r < a.mb; r += NT) {
+                        c128 x = ldcg_c(bp + r), y = ldcg_c(bq + r);
+                        jac_rotate(x, y, c, S);
+                        bp[r] = x;
+                        bq[r] = y;
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        release_both(a.ver);
+        if (a.J) {
+            if (!wait_both(a.jver)) return;
             if (rot) {
-                const double c = jac_spar[0], sn = jac_spar[1];
-                const c128 sp = mk<double>(jac_spar[2], jac_spar[3]), cp = mk<double>(jac_spar[4], jac_spar[5]);
+                const double c = s_c;
+                const c128 S = s_S;
                 c128* jp = a.J + (int64_t)p * a.kk;
                 c128* jq = a.J + (int64_t)q * a.kk;
-                for (int r = tid; r < a.kk; r += kJacThreads) {
+                for (int r = tid; r < a.kk; r += NT) {
                     c128 x = ldcg_c(jp + r), y = ldcg_c(jq + r);
-                    jac_rotate(x, y, c, sn, sp, cp);
+                    jac_rotate(x, y, c, S);
                     jp[r] = x;
                     jq[r] = y;
                 }
             }
-            __syncthreads();  // every store of J issued
-            if (tid == 0) {
-                __threadfence();
-                atomicExch(a.jver + p, round + 1);
-                if (real_pair) atomicExch(a.jver + q, round + 1);
-            }
+            __syncthreads();
+            release_both(a.jver);
         }
     }
 }
-}  // namespace
 
-namespace {
 // out[:, i] = in[:, perm[i]] for the k columns of an m-row matrix (leading dimension m).
 __global__ void gather_cols_kernel(const c128* __restrict__ in, int m, int k, const int* __restrict__ perm,
                                    c128* __restrict__ out) {
@@ -618,88 +600,86 @@ __global__ void gather_cols_kernel(const c128* __restrict__ in, int m, int k, co
 }  // namespace
 
 int jacobi_orthogonalize(c128* B, int mb, int k, c128* J, cudaStream_t s, int max_sweeps, int* sweeps_out,
-                         double abs_floor, double conv, double abs_inner) {
+                         double abs_floor, double conv) {
     if (sweeps_out) *sweeps_out = 0;
     if (k < 2) return RSRR_OK;
     const int npad = k + (k & 1);
+    // 128 threads while they hold the columns in registers: fewer warps to sum over
+    const bool small = mb <= 128 * kJacCache;
+    const void* kern = small ? (const void*)jacobi_sweep_kernel<128> : (const void*)jacobi_sweep_kernel<256>;
+    const int threads = small ? 128 : 256;
     int dev = 0, nsm = 0, occ = 0;
     RSRR_CUDA(cudaGetDevice(&dev));
     RSRR_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    RSRR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, jacobi_sweep_kernel, kJacThreads, 0));
+    RSRR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, 0));
     if (occ < 1) return set_error(RSRR_ECUDA, "jacobi kernel cannot be resident");
-    // as many CTAs as are resident (up to 4 per SM), also when that is more than a round's npad / 2
-    // pairs: the surplus starts the next round's pairs while this round's J rotations finish
-    const int G = (int)std::min<int64_t>((int64_t)nsm * std::min(occ, 4), (int64_t)(npad - 1) * (npad / 2));
-    unsigned long long* dmax = nullptr;
-    int* drot = nullptr;
-    unsigned* bar = nullptr;
-    double* dn2 = nullptr;
-    int* dver = nullptr;
-    int* djver = nullptr;
+    // One CTA a pair where all are resident.  With J, twice as many: the surplus starts the next
+    // round's pairs while this round's J rotations finish.  More would only poll: with four CTAs an
+    // SM and the counts packed in a few lines a round took 5.7 us instead of 3.0.
+    const int G = (int)std::min<int64_t>((int64_t)nsm * std::min(occ, 4), (int64_t)(J ? 2 : 1) * (npad / 2));
+    const size_t ctl_bytes = sizeof(JacobiCtl) + (size_t)2 * k * kJacVer * sizeof(unsigned);
+    const size_t ord_bytes = (size_t)k * (sizeof(double) + sizeof(int));  // squared norms, then the order
+    uint8_t *ctl = nullptr, *ord = nullptr;
     double* dnrm = nullptr;
-    int* dperm = nullptr;
     c128* tmp = nullptr;
     auto cleanup = [&]() {
-        dfree(dn2, s);
-        dfree(dver, s);
-        dfree(djver, s);
-        dfree(dmax, s);
-        dfree(drot, s);
-        dfree(bar, s);
-        dfree(dnrm, s);
-        dfree(dperm, s);
-        dfree(tmp, s);
+        for (void* p : {(void*)ctl, (void*)ord, (void*)dnrm, (void*)tmp}) dfree(p, s);
     };
     int rc = RSRR_OK;
 #define JTRY(expr) do { rc = (expr); if (rc != RSRR_OK) { cleanup(); return rc; } } while (0)
-    JTRY(dalloc_n(&dn2, (size_t)k, s));
-    JTRY(dalloc_n(&dver, (size_t)k, s));
-    JTRY(dalloc_n(&djver, (size_t)k, s));
-    JTRY(dalloc_n(&dmax, 1, s));
-    JTRY(dalloc_n(&drot, 2, s));
-    JTRY(dalloc_n(&bar, kGridBarWords, s));
+    JTRY(dalloc_n(&ctl, ctl_bytes, s));
+    JTRY(dalloc_n(&ord, ord_bytes, s));
     // Before each sweep the columns (and J's with them) are put in order of decreasing norm: the
     // round-robin pairs then meet in an order that converges in fewer sweeps, and the caller,
     // which sorts the final column norms itself, sees no difference.
     JTRY(dalloc_n(&dnrm, (size_t)k, s));
-    JTRY(dalloc_n(&dperm, (size_t)k, s));
     JTRY(dalloc_n(&tmp, (size_t)mb * k + (J ? (size_t)k * k : 0), s));
-    if (cudaMemsetAsync(bar, 0, kGridBarWords * sizeof(unsigned), s) != cudaSuccess)
-        JTRY(set_error(RSRR_ECUDA, "jacobi: clearing the grid barrier"));
 #undef JTRY
-    JacobiArgs ja{B, mb, k, npad, J, sqrt((double)mb) * 1.1102230246251565e-16, abs_floor * abs_floor, abs_inner,
-                  dn2, dver, djver, dmax, drot, grid_bar_at(bar)};
+    c128 *curB = B, *altB = tmp, *curJ = J, *altJ = J ? tmp + (size_t)mb * k : nullptr;
+    JacobiCtl* dctl = reinterpret_cast<JacobiCtl*>(ctl);
+    JacobiArgs ja{};
+    ja.mb = mb;
+    ja.kk = k;
+    ja.npad = npad;
+    ja.tol2 = (double)mb * 1.1102230246251565e-16 * 1.1102230246251565e-16;
+    ja.floor2 = abs_floor * abs_floor;
+    ja.nrm2 = reinterpret_cast<double*>(ord);
+    ja.ver = reinterpret_cast<unsigned*>(ctl + sizeof(JacobiCtl));
+    ja.jver = ja.ver + (size_t)k * kJacVer;
+    ja.ctl = dctl;
+    int* dperm = reinterpret_cast<int*>(ord + (size_t)k * sizeof(double));
     std::vector<double> hn(k);
     std::vector<int> order(k);
+    std::vector<uint8_t> hord(ord_bytes);
     int sweep = 0;
     for (; sweep < max_sweeps; ++sweep) {
-        column_norms(B, mb, k, mb, dnrm, s);
+        column_norms(curB, mb, k, mb, dnrm, s);
         if (cudaMemcpyAsync(hn.data(), dnrm, (size_t)k * 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess) { rc = set_error(RSRR_ECUDA, "jacobi norms"); break; }
         for (int i = 0; i < k; ++i) order[i] = i;
         std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return hn[a] > hn[b]; });
         bool sorted = true;
-        for (int i = 0; i < k && sorted; ++i) sorted = order[i] == i;
-        if (!sorted) {
-            if (cudaMemcpyAsync(dperm, order.data(), (size_t)k * 4, cudaMemcpyHostToDevice, s) != cudaSuccess) {
-                rc = set_error(RSRR_ECUDA, "jacobi: column order upload");
-                break;
-            }
-            { gather_cols_kernel<<<(unsigned)ceil_div((int64_t)mb * k, 256), 256, 0, s>>>(B, mb, k, dperm, tmp); note_launch(); }
-            cudaError_t ce = cudaMemcpyAsync(B, tmp, (size_t)mb * k * sizeof(c128), cudaMemcpyDeviceToDevice, s);
-            if (J && ce == cudaSuccess) {
-                c128* tj = tmp + (size_t)mb * k;
-                { gather_cols_kernel<<<(unsigned)ceil_div((int64_t)k * k, 256), 256, 0, s>>>(J, k, k, dperm, tj); note_launch(); }
-                ce = cudaMemcpyAsync(J, tj, (size_t)k * k * sizeof(c128), cudaMemcpyDeviceToDevice, s);
-            }
-            if (ce != cudaSuccess) { rc = set_error(RSRR_ECUDA, "jacobi: column reorder"); break; }
+        for (int i = 0; i < k; ++i) {
+            sorted = sorted && order[i] == i;
+            const double n2 = hn[order[i]] * hn[order[i]];
+            std::memcpy(hord.data() + (size_t)i * 8, &n2, 8);
         }
-        if (cudaMemsetAsync(dmax, 0, 8, s) != cudaSuccess || cudaMemsetAsync(drot, 0, 8, s) != cudaSuccess ||
-            cudaMemsetAsync(dver, 0, (size_t)k * sizeof(int), s) != cudaSuccess ||
-            cudaMemsetAsync(djver, 0, (size_t)k * sizeof(int), s) != cudaSuccess) {
-            rc = set_error(RSRR_ECUDA, "jacobi: clearing the sweep counters");
+        std::memcpy(hord.data() + (size_t)k * 8, order.data(), (size_t)k * 4);
+        if (cudaMemcpyAsync(ord, hord.data(), ord_bytes, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+            cudaMemsetAsync(ctl, 0, ctl_bytes, s) != cudaSuccess) {
+            rc = set_error(RSRR_ECUDA, "jacobi: column order and counters");
             break;
         }
+        if (!sorted) {
+            { gather_cols_kernel<<<(unsigned)ceil_div((int64_t)mb * k, 256), 256, 0, s>>>(curB, mb, k, dperm, altB); note_launch(); }
+            std::swap(curB, altB);
+            if (J) {
+                { gather_cols_kernel<<<(unsigned)ceil_div((int64_t)k * k, 256), 256, 0, s>>>(curJ, k, k, dperm, altJ); note_launch(); }
+                std::swap(curJ, altJ);
+            }
+        }
+        ja.B = curB;
+        ja.J = curJ;
         void* args[] = {&ja};
         cudaEvent_t ea = nullptr, eb = nullptr;
         if (g_jprof.on) {
@@ -707,31 +687,30 @@ int jacobi_orthogonalize(c128* B, int mb, int k, c128* J, cudaStream_t s, int ma
             cudaEventCreate(&eb);
             cudaEventRecord(ea, s);
         }
-        cudaError_t e = cudaLaunchCooperativeKernel((void*)jacobi_sweep_kernel, G, kJacThreads, args, 0, s);
+        cudaError_t e = cudaLaunchCooperativeKernel(kern, G, threads, args, 0, s);
         note_launch();
         if (g_jprof.on) {
             cudaEventRecord(eb, s);
             g_jprof.ev.emplace_back(ea, eb);
         }
         if (e != cudaSuccess) { rc = set_error(RSRR_ECUDA, cudaGetErrorString(e)); break; }
-        int hrot[2] = {0, 0}, herr = 0;
-        unsigned long long hmax = 0;
-        if (cudaMemcpyAsync(hrot, drot, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaMemcpyAsync(&herr, bar + kGridBarErrWord, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaMemcpyAsync(&hmax, dmax, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        JacobiCtl hc;
+        if (cudaMemcpyAsync(&hc, dctl, sizeof(hc), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess) { rc = set_error(RSRR_ECUDA, "jacobi sync"); break; }
-        if (herr) { rc = set_error(RSRR_ETIMEOUT, "a wait in the Jacobi sweep gave up"); break; }
-        // the sweep's work: the column norms (4 real flops a row), one complex inner product for
-        // every pair formed (8 a row), and for every rotated pair the rotation of both columns of
-        // B and J (24 a row each) and the two new norms (8 a row)
-        if (g_jprof.on)
-            g_jprof.flops += 4.0 * mb * k + 8.0 * mb * hrot[1] + hrot[0] * (32.0 * mb + (J ? 24.0 * k : 0.0));
+        if (hc.err) { rc = set_error(RSRR_ETIMEOUT, "a wait in the Jacobi sweep gave up"); break; }
+        // the sweep's work: one complex inner product and two norms for every pair formed (16 real
+        // flops a row), and for every rotated pair the rotation of both columns of B and J (24 a row)
+        if (g_jprof.on) g_jprof.flops += 16.0 * mb * hc.formed + hc.rotations * (24.0 * mb + (J ? 24.0 * k : 0.0));
         double off;
-        std::memcpy(&off, &hmax, 8);
+        std::memcpy(&off, &hc.max_off, 8);
         // converged: no rotation left, or every pair above the floor orthogonal to `conv` (the
         // remaining effect on the singular values is of second order in that number)
-        if (hrot[0] == 0 || off <= conv) { ++sweep; break; }
+        if (hc.rotations == 0 || off <= conv) { ++sweep; break; }
     }
+    if (rc == RSRR_OK && curB != B &&
+        (cudaMemcpyAsync(B, curB, (size_t)mb * k * sizeof(c128), cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
+         (J && cudaMemcpyAsync(J, curJ, (size_t)k * k * sizeof(c128), cudaMemcpyDeviceToDevice, s) != cudaSuccess)))
+        rc = set_error(RSRR_ECUDA, "jacobi: copy of the columns");
     cleanup();
     if (sweeps_out) *sweeps_out = sweep;
     return rc;

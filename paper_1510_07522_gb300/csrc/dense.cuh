@@ -87,49 +87,54 @@ __device__ __forceinline__ double block_sum_all(double v) {
 
 // Device-wide barrier for cooperative kernels.  Every wait is bounded: after the spin limit
 // the barrier records a timeout in *err and returns false, and the kernel returns.
+// One word: every CTA adds 1 but CTA 0, which adds 2^31 - (n - 1), so the top bit flips when all n
+// have arrived and the low bits are zero again.  A CTA reads the top bit when the kernel starts (it
+// cannot flip before that CTA's own arrival) and then polls the word it added to: one trip to L2
+// and back, 1.27 us with 152 CTAs, against 2.31 us for an arrival count whose last CTA releases
+// the others through a second word.
 struct GridBar {
     unsigned* count;
-    unsigned* gen;
     int* err;
-    long long spin_limit;  // polls before a wait gives up (2^24 with backoff: about a second)
+    long long spin_limit;  // polls of about half a microsecond before a wait gives up
+    unsigned ctas;         // 0: gridDim.x
 };
-// The three words sit on separate 128-byte lines: the arrival atomics on `count` must not
-// queue behind hundreds of CTAs polling `gen` in the same L2 line.
-constexpr int kGridBarWords = 96;  // allocation size in unsigned words
-inline GridBar grid_bar_at(unsigned* base, long long spin_limit = 1LL << 24) {
-    return GridBar{base, base + 32, reinterpret_cast<int*>(base + 64), spin_limit};
+// The two words sit on separate 128-byte lines.
+constexpr int kGridBarWords = 64;  // allocation size in unsigned words
+constexpr int kGridBarErrWord = 32;
+inline GridBar grid_bar_at(unsigned* base, long long spin_limit = 1LL << 22, unsigned ctas = 0) {
+    return GridBar{base, reinterpret_cast<int*>(base + kGridBarErrWord), spin_limit, ctas};
 }
-constexpr int kGridBarErrWord = 64;
-__device__ __forceinline__ bool grid_sync(const GridBar& gb) {
+__device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release_gpu(unsigned* p, unsigned v) {
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// The barrier's phase, read once at the start of the kernel (meaningful in thread 0).
+__device__ __forceinline__ unsigned grid_phase(const GridBar& gb) {
+    return threadIdx.x == 0 ? ld_acquire_gpu(gb.count) & 0x80000000u : 0u;
+}
+__device__ __forceinline__ bool grid_sync(const GridBar& gb, unsigned& phase) {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        volatile unsigned* vgen = gb.gen;
-        const unsigned g = *vgen;
-        __threadfence();
-        const unsigned arrived = atomicAdd(gb.count, 1u);
+        const unsigned n = gb.ctas ? gb.ctas : gridDim.x;
+        asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(gb.count),
+                     "r"(blockIdx.x == 0 ? 0x80000000u - (n - 1) : 1u) : "memory");
         int ok = 1;
-        if (arrived == gridDim.x - 1) {
-            atomicExch(gb.count, 0u);
-            __threadfence();
-            atomicAdd(gb.gen, 1u);
-        } else {
-            long long spins = 0;
-            unsigned backoff = 8;
-            while (*vgen == g) {
-                if (++spins > gb.spin_limit) {  // bounded: give up, report, return
-                    atomicExch(gb.err, 1);
-                    ok = 0;
-                    break;
-                }
-                // short backoff from the first miss, so that a few hundred pollers do not
-                // saturate the line the releasing CTA has to write
-                __nanosleep(backoff);
-                if (backoff < 128) backoff <<= 1;
+        long long spins = 0;
+        while (((ld_acquire_gpu(gb.count) ^ phase) & 0x80000000u) == 0) {
+            // bounded: give up, report, return; also when another CTA has
+            if (++spins > gb.spin_limit || ((spins & 255) == 0 && *(volatile int*)gb.err != 0)) {
+                atomicExch(gb.err, 1);
+                ok = 0;
+                break;
             }
         }
-        __threadfence();
-        s_ok = ok && (*(volatile int*)gb.err == 0);
+        phase ^= 0x80000000u;
+        s_ok = ok;
     }
     __syncthreads();
     return s_ok != 0;
@@ -140,9 +145,9 @@ __device__ __forceinline__ bool grid_sync(const GridBar& gb) {
 // rotations into J (k x k, ld k, initialised to I by the caller when wanted; may be null).
 // Sweeps stop once every pair of columns above abs_floor has |<b_p, b_q>| / (|b_p| |b_q|) <=
 // conv (singular values are then exact to second order in conv); columns below abs_floor are
-// not rotated, nor are pairs with |<b_p, b_q>| <= abs_inner (absolute).
+// not rotated.
 int jacobi_orthogonalize(c128* B, int mb, int k, c128* J, cudaStream_t s, int max_sweeps, int* sweeps_out,
-                         double abs_floor, double conv, double abs_inner);
+                         double abs_floor, double conv);
 
 // Column 2-norms of B (mb x k) into out[k] (device).
 void column_norms(const c128* B, int mb, int k, int64_t ld, double* out, cudaStream_t s);

@@ -15,7 +15,8 @@ namespace {
 
 // Every CTA enters the grid barrier once; `result` counts the CTAs that saw it complete.
 __global__ void selftest_grid_kernel(GridBar gb, int* result) {
-    const bool ok = grid_sync(gb);
+    unsigned phase = grid_phase(gb);
+    const bool ok = grid_sync(gb, phase);
     if (threadIdx.x == 0 && ok) atomicAdd(result, 1);
 }
 
@@ -59,14 +60,8 @@ extern "C" int rsrr_selftest_bounded_wait(int32_t kind, void* stream) {
         return done(set_error(RSRR_ECUDA, "rsrr_selftest_bounded_wait: memset"));
     int herr = 0, hres = 0;
     if (kind == 0 || kind == 2) {
-        if (kind == 0) {
-            // an arrival count no CTA can complete: the releasing CTA is the one that finds
-            // gridDim.x - 1 arrivals before its own, which never happens from this start
-            const unsigned far = 0x40000000u;
-            if (cudaMemcpyAsync(bar, &far, sizeof(unsigned), cudaMemcpyHostToDevice, st) != cudaSuccess)
-                return done(set_error(RSRR_ECUDA, "rsrr_selftest_bounded_wait: copy"));
-        }
-        GridBar gb = grid_bar_at(bar, 4096);  // ~0.5 ms of polling with backoff
+        // kind 0: a barrier over one CTA more than are launched, which nothing can complete
+        GridBar gb = grid_bar_at(bar, 4096, kind == 0 ? kCtas + 1 : kCtas);  // about 2 ms of polling
         void* args[] = {&gb, &result};
         const cudaError_t e = cudaLaunchCooperativeKernel((const void*)selftest_grid_kernel, dim3(kCtas), dim3(64),
                                                           args, 0, st);
