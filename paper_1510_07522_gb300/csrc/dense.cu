@@ -274,7 +274,7 @@ int zgemm(const Zgemm& g0, cudaStream_t s) {
     cudaEventRecord(a, s);
     const int rc = zgemm_dispatch(g0, s);
     cudaEventRecord(b, s);
-    const bool tc = g_zpath == 2 || (g_zpath == 0 && !g0.fp64 && zgemm_tc_fits(g0));
+    const bool tc = !g0.fp64 && (g_zpath == 2 || (g_zpath == 0 && zgemm_tc_fits(g0)));
     g_zprof.ev.push_back({a, b, tc});
     const double f = 8.0 * g0.M * (double)g0.N * g0.K * g0.batch;
     g_zprof.flops += f;
@@ -291,7 +291,7 @@ static int zgemm_dispatch(const Zgemm& g0, cudaStream_t s) {
         RSRR_CUDA(cudaGetLastError());
         return RSRR_OK;
     }
-    if (g_zpath == 2 || (g_zpath == 0 && !g.fp64 && zgemm_tc_fits(g))) return zgemm_tc(g, s);
+    if (!g.fp64 && (g_zpath == 2 || (g_zpath == 0 && zgemm_tc_fits(g)))) return zgemm_tc(g, s);
     return g.N <= 8 ? zgemm_fp64<64, 4>(g, s) : zgemm_fp64<16, 16>(g, s);
 }
 
@@ -361,7 +361,7 @@ void block_norm2(const c128* A, int64_t lda, int r0, int r1, int c0, int c1, dou
 // rotation is unitary to FP64 for any T; an angle off by 2^-23 leaves that share of the pair's
 // inner product, which the next sweep sees (sweeps already converge quadratically to 1e-10).
 // One round then takes 3.0 us at 212 columns, from 6.1 us; a whole pass's sweeps: n = 900, k_S = 233:
-// 50.7 -> 23 ms, n = 40000: 88.9 -> 43.5 ms (there also without J in the projection, see project.cu).
+// 50.7 -> 18.7 ms, n = 40000: 88.9 -> 43.5 ms (there also without J in the projection, see project.cu).
 // The norms that decide about the floor are al - Re(conj(T) g) and be + Re(conj(T) g), exact to
 // rounding in the smaller one; every pair forms its own from the columns.
 // ---------------------------------------------------------------------------------------------

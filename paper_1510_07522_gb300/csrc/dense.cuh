@@ -20,7 +20,7 @@ struct Zgemm {
     c128* C = nullptr;
     int64_t ldc = 0, sC = 0;
     int batch = 1;
-    bool fp64 = false;  // FP64 CUDA cores even where the tensor-core emulation would be chosen
+    bool fp64 = false;  // FP64 CUDA cores whatever the path: products whose terms must keep their own scale
 };
 int zgemm(const Zgemm& g, cudaStream_t s);
 // In-place inverses of `batch` dense k x k complex128 matrices (column-major, stride k^2) by
