@@ -136,59 +136,91 @@ __global__ void csr_residual_kernel(const int64_t* rowptr, const int32_t* colind
 // deflation (Givens rotations), eigenvectors of the triangular Schur factor by back
 // substitution, back-transformed by the accumulated unitary Z.  Writes lam[n], X[n x n]
 // (unit columns).  status: 0 ok, 1 no convergence.
+//
+// The QR sweeps are a chain of rotations, so their latency is the kernel's time: a dependent FP64
+// operation takes 70-85 ns here, a division 260 ns, a square root 350 ns, an access to L2 as much
+// as four operations.  A and Z therefore stay in shared memory (n <= kEigSmemN), and the rotation is
+// [conj(x) conj(y); -y x] / sqrt(|x|^2 + |y|^2): unitary with one reciprocal square root (an FP32 seed
+// and one third-order step) and no phase, formed by every thread for itself.  n = 29: 5.2 -> 2.9 ms
+// against A and Z in global memory and rotations with a real cosine from one thread.
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) small_eig_kernel(c128* A, int n, c128* Z, c128* vtmp, c128* lam,
-                                                        c128* X, int* status) {
-    const int tid = threadIdx.x;
-    __shared__ c128 s_c, s_s, s_tau;
+constexpr int kEigThreads = 128;
+constexpr int kEigSmemN = 80;
+constexpr size_t eig_smem(int n) { return n <= kEigSmemN ? (size_t)2 * n * n * sizeof(c128) : 0; }
+
+// 1 / sqrt(v), v > 0 normal
+__device__ __forceinline__ double rsqrt64(double v) {
+    const int e = ((__double2hiint(v) >> 20) & 0x7ff) - 1023, h = e >> 1;       // v = m 4^h, m in [1, 4)
+    const double m = v * __hiloint2double((1023 - 2 * h) << 20, 0);
+    const double y = (double)rsqrtf((float)m), r = fma(-(m * y), y, 1.0);
+    return fma(fma(0.375, r, 0.5), y * r, y) * __hiloint2double((1023 - h) << 20, 0);
+}
+
+__global__ void __launch_bounds__(kEigThreads) small_eig_kernel(c128* Ag, int n, c128* Zg, c128* vtmp, c128* lam,
+                                                                c128* X, int* status) {
+    extern __shared__ __align__(16) unsigned char eig_dyn[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int NT = kEigThreads;
+    static_assert(NT == 128, "one warp for each scalar of a rotated pair");
+    __shared__ c128 s_tau, s_scal;
+    __shared__ double s_beta;
     __shared__ int s_flag;
+    const bool smem = n <= kEigSmemN;
+    c128* A = smem ? reinterpret_cast<c128*>(eig_dyn) : Ag;
+    c128* Z = smem ? A + n * n : Zg;
 #define Am(i, j) A[(i) + (int64_t)(j) * n]
 #define Zm(i, j) Z[(i) + (int64_t)(j) * n]
-    for (int idx = tid; idx < n * n; idx += 256) Z[idx] = (idx % n == idx / n) ? mk<double>(1.0, 0.0) : czero<double>();
+    for (int idx = tid; idx < n * n; idx += NT) {
+        if (smem) A[idx] = Ag[idx];
+        Z[idx] = (idx % n == idx / n) ? mk<double>(1.0, 0.0) : czero<double>();
+    }
     __syncthreads();
     // Hessenberg reduction
     for (int j = 0; j + 2 < n; ++j) {
         // reflector from A[j+1:n, j]
         double xs = 0.0;
-        for (int i = j + 2 + tid; i < n; i += 256) xs += cnorm2(Am(i, j));
+        for (int i = j + 2 + tid; i < n; i += NT) xs += cnorm2(Am(i, j));
         xs = block_sum_all(xs);
         if (tid == 0) {
             const c128 al = Am(j + 1, j);
-            if (xs == 0.0 && al.im == 0.0) {
-                s_tau = czero<double>();
-                s_flag = 1;
-            } else {
-                const double beta = -copysign(sqrt(al.re * al.re + al.im * al.im + xs), al.re);
-                s_tau = mk<double>((beta - al.re) / beta, -al.im / beta);
-                s_c = crecip(mk<double>(al.re - beta, al.im));
-                s_s = mk<double>(beta, 0.0);
-                s_flag = 0;
+            s_flag = xs == 0.0 && al.im == 0.0;
+            if (!s_flag) {
+                s_beta = -copysign(sqrt(al.re * al.re + al.im * al.im + xs), al.re);
+                s_tau = mk<double>((s_beta - al.re) / s_beta, -al.im / s_beta);
+                s_scal = crecip(mk<double>(al.re - s_beta, al.im));
             }
         }
         __syncthreads();
         if (s_flag) continue;
-        for (int i = tid; i < n; i += 256) vtmp[i] = (i < j + 1) ? czero<double>() : (i == j + 1 ? mk<double>(1.0, 0.0) : Am(i, j) * s_c);
+        for (int i = j + 1 + tid; i < n; i += NT) vtmp[i] = i == j + 1 ? mk<double>(1.0, 0.0) : Am(i, j) * s_scal;
         __syncthreads();
-        if (tid == 0) Am(j + 1, j) = s_s;
-        for (int i = j + 2 + tid; i < n; i += 256) Am(i, j) = czero<double>();
-        __syncthreads();
+        for (int i = j + 1 + tid; i < n; i += NT) Am(i, j) = i == j + 1 ? mk<double>(s_beta, 0.0) : czero<double>();
         const c128 tau = s_tau;
-        // A <- H^H A (columns j+1..n-1), H = I - tau v v^H
-        for (int c = j + 1 + tid; c < n; c += 256) {
-            c128 w = czero<double>();
-            for (int i = j + 1; i < n; ++i) cfma_conj(w, vtmp[i], Am(i, c));
-            const c128 f = cconj(tau) * w;
-            for (int i = j + 1; i < n; ++i) cfms(Am(i, c), vtmp[i], f);
+        // A <- H^H A (columns j+1..n-1), H = I - tau v v^H; four sums in flight
+        for (int c = j + 1 + tid; c < n; c += NT) {
+            c128 w[4] = {czero<double>(), czero<double>(), czero<double>(), czero<double>()};
+            int i = j + 1;
+            for (; i + 3 < n; i += 4)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) cfma_conj(w[u], vtmp[i + u], Am(i + u, c));
+            for (; i < n; ++i) cfma_conj(w[0], vtmp[i], Am(i, c));
+            const c128 f = cconj(tau) * ((w[0] + w[1]) + (w[2] + w[3]));
+#pragma unroll 4
+            for (i = j + 1; i < n; ++i) cfms(Am(i, c), vtmp[i], f);
         }
         __syncthreads();
         // A <- A H (rows 0..n-1), Z <- Z H
-        for (int r = tid; r < 2 * n; r += 256) {
-            c128* M = (r < n) ? A : Z;
-            const int rr = (r < n) ? r : r - n;
-            c128 w = czero<double>();
-            for (int i = j + 1; i < n; ++i) cfma(w, M[rr + (int64_t)i * n], vtmp[i]);
-            const c128 f = w * tau;
-            for (int i = j + 1; i < n; ++i) cfms(M[rr + (int64_t)i * n], f, cconj(vtmp[i]));
+        for (int r = tid; r < 2 * n; r += NT) {
+            c128* M = (r < n) ? A + r : Z + (r - n);
+            c128 w[4] = {czero<double>(), czero<double>(), czero<double>(), czero<double>()};
+            int i = j + 1;
+            for (; i + 3 < n; i += 4)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) cfma(w[u], M[(int64_t)(i + u) * n], vtmp[i + u]);
+            for (; i < n; ++i) cfma(w[0], M[(int64_t)i * n], vtmp[i]);
+            const c128 f = ((w[0] + w[1]) + (w[2] + w[3])) * tau;
+#pragma unroll 4
+            for (i = j + 1; i < n; ++i) cfms(M[(int64_t)i * n], f, cconj(vtmp[i]));
         }
         __syncthreads();
     }
@@ -196,21 +228,26 @@ __global__ void __launch_bounds__(256) small_eig_kernel(c128* A, int n, c128* Z,
     int hi = n - 1, iter = 0, total = 0;
     const double eps = 1.1102230246251565e-16;
     while (hi > 0) {
-        // deflation check (thread 0 decides, everyone follows)
-        if (tid == 0) {
-            int l = hi;
-            while (l > 0) {
-                const double sub = cabs1(Am(l, l - 1));
+        // deflation check, from the bottom: every warp finds the first negligible subdiagonal entry
+        int lo = 0;
+        for (int base = hi; base > 0; base -= 32) {
+            const int l = base - lane;
+            bool neg = false;
+            if (l > 0) {
                 const double dd = cabs1(Am(l, l)) + cabs1(Am(l - 1, l - 1));
-                if (sub <= eps * (dd == 0.0 ? 1.0 : dd)) { Am(l, l - 1) = czero<double>(); break; }
-                --l;
+                neg = cabs1(Am(l, l - 1)) <= eps * (dd == 0.0 ? 1.0 : dd);
             }
-            s_flag = l;
+            const unsigned m = __ballot_sync(0xffffffffu, neg);
+            if (m) { lo = base - (__ffs(m) - 1); break; }
         }
-        __syncthreads();
-        const int lo = s_flag;
-        __syncthreads();  // everyone has read s_flag before thread 0 may write it again
-        if (lo == hi) { --hi; iter = 0; continue; }
+        __syncthreads();  // everyone has looked before the entry is cleared
+        if (tid == 0 && lo > 0) Am(lo, lo - 1) = czero<double>();
+        if (lo == hi) {
+            --hi;
+            iter = 0;
+            __syncthreads();
+            continue;
+        }
         if (++total > 60 * n) { if (tid == 0) *status = 1; return; }
         ++iter;
         // Wilkinson shift from the trailing 2x2 (exceptional shift every 10 iterations)
@@ -235,57 +272,51 @@ __global__ void __launch_bounds__(256) small_eig_kernel(c128* A, int n, c128* Z,
         }
         // implicit single-shift QR sweep on [lo, hi] by Givens rotations
         for (int k = lo; k < hi; ++k) {
-            if (tid == 0) {
-                c128 x, y;
-                if (k == lo) { x = Am(lo, lo) - mu; y = Am(lo + 1, lo); }
-                else { x = Am(k, k - 1); y = Am(k + 1, k - 1); }
-                const double nx = sqrt(cnorm2(x)), ny = sqrt(cnorm2(y));
-                const double nr = sqrt(nx * nx + ny * ny);
-                if (nr == 0.0) { s_c = mk<double>(1.0, 0.0); s_s = czero<double>(); }
-                else {
-                    // G = [c s; -conj(s) c] with c real: G [x; y] = [r; 0]
-                    const double c = nx / nr;
-                    const c128 ph = (nx == 0.0) ? mk<double>(1.0, 0.0) : cscale(x, 1.0 / nx);
-                    const c128 s = cscale(ph * cconj(y), 1.0 / nr);
-                    s_c = mk<double>(c, 0.0);
-                    s_s = s;
-                }
+            const c128 x = k == lo ? Am(lo, lo) - mu : Am(k, k - 1), y = k == lo ? Am(lo + 1, lo) : Am(k + 1, k - 1);
+            const double r2 = fma(x.re, x.re, x.im * x.im) + fma(y.re, y.re, y.im * y.im);
+            c128 c = mk<double>(1.0, 0.0), s = czero<double>();
+            if (r2 >= 2.2250738585072014e-308) {
+                // G = [c s; -conj(s) conj(c)], G [x; y] = [sqrt(r2); 0]
+                const double iv = rsqrt64(r2);
+                c = mk<double>(x.re * iv, -x.im * iv);
+                s = mk<double>(y.re * iv, -y.im * iv);
             }
-            __syncthreads();
-            const double c = s_c.re;
-            const c128 s = s_s;
+            // Each warp forms one of the four scalars (u.re, u.im, v.re, v.im) of the new pair, so that
+            // the four sub-partitions share the FP64 instructions: c u + s v, conj(c) v - conj(s) u
+            // for the rows; the columns take G^H, the same coefficients with b and d negated.
+            const double pa = warp < 2 ? c.re : -s.re, pd = warp < 2 ? s.re : c.re;
+            double pb = warp < 2 ? c.im : s.im, pe = warp < 2 ? s.im : -c.im;
+            if ((warp & 1) == 0) { pb = -pb; pe = -pe; }
+            auto pair = [&](c128* pu, c128* pv, bool on, double b, double e) {
+                const c128 u = *pu, v = *pv;
+                double val;
+                if ((warp & 1) == 0) val = fma(pa, u.re, b * u.im) + fma(pd, v.re, e * v.im);
+                else val = fma(pa, u.im, b * u.re) + fma(pd, v.im, e * v.re);
+                __syncthreads();  // all four warps have read
+                double* q = reinterpret_cast<double*>(warp < 2 ? pu : pv) + (warp & 1);
+                if (on) *q = val;
+            };
             // rows k, k+1 from the left (columns from max(lo, k-1))
-            for (int col = max(lo, k - 1) + tid; col < n; col += 256) {
-                const c128 u = Am(k, col), v = Am(k + 1, col);
-                Am(k, col) = cscale(u, c) + s * v;
-                Am(k + 1, col) = cscale(v, c) - cconj(s) * u;
+            for (int c0 = max(lo, k - 1); c0 < n; c0 += 32) {
+                const int col = min(c0 + lane, n - 1);
+                pair(&Am(k, col), &Am(k + 1, col), c0 + lane < n, pb, pe);
             }
             __syncthreads();
-            // columns k, k+1 from the right (rows up to min(hi, k+2)), and Z
+            // columns k, k+1 from the right by G^H (rows up to min(hi, k+2)), and Z
             const int rmax = min(hi, k + 2);
-            for (int r = tid; r <= rmax + n; r += 256) {
-                if (r <= rmax) {
-                    const c128 u = Am(r, k), v = Am(r, k + 1);
-                    Am(r, k) = cscale(u, c) + cconj(s) * v;
-                    Am(r, k + 1) = cscale(v, c) - s * u;
-                } else {
-                    const int rr = r - rmax - 1;
-                    if (rr < n) {
-                        const c128 u = Zm(rr, k), v = Zm(rr, k + 1);
-                        Zm(rr, k) = cscale(u, c) + cconj(s) * v;
-                        Zm(rr, k + 1) = cscale(v, c) - s * u;
-                    }
-                }
+            for (int c0 = 0; c0 <= rmax + n; c0 += 32) {
+                const int r = min(c0 + lane, rmax + n);
+                c128* M = r <= rmax ? A + r : Z + (r - rmax - 1);
+                pair(M + (int64_t)k * n, M + (int64_t)(k + 1) * n, c0 + lane <= rmax + n, -pb, -pe);
             }
             __syncthreads();
         }
     }
     __syncthreads();
     // eigenvalues and eigenvectors of the triangular Schur form, back-transformed by Z
-    for (int k = tid; k < n; k += 256) lam[k] = Am(k, k);
-    __syncthreads();
+    for (int k = tid; k < n; k += NT) lam[k] = Am(k, k);
     const double small = 1e-300;
-    for (int k = tid; k < n; k += 256) {
+    for (int k = tid; k < n; k += NT) {
         // y = eigenvector of upper-triangular T for lambda_k, stored in column k of X (scratch)
         c128* y = X + (int64_t)k * n;
         for (int i = 0; i < n; ++i) y[i] = czero<double>();
@@ -294,28 +325,37 @@ __global__ void __launch_bounds__(256) small_eig_kernel(c128* A, int n, c128* Z,
         double tnorm = 0.0;
         for (int i = 0; i <= k; ++i) tnorm = fmax(tnorm, cabs1(Am(i, i)));
         for (int i = k - 1; i >= 0; --i) {
-            c128 s = czero<double>();
-            for (int j = i + 1; j <= k; ++j) cfma(s, Am(i, j), y[j]);
+            c128 w[4] = {czero<double>(), czero<double>(), czero<double>(), czero<double>()};
+            int j = i + 1;
+            for (; j + 3 <= k; j += 4)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) cfma(w[u], Am(i, j + u), y[j + u]);
+            for (; j <= k; ++j) cfma(w[0], Am(i, j), y[j]);
             c128 den = Am(i, i) - lk;
             if (cabs1(den) < eps * fmax(tnorm, small)) den = mk<double>(eps * fmax(tnorm, small), 0.0);
-            y[i] = czero<double>() - s * crecip(den);
+            y[i] = czero<double>() - ((w[0] + w[1]) + (w[2] + w[3])) * crecip(den);
         }
     }
     __syncthreads();
-    // X <- Z Y (in place per column is not possible: use vtmp as one column of workspace each)
-    for (int k = 0; k < n; ++k) {
-        for (int r = tid; r < n; r += 256) {
-            c128 s = czero<double>();
-            for (int j = 0; j <= k; ++j) cfma(s, Zm(r, j), X[j + (int64_t)k * n]);
-            vtmp[r] = s;
+    // X <- Z Y by way of A (no longer needed), then unit columns
+    for (int idx = tid; idx < n * n; idx += NT) {
+        const int r = idx % n, k = idx / n;
+        c128 w[2] = {czero<double>(), czero<double>()};
+        int j = 0;
+        for (; j + 1 <= k; j += 2) {
+            cfma(w[0], Zm(r, j), X[j + (int64_t)k * n]);
+            cfma(w[1], Zm(r, j + 1), X[j + 1 + (int64_t)k * n]);
         }
-        __syncthreads();
+        if (j <= k) cfma(w[0], Zm(r, j), X[j + (int64_t)k * n]);
+        A[idx] = w[0] + w[1];
+    }
+    __syncthreads();
+    for (int k = warp; k < n; k += NT / 32) {
         double nn = 0.0;
-        for (int r = tid; r < n; r += 256) nn += cnorm2(vtmp[r]);
-        nn = block_sum_all(nn);
+        for (int r = lane; r < n; r += 32) nn += cnorm2(Am(r, k));
+        for (int off = 16; off; off >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, off);
         const double inv = nn > 0 ? 1.0 / sqrt(nn) : 1.0;
-        for (int r = tid; r < n; r += 256) X[r + (int64_t)k * n] = cscale(vtmp[r], inv);
-        __syncthreads();
+        for (int r = lane; r < n; r += 32) X[r + (int64_t)k * n] = cscale(Am(r, k), inv);
     }
     if (tid == 0) *status = 0;
 #undef Am
@@ -573,6 +613,7 @@ int solve_run(rsrr_nep h, int N_S, int K, double tol_gap, int cap, double* lambd
         CUDAC(cudaMemcpyAsync(Hr, mom, (size_t)k * D * sizeof(c128), cudaMemcpyDeviceToDevice, st));
     }
 
+    CUDAC(cudaFuncSetAttribute(small_eig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)eig_smem(kEigSmemN)));
     // extract(nb): eigenvalues (host) and g = H_r W_0 Sigma_0^{-1} g' in G (k x nb, device)
     std::vector<zd> lam_h;
     auto extract = [&](int nb) -> int {
@@ -587,7 +628,7 @@ int solve_run(rsrr_nep h, int N_S, int K, double tol_gap, int cap, double* lambd
         a2.A = V0; a2.lda = D; a2.B = T1; a2.ldb = D; a2.C = Am; a2.ldc = nb;
         RSRR_TRY(zgemm(a2, st));
         { scale_cols_kernel<<<(unsigned)ceil_div((int64_t)nb * nb, 256), 256, 0, st>>>(Am, nb, nb, nb, sigsafe, 1); note_launch(); }
-        { small_eig_kernel<<<1, 256, 0, st>>>(Am, nb, Zs, vt, lam_d, Xe, est); note_launch(); }
+        { small_eig_kernel<<<1, kEigThreads, eig_smem(nb), st>>>(Am, nb, Zs, vt, lam_d, Xe, est); note_launch(); }
         RSRR_CUDA(cudaGetLastError());
         int hst = 0;
         std::vector<c128> lh(nb);
