@@ -5,8 +5,8 @@
 //      interchanges and L11^{-1} applied to the right half, rank-32 update of the right half,
 //      right leaf, its interchanges applied back to the left half).  A leaf is column-by-
 //      column getf2 (pivot by cabs1 = |re| + |im|, lowest row on ties).  Panels of at most
-//      ~380 (complex64) / ~190 (complex128) rows are staged in shared memory, taller ones are
-//      factored in place in global memory.
+//      ~380 (complex64) / ~190 (complex128) rows are staged in shared memory whole, taller ones by
+//      leaves of 16, 8 or 4 columns.
 //   2. the panel's 64 interchanges are composed into one permutation of the <= 128 rows they
 //      touch; inv(L11) and inv(U11) of the diagonal block are formed once.
 //   3. trailing rows: per block of columns, the touched rows are gathered, permuted, and the
@@ -15,7 +15,9 @@
 //      L21 tiles double-buffered in shared memory by cp.async, U12 block resident, each
 //      thread holding an 8 x 8 (4 x 4) block of the tile in registers.
 // The update is the dense contraction that carries (8/3) n^3 real flops per point; steps 1-3
-// are O(n^2 NB).
+// are O(n^2 NB), but they, the operand images and the FP64 residuals took 52 of the 62 ms of a point at
+// n = 1600.  With leaves in shared memory, 16-byte image stores, four columns a thread in step 3 and T
+// kept for the residuals, a pass of 32 such points takes 38 ms.
 #include <algorithm>
 #include <climits>
 #include <string>
@@ -83,6 +85,7 @@ struct DShared {
     int info;
     int job;
     int red_i[NW];
+    unsigned red_u[NW];
     double red_v[NW];
 };
 
@@ -104,35 +107,56 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
 
-// Row of the largest cabs1 in col[c..m) (lowest row on ties; c if every entry is NaN).
+// Row of the largest cabs1 in col[c..m) (lowest row on ties; c if every entry is NaN).  Complex64
+// compares the bit patterns (non-negative floats order like integers) with warp reductions of the
+// integer pipe: a conversion to FP64 would cost 64 clocks a warp and row.
 template <typename R>
 __device__ int col_argmax(const cplx<R>* col, int c, int m, DShared& sh) {
-    double best = -1.0;
-    int bi = INT_MAX;
-    for (int r = c + (int)threadIdx.x; r < m; r += NT) {
-        const double a = (double)cabs1(col[r]);
-        if (a > best) { best = a; bi = r; }
-    }
-    for (int off = 16; off; off >>= 1) {
-        const double ob = __shfl_down_sync(FULL, best, off);
-        const int oi = __shfl_down_sync(FULL, bi, off);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-    }
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) { sh.red_v[w] = best; sh.red_i[w] = bi; }
-    wsync();
-    if (w == 0) {
-        best = lane < NW ? sh.red_v[lane] : -1.0;
+    if constexpr (sizeof(R) == 4) {
+        unsigned best = 0;  // 1 + bits of the largest value so far
+        int bi = INT_MAX;
+        for (int r = c + (int)threadIdx.x; r < m; r += NT) {
+            const float a = cabs1(col[r]);
+            const unsigned key = a >= 0.f ? __float_as_uint(a) + 1u : 0u;  // 0: NaN
+            if (key > best) { best = key; bi = r; }
+        }
+        const unsigned top = __reduce_max_sync(FULL, best);
+        const int row = (int)__reduce_min_sync(FULL, (unsigned)(best == top ? bi : INT_MAX));
+        if (lane == 0) { sh.red_u[w] = top; sh.red_i[w] = row; }
+        wsync();
+        best = lane < NW ? sh.red_u[lane] : 0u;
         bi = lane < NW ? sh.red_i[lane] : INT_MAX;
+        const unsigned all = __reduce_max_sync(FULL, best);
+        const int res = (int)__reduce_min_sync(FULL, (unsigned)(best == all ? bi : INT_MAX));
+        return res == INT_MAX ? c : res;
+    } else {
+        double best = -1.0;
+        int bi = INT_MAX;
+        for (int r = c + (int)threadIdx.x; r < m; r += NT) {
+            const double a = (double)cabs1(col[r]);
+            if (a > best) { best = a; bi = r; }
+        }
         for (int off = 16; off; off >>= 1) {
             const double ob = __shfl_down_sync(FULL, best, off);
             const int oi = __shfl_down_sync(FULL, bi, off);
             if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
         }
-        if (lane == 0) sh.res = (bi == INT_MAX) ? c : bi;
+        if (lane == 0) { sh.red_v[w] = best; sh.red_i[w] = bi; }
+        wsync();
+        if (w == 0) {
+            best = lane < NW ? sh.red_v[lane] : -1.0;
+            bi = lane < NW ? sh.red_i[lane] : INT_MAX;
+            for (int off = 16; off; off >>= 1) {
+                const double ob = __shfl_down_sync(FULL, best, off);
+                const int oi = __shfl_down_sync(FULL, bi, off);
+                if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+            }
+            if (lane == 0) sh.res = (bi == INT_MAX) ? c : bi;
+        }
+        wsync();
+        return sh.res;
     }
-    wsync();
-    return sh.res;
 }
 
 // getf2 on the m x w block P (leading dimension ld): pivots piv[c] relative to row 0.
@@ -142,24 +166,24 @@ __device__ void leaf_factor(cplx<R>* P, int64_t ld, int m, int w, int* piv, int 
         cplx<R>* colc = P + (int64_t)c * ld;
         const int p = col_argmax(colc, c, m, sh);
         if (threadIdx.x == 0) piv[c] = p;
-        if (p != c)
-            for (int q = threadIdx.x; q < w; q += NT) {
-                cplx<R>* cq = P + (int64_t)q * ld;
-                const cplx<R> t = cq[c];
-                cq[c] = cq[p];
-                cq[p] = t;
+        // the interchange, and U row c of the leaf in shared memory (read by every thread); each row's
+        // entries are loaded in chunks before any is stored, so a tall leaf in global memory pays the
+        // memory latency once per chunk instead of once per column.
+        cplx<R>* urow = sh_u12<R>(sh);
+        if ((int)threadIdx.x < w) {
+            cplx<R>* cq = P + (int64_t)threadIdx.x * ld;
+            const cplx<R> t = cq[p];
+            urow[threadIdx.x] = t;
+            if (p != c) {
+                cq[p] = cq[c];
+                cq[c] = t;
             }
+        }
         wsync();
-        const cplx<R> pv = colc[c];
+        const cplx<R> pv = urow[c];
         const bool zero = cis_zero(pv);
         if (zero && threadIdx.x == 0 && sh.info == 0) sh.info = col_base + c + 1;
         const cplx<R> rp = zero ? czero<R>() : crecip(pv);
-        // U row c of the leaf in shared memory (read by every thread); each row's entries are
-        // loaded in chunks before any is stored, so a tall leaf in global memory pays the memory
-        // latency once per chunk instead of once per column.
-        cplx<R>* urow = sh_u12<R>(sh);
-        if ((int)threadIdx.x < w) urow[threadIdx.x] = P[c + (int64_t)threadIdx.x * ld];
-        wsync();
         constexpr int QL = sizeof(R) == 4 ? 16 : 8;
         for (int r = c + 1 + (int)threadIdx.x; r < m; r += NT) {
             cplx<R> l = colc[r];
@@ -265,14 +289,14 @@ __device__ void panel_factor(cplx<R>* P, int64_t ld, int m, int nbk, int col_bas
 // Compose the panel's interchanges (applied in order t = 0..nbk-1) into one permutation of the
 // rows they touch.  Entries 0..nbk-1 are the diagonal rows; further entries are pivot rows
 // below the panel's diagonal block.  Warp 0 does it; everyone waits.
-__device__ void compose_swaps(int nbk, DShared& sh) {
+__device__ void compose_swaps(int nbk, const int* piv, DShared& sh) {
     if (threadIdx.x < 32) {
         const int lane = threadIdx.x;
         for (int t = lane; t < nbk; t += 32) { sh.rows[t] = t; sh.src[t] = t; }
         __syncwarp();
         int cnt = nbk;
         for (int t = 0; t < nbk; ++t) {
-            const int p = sh.piv[t];
+            const int p = piv[t];
             if (p == t) continue;
             int e = -1;
             if (p < nbk) {
@@ -300,6 +324,84 @@ __device__ void compose_swaps(int nbk, DShared& sh) {
         if (lane == 0) sh.cnt = cnt;
     }
     wsync();
+}
+
+// panel_factor for a panel too tall for shared memory: leaves of lw columns (16, or fewer so that
+// m x lw fits), each factored in shared memory; then its interchanges, composed into one permutation, go
+// to the panel's other columns, and the columns right of it get their U rows and the rank-lw update.
+// The panel's columns cross L2 twice a leaf and column to its right (96 column passes for 64 columns),
+// against 1024 when every column of a 32-column leaf updated the others in global memory.
+constexpr int kLeafMax = 16;
+template <typename R>
+__device__ void panel_factor_tall(cplx<R>* P, int64_t ld, int m, int nbk, int lw, int col_base, cplx<R>* sm,
+                                  DShared& sh) {
+    const int tid = threadIdx.x;
+    cplx<R>* u = sh_u12<R>(sh);  // [right column][kLeafMax]
+    for (int w0 = 0; w0 < nbk; w0 += lw) {
+        const int w = min(lw, nbk - w0), mL = m - w0, nright = nbk - w0 - w, nother = nbk - w;
+        cplx<R>* L0 = P + w0 + (int64_t)w0 * ld;
+        for (int idx = tid; idx < mL * w; idx += NT) sm[idx] = L0[idx % mL + (int64_t)(idx / mL) * ld];
+        wsync();
+        leaf_factor(sm, (int64_t)mL, mL, w, sh.piv + w0, col_base + w0, sh);
+        compose_swaps(w, sh.piv + w0, sh);
+        for (int idx = tid; idx < mL * w; idx += NT) L0[idx % mL + (int64_t)(idx / mL) * ld] = sm[idx];
+        const int cnt = sh.cnt;  // at most 2 lw rows are touched
+        if (tid < w) sh.piv[w0 + tid] += w0;
+        {
+            constexpr int MV = 2 * kLeafMax * (NB - kLeafMax) / NT;  // cnt * nother <= 2 lw (NB - lw)
+            cplx<R> v[MV];
+#pragma unroll
+            for (int t = 0; t < MV; ++t) {
+                const int idx = tid + NT * t, e = idx % cnt, j = idx / cnt;
+                if (j < nother) v[t] = P[(w0 + sh.src[e]) + (int64_t)(j < w0 ? j : j + w) * ld];
+            }
+            wsync();
+#pragma unroll
+            for (int t = 0; t < MV; ++t) {
+                const int idx = tid + NT * t, e = idx % cnt, j = idx / cnt;
+                if (j < nother) P[(w0 + sh.rows[e]) + (int64_t)(j < w0 ? j : j + w) * ld] = v[t];
+            }
+        }
+        wsync();
+        if (nright == 0) continue;
+        cplx<R>* Rt = P + w0 + (int64_t)(w0 + w) * ld;
+        if (tid < nright) {  // U rows: unit lower solve of the leaf's top block
+            cplx<R> x[kLeafMax];
+#pragma unroll
+            for (int r = 0; r < kLeafMax; ++r) x[r] = r < w ? Rt[r + (int64_t)tid * ld] : czero<R>();
+#pragma unroll
+            for (int r = 1; r < kLeafMax; ++r)
+                if (r < w)
+#pragma unroll
+                    for (int t = 0; t < r; ++t) cfms(x[r], sm[r + t * mL], x[t]);
+#pragma unroll
+            for (int r = 0; r < kLeafMax; ++r) {
+                u[tid * kLeafMax + r] = x[r];
+                if (r < w) Rt[r + (int64_t)tid * ld] = x[r];
+            }
+        }
+        wsync();
+        constexpr int QC = sizeof(R) == 4 ? 16 : 8;
+        for (int r = w + tid; r < mL; r += NT) {
+            cplx<R> l[kLeafMax];
+#pragma unroll
+            for (int t = 0; t < kLeafMax; ++t) l[t] = t < w ? sm[r + t * mL] : czero<R>();
+            for (int q0 = 0; q0 < nright; q0 += QC) {
+                cplx<R> x[QC];
+#pragma unroll
+                for (int j = 0; j < QC; ++j)
+                    x[j] = (q0 + j < nright) ? Rt[r + (int64_t)(q0 + j) * ld] : czero<R>();
+#pragma unroll
+                for (int j = 0; j < QC; ++j)
+                    if (q0 + j < nright) {
+#pragma unroll
+                        for (int t = 0; t < kLeafMax; ++t) cfms(x[j], l[t], u[(q0 + j) * kLeafMax + t]);
+                        Rt[r + (int64_t)(q0 + j) * ld] = x[j];
+                    }
+            }
+        }
+        wsync();
+    }
 }
 
 // inv(L11) and inv(U11) of the nbk x nbk diagonal block of P; shared layout (r, c) at r * NBP + c:
@@ -380,17 +482,20 @@ __device__ void trailing_rows(cplx<R>* A, int64_t lda, int n, int k0, cplx<R>* s
             A[(int64_t)(k0 + sh.rows[e]) + (int64_t)(c0 + col) * lda] = g[col * 2 * NB + e];
         }
         {
+            // four columns a thread: one entry of inv(L11) and four broadcasts for 16 multiply-adds
             const int t = threadIdx.x % NB, grp = threadIdx.x / NB;
-            for (int col = grp; col < nc; col += NT / NB) {
-                const cplx<R>* gc = g + col * 2 * NB;
-                cplx<R> a0 = czero<R>(), a1 = czero<R>();
-                int s = 0;
-                for (; s + 1 <= t; s += 2) {
-                    cfma(a0, iL[t * NBP + s], gc[s]);
-                    cfma(a1, iL[t * NBP + s + 1], gc[s + 1]);
+            for (int cb = 4 * grp; cb < nc; cb += 4 * (NT / NB)) {
+                const cplx<R>* gc = g + cb * 2 * NB;
+                cplx<R> acc[4] = {czero<R>(), czero<R>(), czero<R>(), czero<R>()};
+#pragma unroll 4
+                for (int s = 0; s <= t; ++s) {
+                    const cplx<R> l = iL[t * NBP + s];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) cfma(acc[j], l, gc[j * 2 * NB + s]);
                 }
-                if (s <= t) cfma(a0, iL[t * NBP + s], gc[s]);
-                A[(int64_t)(k0 + t) + (int64_t)(c0 + col) * lda] = a0 + a1;
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (cb + j < nc) A[(int64_t)(k0 + t) + (int64_t)(c0 + cb + j) * lda] = acc[j];
             }
         }
         wsync();
@@ -505,46 +610,53 @@ struct TcPhase {
 
 __device__ __forceinline__ bool failed(const TcShared& ts) { return *(const volatile int*)&ts.fail != 0; }
 
-// Write the six BF16 pieces of (re, im) at (row r, k) of an operand image with `rows` rows:
-// array q (0..2 re hi/mid/lo, 3..5 im hi/mid/lo) occupies rows * 64 elements.
-__device__ __forceinline__ void put_split(__nv_bfloat16* t, int r, int k, int rows, float re, float im) {
-    const uint32_t at = sw128_index16(r, k), stride = (uint32_t)rows * NB;
-    float x[2] = {re, im};
+// Write the six BF16 pieces of v[0..8) at (row r, k..k+7) of an operand image with `rows` rows: array q
+// (0..2 re hi/mid/lo, 3..5 im hi/mid/lo) occupies rows * 64 elements.  Eight consecutive k are one
+// 16-byte unit of the swizzled layout.
+__device__ __forceinline__ void put_split8(float* img, int r, int k, int rows, const c64* v) {
+    unsigned char* t = reinterpret_cast<unsigned char*>(img) + sw128_index16(r, k) * 2;
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-        const __nv_bfloat16 h = __float2bfloat16_rn(x[c]);
-        const float r1 = x[c] - __bfloat162float(h);
-        const __nv_bfloat16 m = __float2bfloat16_rn(r1);
-        const __nv_bfloat16 l = __float2bfloat16_rn(r1 - __bfloat162float(m));
-        t[(3 * c + 0) * stride + at] = h;
-        t[(3 * c + 1) * stride + at] = m;
-        t[(3 * c + 2) * stride + at] = l;
+        __align__(16) __nv_bfloat16 h[8], m[8], l[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const float x = c ? v[e].im : v[e].re;
+            h[e] = __float2bfloat16_rn(x);
+            const float r1 = x - __bfloat162float(h[e]);
+            m[e] = __float2bfloat16_rn(r1);
+            l[e] = __float2bfloat16_rn(r1 - __bfloat162float(m[e]));
+        }
+        const size_t stride = (size_t)rows * NB * 2;
+        *reinterpret_cast<uint4*>(t + (3 * c + 0) * stride) = *reinterpret_cast<const uint4*>(h);
+        *reinterpret_cast<uint4*>(t + (3 * c + 1) * stride) = *reinterpret_cast<const uint4*>(m);
+        *reinterpret_cast<uint4*>(t + (3 * c + 2) * stride) = *reinterpret_cast<const uint4*>(l);
     }
 }
-
 
 // L21 (rows k0+NB.., panel columns) -> one image per 128-row tile; rows past n are zero.
 __device__ void emit_a_image(const c64* A, int64_t lda, int n, int k0, float* img) {
     const int r_begin = k0 + NB, m = n - r_begin;
     const int rows_pad = (m + TC_ROWS - 1) / TC_ROWS * TC_ROWS;
-    for (int idx = threadIdx.x; idx < rows_pad * NB; idx += NT) {
-        const int rr = idx % rows_pad, k = idx / rows_pad;
-        c64 v = czero<float>();
-        if (rr < m) v = A[(int64_t)(r_begin + rr) + (int64_t)(k0 + k) * lda];
-        put_split(reinterpret_cast<__nv_bfloat16*>(img + (size_t)(rr / TC_ROWS) * TC_A_FLOATS), rr % TC_ROWS, k,
-                  TC_ROWS, v.re, v.im);
+    for (int idx = threadIdx.x; idx < rows_pad * (NB / 8); idx += NT) {
+        const int rr = idx % rows_pad, k = idx / rows_pad * 8;
+        c64 v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            v[e] = rr < m ? A[(int64_t)(r_begin + rr) + (int64_t)(k0 + k + e) * lda] : czero<float>();
+        put_split8(img + (size_t)(rr / TC_ROWS) * TC_A_FLOATS, rr % TC_ROWS, k, TC_ROWS, v);
     }
 }
 // U12 (panel rows, columns k0+NB..) -> one image per 128-column block; columns past n are zero.
 __device__ void emit_b_image(const c64* A, int64_t lda, int n, int k0, float* img) {
     const int c_begin = k0 + NB, m = n - c_begin;
     const int cols_pad = (m + TC_COLS - 1) / TC_COLS * TC_COLS;
-    for (int idx = threadIdx.x; idx < cols_pad * NB; idx += NT) {
-        const int k = idx % NB, cc = idx / NB;
-        c64 v = czero<float>();
-        if (cc < m) v = A[(int64_t)(k0 + k) + (int64_t)(c_begin + cc) * lda];
-        put_split(reinterpret_cast<__nv_bfloat16*>(img + (size_t)(cc / TC_COLS) * TC_B_FLOATS), cc % TC_COLS, k,
-                  TC_COLS, v.re, v.im);
+    for (int idx = threadIdx.x; idx < cols_pad * (NB / 8); idx += NT) {
+        const int k = idx % (NB / 8) * 8, cc = idx / (NB / 8);
+        c64 v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            v[e] = cc < m ? A[(int64_t)(k0 + k + e) + (int64_t)(c_begin + cc) * lda] : czero<float>();
+        put_split8(img + (size_t)(cc / TC_COLS) * TC_B_FLOATS, cc % TC_COLS, k, TC_COLS, v);
     }
 }
 
@@ -732,10 +844,14 @@ __device__ void factor_one(const DenseJob<R>& J, cplx<R>* sm, DShared& sh, float
             }
             wsync();
         } else {
-            panel_factor(Pg, lda, m, nbk, k0, sh);
+            int lw = kLeafMax;
+            while (lw > 2 && (size_t)m * lw * sizeof(cplx<R>) > factor_smem<R>()) lw /= 2;
+            // leaves of fewer than 4 columns would cross L2 as often as the columns themselves
+            if (lw >= 4) panel_factor_tall(Pg, lda, m, nbk, lw, k0, sm, sh);
+            else panel_factor(Pg, lda, m, nbk, k0, sh);
         }
         if ((int)threadIdx.x < nbk) J.ipiv[k0 + threadIdx.x] = k0 + sh.piv[threadIdx.x];
-        compose_swaps(nbk, sh);
+        compose_swaps(nbk, sh.piv, sh);
         int32_t* sw = J.swaps + (int64_t)p * kDenseSwapInts;
         if (threadIdx.x == 0) sw[0] = sh.cnt;
         for (int i = threadIdx.x; i < 2 * NB; i += NT) {
@@ -906,16 +1022,17 @@ struct Slot {
     cplx<R>* inv;
     int32_t* swaps;
     double* colsum;
+    c128* tv;  // T(z_j) on the CSR pattern
 };
 
 __host__ __device__ inline size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 template <typename R>
-__host__ __device__ inline size_t slot_bytes(int n_max, int L_max) {
+__host__ __device__ inline size_t slot_bytes(int n_max, int L_max, int64_t nnz_max) {
     const size_t np = (size_t)dense_panels(n_max);
     return align256((size_t)n_max * n_max * sizeof(cplx<R>)) + align256((size_t)n_max * L_max * sizeof(cplx<R>)) +
            align256((size_t)n_max * 4) + align256(np * 2 * NB * NB * sizeof(cplx<R>)) +
-           align256(np * kDenseSwapInts * 4) + align256((size_t)n_max * 8);
+           align256(np * kDenseSwapInts * 4) + align256((size_t)n_max * 8) + align256((size_t)nnz_max * sizeof(c128));
 }
 
 template <typename R>
@@ -934,6 +1051,8 @@ __device__ Slot<R> slot_at(unsigned char* base, int n_max, int L_max) {
     t.swaps = reinterpret_cast<int32_t*>(p);
     p += align256(np * kDenseSwapInts * 4);
     t.colsum = reinterpret_cast<double*>(p);
+    p += align256((size_t)n_max * 8);
+    t.tv = reinterpret_cast<c128*>(p);
     return t;
 }
 
@@ -948,51 +1067,40 @@ __device__ double worker_max(double v, SampleShared& ss) {
     return m;
 }
 
-// r = U - T X (FP64, T from the CSR values and f_i(z_j)); x = r in precision R; per-column
-// ||r||^2 and ||X||^2 into ss.rn2 / ss.xn2.
+// r = U - T X (FP64, T's CSR values tv); x = r in precision R; per-column ||r||^2 and ||X||^2 into
+// ss.rn2 / ss.xn2.  A warp takes a row: lane = (column of a group of 8, one of 4 entries), so that no
+// lane idles; the FP64 rate bounds it (two multiply-adds a clock: 1 ms for 132000 entries and 8
+// columns, where a thread a row and T formed anew from its terms took 2.7 ms).
 template <typename R>
-__device__ void residual_one(const DenseNep& E, int j, const c128* X, cplx<R>* x, SampleShared& ss) {
-    constexpr int LC = 8;
-    const int n = E.n, L = E.L, J = E.J;
-    const int64_t nnz = E.nnz;
-    const c128* f = E.F + (int64_t)j * J;
+__device__ void residual_one(const DenseNep& E, const c128* X, const c128* tv, cplx<R>* x, SampleShared& ss) {
+    const int n = E.n, L = E.L, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane >> 3;
     for (int l = threadIdx.x; l < L; l += NT) ss.rn2[l] = ss.xn2[l] = 0.0;
     wsync();
-    for (int l0 = 0; l0 < L; l0 += LC) {
-        double pr[LC], px[LC];
+    for (int l0 = 0; l0 < L; l0 += 8) {
+        const int l = l0 + (lane & 7);
+        const bool on = l < L;
+        const c128* Xl = X + (int64_t)(on ? l : l0) * n;
+        double pr = 0.0, px = 0.0;
+        for (int r = warp; r < n; r += NW) {
+            const int64_t end = E.rowptr[r + 1];
+            c128 acc = czero<double>();
+#pragma unroll 4
+            for (int64_t k = E.rowptr[r] + sub; k < end; k += 4) cfma(acc, tv[k], Xl[E.colind[k]]);
 #pragma unroll
-        for (int l = 0; l < LC; ++l) pr[l] = px[l] = 0.0;
-        for (int r = threadIdx.x; r < n; r += NT) {
-            c128 acc[LC];
-#pragma unroll
-            for (int l = 0; l < LC; ++l) acc[l] = (l0 + l < L) ? E.U[r + (int64_t)(l0 + l) * n] : czero<double>();
-            for (int64_t k = E.rowptr[r]; k < E.rowptr[r + 1]; ++k) {
-                c128 t = czero<double>();
-                for (int i = 0; i < J; ++i) cfma(t, f[i], E.vals[(int64_t)i * nnz + k]);
-                const int64_t c = E.colind[k];
-#pragma unroll
-                for (int l = 0; l < LC; ++l)
-                    if (l0 + l < L) cfms(acc[l], t, X[c + (int64_t)(l0 + l) * n]);
+            for (int off = 8; off <= 16; off <<= 1) {
+                acc.re += __shfl_xor_sync(FULL, acc.re, off);
+                acc.im += __shfl_xor_sync(FULL, acc.im, off);
             }
-#pragma unroll
-            for (int l = 0; l < LC; ++l)
-                if (l0 + l < L) {
-                    x[r + (int64_t)(l0 + l) * n] = ccast<R>(acc[l]);
-                    pr[l] += cnorm2(acc[l]);
-                    px[l] += cnorm2(X[r + (int64_t)(l0 + l) * n]);
-                }
+            if (sub == 0 && on) {
+                const c128 res = E.U[r + (int64_t)l * n] - acc;
+                x[r + (int64_t)l * n] = ccast<R>(res);
+                pr += cnorm2(res);
+                px += cnorm2(Xl[r]);
+            }
         }
-#pragma unroll
-        for (int l = 0; l < LC; ++l) {
-            double a = pr[l], b = px[l];
-            for (int off = 16; off; off >>= 1) {
-                a += __shfl_down_sync(FULL, a, off);
-                b += __shfl_down_sync(FULL, b, off);
-            }
-            if ((threadIdx.x & 31) == 0 && l0 + l < L) {
-                atomicAdd(&ss.rn2[l0 + l], a);
-                atomicAdd(&ss.xn2[l0 + l], b);
-            }
+        if (sub == 0 && on) {
+            atomicAdd(&ss.rn2[l], pr);
+            atomicAdd(&ss.xn2[l], px);
         }
     }
     wsync();
@@ -1014,6 +1122,7 @@ __device__ void sample_one(const DenseNep& E, int j, const Slot<R>& sl, cplx<R>*
         for (int64_t k = threadIdx.x; k < nnz; k += NT) {
             c128 t = czero<double>();
             for (int i = 0; i < J; ++i) cfma(t, f[i], E.vals[(int64_t)i * nnz + k]);
+            sl.tv[k] = t;
             const int c = E.colind[k];
             A[E.rowidx[k] + (int64_t)c * n] = ccast<R>(t);
             atomicAdd(&sl.colsum[c], sqrt(cnorm2(t)));
@@ -1056,7 +1165,7 @@ __device__ void sample_one(const DenseNep& E, int j, const Slot<R>& sl, cplx<R>*
     double prev = 0.0;
     int sweeps = 0;
     for (;;) {
-        residual_one(E, j, X, sl.x, ss);
+        residual_one(E, X, sl.tv, sl.x, ss);
         // backward error per column and the decision (one thread decides, all follow)
         double mx = 0.0;
         int nonfinite = 0;
@@ -1184,8 +1293,8 @@ int sm_count() {
 int dense_sample_grid(int njobs) { return std::max(1, std::min(njobs, sm_count())); }
 
 template <typename R>
-size_t dense_slot_bytes(int n_max, int L_max) {
-    return slot_bytes<R>(n_max, L_max);
+size_t dense_slot_bytes(int n_max, int L_max, int64_t nnz_max) {
+    return slot_bytes<R>(n_max, L_max, nnz_max);
 }
 
 template <typename R>
@@ -1197,7 +1306,7 @@ size_t dense_image_bytes(int n_max) {
 
 template <typename R>
 int launch_dense_sample(const DenseNep* d_neps, const DenseSampleJob* d_jobs, int njobs, int n_max, int L_max,
-                        int grid, void* d_slots, void* d_img, int32_t* d_next, DenseSampleCfg cfg, cudaStream_t s) {
+                        int64_t nnz_max, int grid, void* d_slots, void* d_img, int32_t* d_next, DenseSampleCfg cfg, cudaStream_t s) {
     if (njobs <= 0) return RSRR_OK;
     if (L_max > kMaxL) return set_error(RSRR_EINVAL, "dense sampling: L above 256");
     if (sizeof(R) == 4 && !d_img) return set_error(RSRR_EINVAL, "dense sampling: operand images missing");
@@ -1210,7 +1319,7 @@ int launch_dense_sample(const DenseNep* d_neps, const DenseSampleJob* d_jobs, in
     {
         dense_sample_kernel<R><<<grid, threads, sm, s>>>(d_neps, d_jobs, njobs, n_max, L_max,
                                                          static_cast<unsigned char*>(d_slots),
-                                                         dense_slot_bytes<R>(n_max, L_max), static_cast<float*>(d_img),
+                                                         dense_slot_bytes<R>(n_max, L_max, nnz_max), static_cast<float*>(d_img),
                                                          img_stride, img_b, d_next, cfg);
         note_launch();
     }
@@ -1218,13 +1327,13 @@ int launch_dense_sample(const DenseNep* d_neps, const DenseSampleJob* d_jobs, in
     return RSRR_OK;
 }
 
-template size_t dense_slot_bytes<float>(int, int);
-template size_t dense_slot_bytes<double>(int, int);
+template size_t dense_slot_bytes<float>(int, int, int64_t);
+template size_t dense_slot_bytes<double>(int, int, int64_t);
 template size_t dense_image_bytes<float>(int);
 template size_t dense_image_bytes<double>(int);
-template int launch_dense_sample<float>(const DenseNep*, const DenseSampleJob*, int, int, int, int, void*, void*,
+template int launch_dense_sample<float>(const DenseNep*, const DenseSampleJob*, int, int, int, int64_t, int, void*, void*,
                                         int32_t*, DenseSampleCfg, cudaStream_t);
-template int launch_dense_sample<double>(const DenseNep*, const DenseSampleJob*, int, int, int, int, void*, void*,
+template int launch_dense_sample<double>(const DenseNep*, const DenseSampleJob*, int, int, int, int64_t, int, void*, void*,
                                          int32_t*, DenseSampleCfg, cudaStream_t);
 
 }  // namespace rsrr

@@ -73,9 +73,9 @@ struct DenseSampleCfg {
     int32_t max_refine;
 };
 
-// Device bytes of one CTA's slot for n <= n_max, L <= L_max.
+// Device bytes of one CTA's slot for n <= n_max, L <= L_max, nnz <= nnz_max.
 template <typename R>
-size_t dense_slot_bytes(int n_max, int L_max);
+size_t dense_slot_bytes(int n_max, int L_max, int64_t nnz_max);
 // Largest CTA count worth launching for njobs jobs (one per SM at most).
 int dense_sample_grid(int njobs);
 // Device bytes of one CTA's tensor-core operand images (complex64; 0 for complex128).
@@ -84,6 +84,6 @@ size_t dense_image_bytes(int n_max);
 // d_slots: grid * dense_slot_bytes; d_img: grid * dense_image_bytes; d_next: one int32.
 template <typename R>
 int launch_dense_sample(const DenseNep* d_neps, const DenseSampleJob* d_jobs, int njobs, int n_max, int L_max,
-                        int grid, void* d_slots, void* d_img, int32_t* d_next, DenseSampleCfg cfg, cudaStream_t s);
+                        int64_t nnz_max, int grid, void* d_slots, void* d_img, int32_t* d_next, DenseSampleCfg cfg, cudaStream_t s);
 
 }  // namespace rsrr

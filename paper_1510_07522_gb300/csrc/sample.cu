@@ -507,8 +507,9 @@ int sample_dense_set(const std::vector<rsrr_nep>& hs, const std::vector<c128*>& 
     cudaStream_t st = hs[0]->stream;
     const int nh = (int)hs.size();
     int n_max = 0, L_max = 0;
-    int64_t total_points = 0;
+    int64_t total_points = 0, nnz_max = 0;
     for (rsrr_nep h : hs) {
+        nnz_max = std::max<int64_t>(nnz_max, h->nnz);
         n_max = std::max<int>(n_max, (int)h->n);
         L_max = std::max<int>(L_max, h->L);
         total_points += h->N;
@@ -526,7 +527,7 @@ int sample_dense_set(const std::vector<rsrr_nep>& hs, const std::vector<c128*>& 
     // CTAs: one per SM at most, and no more slots than the free memory holds
     size_t free_b = 0, total_b = 0;
     RSRR_CUDA(cudaMemGetInfo(&free_b, &total_b));
-    const size_t per_cta = dense_slot_bytes<R>(n_max, L_max) + dense_image_bytes<R>(n_max);
+    const size_t per_cta = dense_slot_bytes<R>(n_max, L_max, nnz_max) + dense_image_bytes<R>(n_max);
     const size_t budget = (size_t)(0.8 * (double)free_b);
     const int grid = (int)std::min<size_t>((size_t)dense_sample_grid(njobs), budget / per_cta);
     if (grid < 1) return set_error(RSRR_ENOMEM, "one dense sampling slot does not fit in device memory");
@@ -573,7 +574,7 @@ int sample_dense_set(const std::vector<rsrr_nep>& hs, const std::vector<c128*>& 
     TRYD(dalloc_n(&d_neps, (size_t)nh, st));
     TRYD(dalloc_n(&d_jobs, (size_t)njobs, st));
     TRYD(dalloc_n(&d_next, 1, st));
-    TRYD(dalloc(&d_slots, (size_t)grid * dense_slot_bytes<R>(n_max, L_max), st));
+    TRYD(dalloc(&d_slots, (size_t)grid * dense_slot_bytes<R>(n_max, L_max, nnz_max), st));
     if (dense_image_bytes<R>(n_max)) TRYD(dalloc(&d_img, (size_t)grid * dense_image_bytes<R>(n_max), st));
     CUDAD(cudaMemcpyAsync(d_neps, neps.data(), neps.size() * sizeof(DenseNep), cudaMemcpyHostToDevice, st));
     CUDAD(cudaMemcpyAsync(d_jobs, jobs.data(), jobs.size() * sizeof(DenseSampleJob), cudaMemcpyHostToDevice, st));
@@ -583,7 +584,7 @@ int sample_dense_set(const std::vector<rsrr_nep>& hs, const std::vector<c128*>& 
     cfg.max_refine = max_refine;
     EvPair ev;
     ev.start(st);
-    TRYD(launch_dense_sample<R>(d_neps, d_jobs, njobs, n_max, L_max, grid, d_slots, d_img, d_next, cfg, st));
+    TRYD(launch_dense_sample<R>(d_neps, d_jobs, njobs, n_max, L_max, nnz_max, grid, d_slots, d_img, d_next, cfg, st));
     ev.stop(st);
     bool singular = false, timeout = false, nonfinite = false, notconv = false;
     for (int i = 0; i < nh; ++i) {
