@@ -1,4 +1,5 @@
-// Dense complex LU with partial pivoting, one CTA per sampling point, and its block solves.
+// Dense complex LU with partial pivoting, one thread-block cluster (1, 2, 4 or 8 CTAs) per sampling
+// point, and its block solves.
 //
 // Factorisation of one point (right-looking, panels of NB = 64 columns):
 //   1. panel: the m x 64 panel is factored as two 32-column leaves (left leaf, its
@@ -17,17 +18,24 @@
 // The update is the dense contraction that carries (8/3) n^3 real flops per point; steps 1-3
 // are O(n^2 NB), but they, the operand images and the FP64 residuals took 52 of the 62 ms of a point at
 // n = 1600.  With leaves in shared memory, 16-byte image stores, four columns a thread in step 3 and T
-// kept for the residuals, a pass of 32 such points takes 38 ms.
+// kept for the residuals, a pass of 32 such points takes 38 ms on 32 CTAs, and 16 ms with a cluster of
+// four CTAs a point (CTA 0 factors the panels, everything else is dealt out).
 #include <algorithm>
 #include <climits>
+#include <functional>
+#include <queue>
 #include <string>
+#include <vector>
 
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include "dense_lu.cuh"
 #include "tc.cuh"
 
 namespace rsrr {
+
+namespace cg = cooperative_groups;
 
 namespace {
 using namespace tc;
@@ -76,6 +84,8 @@ constexpr size_t factor_smem() {
 }
 
 struct DShared {
+    uint64_t cbar;      // the cluster's barrier: one arrival per CTA
+    int cok;
     double2 u12[32 * 32];  // U12 of the panel's left leaf (32 x 32, complex64 or complex128)
     int piv[NB];        // panel pivots, relative to the panel's first row
     int rows[2 * NB];   // composed interchanges: row rows[e] receives row src[e]
@@ -88,6 +98,42 @@ struct DShared {
     unsigned red_u[NW];
     double red_v[NW];
 };
+
+// The worker threads of the cluster's CTAs.  `fail` is sticky and the same for all of a CTA's workers.
+struct Cluster {
+    int rank = 0, size = 1;
+    uint32_t phase = 0;
+    bool fail = false;
+};
+
+// Barrier of all workers of the cluster, ordering their global and shared memory accesses.  The
+// hardware cluster barrier counts every thread, and the tensor-core producer warp takes no part, so the
+// CTAs arrive on one another's mbarrier.  Bounded: when a wait gives up, `fail` is set and no
+// later one is entered (the other CTAs then run out of arrivals and give up too).
+__device__ __forceinline__ bool csync(Cluster& c, DShared& sh) {
+    wsync();
+    if (c.size == 1 || c.fail) return !c.fail;
+    if ((int)threadIdx.x < c.size) {
+        __threadfence();
+        asm volatile("{\n .reg .b32 ra;\n mapa.shared::cluster.u32 ra, %0, %1;\n"
+                     " mbarrier.arrive.release.cluster.shared::cluster.b64 _, [ra];\n}\n" ::"r"(smem_u32(&sh.cbar)),
+                     "r"(threadIdx.x) : "memory");
+    }
+    if (threadIdx.x == 0) {
+        uint32_t done = 0;
+        for (uint32_t it = 0; it < (1u << 21) && !done; ++it) {
+            asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+                         " selp.u32 %0, 1, 0, p;\n}\n" : "=r"(done) : "r"(smem_u32(&sh.cbar)), "r"(c.phase) : "memory");
+            if (!done && it > 4096) __nanosleep(64);
+        }
+        __threadfence();
+        sh.cok = (int)done;
+    }
+    wsync();
+    c.phase ^= 1;
+    if (!sh.cok) c.fail = true;
+    return !c.fail;
+}
 
 template <typename R>
 __device__ __forceinline__ cplx<R>* sh_u12(DShared& sh) { return reinterpret_cast<cplx<R>*>(sh.u12); }
@@ -331,6 +377,7 @@ __device__ void compose_swaps(int nbk, const int* piv, DShared& sh) {
 // to the panel's other columns, and the columns right of it get their U rows and the rank-lw update.
 // The panel's columns cross L2 twice a leaf and column to its right (96 column passes for 64 columns),
 // against 1024 when every column of a 32-column leaf updated the others in global memory.
+constexpr double kDenseSerial = 0.25;  // share of a point's time in its panels (dense_plan)
 constexpr int kLeafMax = 16;
 template <typename R>
 __device__ void panel_factor_tall(cplx<R>* P, int64_t ld, int m, int nbk, int lw, int col_base, cplx<R>* sm,
@@ -406,9 +453,9 @@ __device__ void panel_factor_tall(cplx<R>* P, int64_t ld, int m, int nbk, int lw
 
 // inv(L11) and inv(U11) of the nbk x nbk diagonal block of P; shared layout (r, c) at r * NBP + c:
 // sm[0 ..) = inv(L11), then inv(U11), then a copy of the block (its padding column holds 1/U(r,r)).
-// Both go to ginv (column-major, leading dimension NB, zero outside nbk x nbk).
+// Both go to ginv (column-major, leading dimension NB, zero outside nbk x nbk) when `write`.
 template <typename R>
-__device__ void diag_inverses(const cplx<R>* P, int64_t ld, int nbk, cplx<R>* sm, cplx<R>* ginv) {
+__device__ void diag_inverses(const cplx<R>* P, int64_t ld, int nbk, cplx<R>* sm, cplx<R>* ginv, bool write) {
     cplx<R>* iL = sm;
     cplx<R>* iU = sm + NB * NBP;
     cplx<R>* T = sm + 2 * NB * NBP;
@@ -453,7 +500,7 @@ __device__ void diag_inverses(const cplx<R>* P, int64_t ld, int nbk, cplx<R>* sm
         }
     }
     wsync();
-    for (int idx = threadIdx.x; idx < NB * NB; idx += NT) {
+    for (int idx = threadIdx.x; write && idx < NB * NB; idx += NT) {
         const int r = idx % NB, c = idx / NB;
         const bool in = r < nbk && c < nbk;
         ginv[idx] = in ? iL[r * NBP + c] : czero<R>();
@@ -463,14 +510,16 @@ __device__ void diag_inverses(const cplx<R>* P, int64_t ld, int nbk, cplx<R>* sm
 }
 
 // Trailing columns, rows of the panel: apply the composed interchanges and form
-// U12 = inv(L11) * (pivot rows), block of TN columns at a time.  sm[0..NB*NBP) = inv(L11).
+// U12 = inv(L11) * (pivot rows), block of TN columns at a time, blocks dealt out over the cluster.
+// sm[0..NB*NBP) = inv(L11).
 template <typename R>
-__device__ void trailing_rows(cplx<R>* A, int64_t lda, int n, int k0, cplx<R>* sm, const DShared& sh) {
+__device__ void trailing_rows(cplx<R>* A, int64_t lda, int n, int k0, cplx<R>* sm, const DShared& sh,
+                              const Cluster& cl) {
     constexpr int TN = DTile<R>::TN;
     const cplx<R>* iL = sm;
     cplx<R>* g = sm + NB * NBP;  // gathered rows, g[col * 2NB + e]
     const int cnt = sh.cnt, extra = cnt - NB;
-    for (int c0 = k0 + NB; c0 < n; c0 += TN) {
+    for (int c0 = k0 + NB + cl.rank * TN; c0 < n; c0 += cl.size * TN) {
         const int nc = min(TN, n - c0);
         for (int idx = threadIdx.x; idx < cnt * nc; idx += NT) {
             const int e = idx % cnt, col = idx / cnt;
@@ -504,7 +553,7 @@ __device__ void trailing_rows(cplx<R>* A, int64_t lda, int n, int k0, cplx<R>* s
 
 // A22 -= L21 * U12 over rows and columns [k0 + NB, n).
 template <typename R>
-__device__ void trailing_update(cplx<R>* A, int64_t lda, int n, int k0, cplx<R>* sm) {
+__device__ void trailing_update(cplx<R>* A, int64_t lda, int n, int k0, cplx<R>* sm, const Cluster& cl) {
     using T = DTile<R>;
     constexpr int TM = T::TM, TN = T::TN, MI = T::MI, MJ = T::MJ, TNP = TN + 1;
     cplx<R>* As = sm;                 // [2][NB][TM]
@@ -520,7 +569,7 @@ __device__ void trailing_update(cplx<R>* A, int64_t lda, int n, int k0, cplx<R>*
             cp_elem(&buf[k * TM + r], ok ? L21 + (i0 + r) + (int64_t)k * lda : A, ok);
         }
     };
-    for (int c0 = r_begin; c0 < n; c0 += TN) {
+    for (int c0 = r_begin + cl.rank * TN; c0 < n; c0 += cl.size * TN) {
         const int ce = min(n, c0 + TN);
         for (int idx = tid; idx < NB * TN; idx += NT) {
             const int k = idx % NB, c = idx / NB;
@@ -603,6 +652,7 @@ struct TcShared {
     int64_t lda;
     const float* imgA;
     const float* imgB;
+    int rank, size;      // of the cluster: step g of an update is CTA g % size's
 };
 struct TcPhase {
     uint32_t a = 0, b = 0, go = 0, e[2] = {0, 0}, d[2] = {0, 0};
@@ -634,10 +684,10 @@ __device__ __forceinline__ void put_split8(float* img, int r, int k, int rows, c
 }
 
 // L21 (rows k0+NB.., panel columns) -> one image per 128-row tile; rows past n are zero.
-__device__ void emit_a_image(const c64* A, int64_t lda, int n, int k0, float* img) {
+__device__ void emit_a_image(const c64* A, int64_t lda, int n, int k0, float* img, const Cluster& cl) {
     const int r_begin = k0 + NB, m = n - r_begin;
     const int rows_pad = (m + TC_ROWS - 1) / TC_ROWS * TC_ROWS;
-    for (int idx = threadIdx.x; idx < rows_pad * (NB / 8); idx += NT) {
+    for (int idx = cl.rank * NT + threadIdx.x; idx < rows_pad * (NB / 8); idx += cl.size * NT) {
         const int rr = idx % rows_pad, k = idx / rows_pad * 8;
         c64 v[8];
 #pragma unroll
@@ -646,12 +696,15 @@ __device__ void emit_a_image(const c64* A, int64_t lda, int n, int k0, float* im
         put_split8(img + (size_t)(rr / TC_ROWS) * TC_A_FLOATS, rr % TC_ROWS, k, TC_ROWS, v);
     }
 }
-// U12 (panel rows, columns k0+NB..) -> one image per 128-column block; columns past n are zero.
-__device__ void emit_b_image(const c64* A, int64_t lda, int n, int k0, float* img) {
+// U12 (panel rows, columns k0+NB..) -> one image per 128-column block (the CTA's own blocks, whose
+// U12 it has just formed); columns past n are zero.
+__device__ void emit_b_image(const c64* A, int64_t lda, int n, int k0, float* img, const Cluster& cl) {
+    static_assert(TC_COLS == (uint32_t)DTile<float>::TN, "a CTA's U12 blocks are its image blocks");
     const int c_begin = k0 + NB, m = n - c_begin;
-    const int cols_pad = (m + TC_COLS - 1) / TC_COLS * TC_COLS;
-    for (int idx = threadIdx.x; idx < cols_pad * (NB / 8); idx += NT) {
-        const int k = idx % (NB / 8) * 8, cc = idx / (NB / 8);
+    const int nblk = (m + TC_COLS - 1) / TC_COLS, own = (nblk - cl.rank + cl.size - 1) / cl.size;
+    for (int idx = threadIdx.x; idx < own * (int)TC_COLS * (NB / 8); idx += NT) {
+        const int k = idx % (NB / 8) * 8, q = idx / (NB / 8);
+        const int cc = (cl.rank + q / TC_COLS * cl.size) * TC_COLS + q % TC_COLS;
         c64 v[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e)
@@ -735,8 +788,8 @@ __device__ void trailing_update_tc(c64* A, int64_t lda, int n, int k0, const flo
         mbar_arrive(&ts.bar[2]);  // release: the producer reads the parameters after its wait
     }
     c64 v[32];
-    for (int g = 0; g < steps && !failed(ts); ++g) {
-        const int b = g & 1;
+    for (int g = ts.rank, i = 0; g < steps && !failed(ts); g += ts.size, ++i) {
+        const int b = i & 1;
         const int i0 = r_begin + (g / ncb) * TC_ROWS, c0 = r_begin + (g % ncb) * TC_COLS;
         const uint32_t tb = ts.tmem + b * 256;
         tc_load_c(A, lda, n, i0, c0, 0, v);
@@ -786,11 +839,14 @@ __device__ void tc_producer(unsigned char* smem_raw, TcShared& ts) {
         const float* imgB = *(const float* volatile*)&ts.imgB;
         const int r_begin = k0 + NB, m = n - r_begin;
         const int ncb = (m + TC_COLS - 1) / TC_COLS, steps = (m + TC_ROWS - 1) / TC_ROWS * ncb;
-        for (int g = 0; g < steps; ++g) {
-            const int rt = g / ncb, t = g % ncb, b = g & 1;
-            if (g > 0) wait(&ts.bar[5 + ((g - 1) & 1)], pm[(g - 1) & 1]);  // the operand buffers are free
+        const int mine = steps > ts.rank ? (steps - ts.rank + ts.size - 1) / ts.size : 0;
+        for (int i = 0, prev_rt = -1; i < mine; ++i) {
+            const int g = ts.rank + i * ts.size, rt = g / ncb, t = g % ncb, b = i & 1;
+            const bool new_a = rt != prev_rt;  // L21 tile to load
+            prev_rt = rt;
+            if (i > 0) wait(&ts.bar[5 + ((i - 1) & 1)], pm[(i - 1) & 1]);  // the operand buffers are free
             if (leader && !failed(ts)) {
-                if (t == 0) {
+                if (new_a) {
                     mbar_expect_tx(&ts.bar[0], TC_A_BYTES);
                     for (int c = 0; c < 6; ++c)
                         bulk_g2s(base + c * (TC_A_BYTES / 6), imgA + (size_t)rt * TC_A_FLOATS + c * (TC_A_FLOATS / 6),
@@ -800,13 +856,16 @@ __device__ void tc_producer(unsigned char* smem_raw, TcShared& ts) {
                 const float* src = imgB + (size_t)t * TC_B_FLOATS;
                 for (int c = 0; c < 6; ++c)
                     bulk_g2s(sB + c * (TC_B_BYTES / 6), src + c * (TC_B_FLOATS / 6), TC_B_BYTES / 6, &ts.bar[1]);
-                if (t + 1 < ncb) prefetch_l2(src + TC_B_FLOATS, TC_B_BYTES);
-                else if ((rt + 1) * TC_ROWS < m) prefetch_l2(imgA + (size_t)(rt + 1) * TC_A_FLOATS, TC_A_BYTES);
+                if (i + 1 < mine) {
+                    const int gn = g + ts.size;
+                    prefetch_l2(imgB + (size_t)(gn % ncb) * TC_B_FLOATS, TC_B_BYTES);
+                    if (gn / ncb != rt) prefetch_l2(imgA + (size_t)(gn / ncb) * TC_A_FLOATS, TC_A_BYTES);
+                }
             }
             __syncwarp();
-            if (t == 0) wait(&ts.bar[0], pa);
+            if (new_a) wait(&ts.bar[0], pa);
             wait(&ts.bar[1], pb);
-            if (g >= 2) wait(&ts.bar[3 + b], pe[b]);  // the workers have read accumulator pair b
+            if (i >= 2) wait(&ts.bar[3 + b], pe[b]);  // the workers have read accumulator pair b
             tc_fence_after();
             if (leader) {
                 if (!failed(ts)) tc_issue(adesc, bdesc, ts.tmem + b * 256);
@@ -815,15 +874,17 @@ __device__ void tc_producer(unsigned char* smem_raw, TcShared& ts) {
             __syncwarp();
         }
         // consume the completions not waited for above, so every barrier's phase stays in step
-        if (steps > 0) wait(&ts.bar[5 + ((steps - 1) & 1)], pm[(steps - 1) & 1]);
-        if (steps > 1) wait(&ts.bar[3 + ((steps - 2) & 1)], pe[(steps - 2) & 1]);
-        if (steps > 0) wait(&ts.bar[3 + ((steps - 1) & 1)], pe[(steps - 1) & 1]);
+        if (mine > 0) wait(&ts.bar[5 + ((mine - 1) & 1)], pm[(mine - 1) & 1]);
+        if (mine > 1) wait(&ts.bar[3 + ((mine - 2) & 1)], pe[(mine - 2) & 1]);
+        if (mine > 0) wait(&ts.bar[3 + ((mine - 1) & 1)], pe[(mine - 1) & 1]);
     }
 }
 
+// The panel is CTA 0's; U12's column blocks, the images and the update's steps are dealt out over the
+// cluster.  sh.info is the same in every CTA after the barrier that follows a panel.
 template <typename R>
 __device__ void factor_one(const DenseJob<R>& J, cplx<R>* sm, DShared& sh, float* img, size_t img_b, TcShared* ts,
-                           TcPhase* ph) {
+                           TcPhase* ph, Cluster& cl) {
     const int n = J.n;
     const int64_t lda = J.lda;
     cplx<R>* A = J.a;
@@ -831,53 +892,70 @@ __device__ void factor_one(const DenseJob<R>& J, cplx<R>* sm, DShared& sh, float
     for (int p = 0, k0 = 0; k0 < n; ++p, k0 += NB) {
         const int nbk = min(NB, n - k0), m = n - k0;
         cplx<R>* Pg = A + k0 + (int64_t)k0 * lda;
-        if (m <= cap_rows) {
-            for (int idx = threadIdx.x; idx < m * nbk; idx += NT) {
-                const int r = idx % m, c = idx / m;
-                sm[r + c * m] = Pg[r + (int64_t)c * lda];
-            }
-            wsync();
-            panel_factor(sm, (int64_t)m, m, nbk, k0, sh);
-            for (int idx = threadIdx.x; idx < m * nbk; idx += NT) {
-                const int r = idx % m, c = idx / m;
-                Pg[r + (int64_t)c * lda] = sm[r + c * m];
-            }
-            wsync();
-        } else {
-            int lw = kLeafMax;
-            while (lw > 2 && (size_t)m * lw * sizeof(cplx<R>) > factor_smem<R>()) lw /= 2;
-            // leaves of fewer than 4 columns would cross L2 as often as the columns themselves
-            if (lw >= 4) panel_factor_tall(Pg, lda, m, nbk, lw, k0, sm, sh);
-            else panel_factor(Pg, lda, m, nbk, k0, sh);
-        }
-        if ((int)threadIdx.x < nbk) J.ipiv[k0 + threadIdx.x] = k0 + sh.piv[threadIdx.x];
-        compose_swaps(nbk, sh.piv, sh);
         int32_t* sw = J.swaps + (int64_t)p * kDenseSwapInts;
-        if (threadIdx.x == 0) sw[0] = sh.cnt;
-        for (int i = threadIdx.x; i < 2 * NB; i += NT) {
-            sw[1 + i] = i < sh.cnt ? sh.rows[i] : 0;
-            sw[1 + 2 * NB + i] = i < sh.cnt ? sh.src[i] : 0;
+        if (cl.rank == 0) {
+            if (m <= cap_rows) {
+                for (int idx = threadIdx.x; idx < m * nbk; idx += NT) {
+                    const int r = idx % m, c = idx / m;
+                    sm[r + c * m] = Pg[r + (int64_t)c * lda];
+                }
+                wsync();
+                panel_factor(sm, (int64_t)m, m, nbk, k0, sh);
+                for (int idx = threadIdx.x; idx < m * nbk; idx += NT) {
+                    const int r = idx % m, c = idx / m;
+                    Pg[r + (int64_t)c * lda] = sm[r + c * m];
+                }
+                wsync();
+            } else {
+                int lw = kLeafMax;
+                while (lw > 2 && (size_t)m * lw * sizeof(cplx<R>) > factor_smem<R>()) lw /= 2;
+                // leaves of fewer than 4 columns would cross L2 as often as the columns themselves
+                if (lw >= 4) panel_factor_tall(Pg, lda, m, nbk, lw, k0, sm, sh);
+                else panel_factor(Pg, lda, m, nbk, k0, sh);
+            }
+            if ((int)threadIdx.x < nbk) J.ipiv[k0 + threadIdx.x] = k0 + sh.piv[threadIdx.x];
+            compose_swaps(nbk, sh.piv, sh);
+            if (threadIdx.x == 0) sw[0] = sh.cnt;
+            for (int i = threadIdx.x; i < 2 * NB; i += NT) {
+                sw[1 + i] = i < sh.cnt ? sh.rows[i] : 0;
+                sw[1 + 2 * NB + i] = i < sh.cnt ? sh.src[i] : 0;
+            }
+            if ((int)threadIdx.x < cl.size && threadIdx.x > 0)
+                *cg::this_cluster().map_shared_rank(&sh.info, threadIdx.x) = sh.info;
         }
-        diag_inverses(Pg, lda, nbk, sm, J.inv + (int64_t)p * 2 * NB * NB);
+        if (!csync(cl, sh)) { sh.info = -1; break; }
+        if (cl.rank != 0) {
+            if (threadIdx.x == 0) sh.cnt = __ldcg(sw);
+            for (int i = threadIdx.x; i < 2 * NB; i += NT) {
+                sh.rows[i] = __ldcg(sw + 1 + i);
+                sh.src[i] = __ldcg(sw + 1 + 2 * NB + i);
+            }
+            wsync();
+        }
+        diag_inverses(Pg, lda, nbk, sm, J.inv + (int64_t)p * 2 * NB * NB, cl.rank == 0);
         if (k0 + nbk < n) {
-            trailing_rows(A, lda, n, k0, sm, sh);
+            trailing_rows(A, lda, n, k0, sm, sh, cl);
             if constexpr (sizeof(R) == 4) {
-                emit_a_image(A, lda, n, k0, img);
-                emit_b_image(A, lda, n, k0, img + img_b);
+                emit_a_image(A, lda, n, k0, img, cl);
+                emit_b_image(A, lda, n, k0, img + img_b, cl);
                 // the images (global) and the shared buffers were last touched through the generic
                 // proxy; the bulk copies and MMAs that follow go through the async proxy
                 asm volatile("fence.proxy.async.global;" ::: "memory");
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                wsync();
+                if (!csync(cl, sh)) { sh.info = -1; break; }
+                asm volatile("fence.proxy.async.global;" ::: "memory");
                 trailing_update_tc(A, lda, n, k0, img, img + img_b, *ts, *ph);
                 if (ts->stop) {  // uniform: written by thread 0 between two worker barriers
-                    if (threadIdx.x == 0) sh.info = -1;
+                    sh.info = -1;
+                    cl.fail = true;
                     break;
                 }
             } else {
-                trailing_update(A, lda, n, k0, sm);
+                if (!csync(cl, sh)) { sh.info = -1; break; }
+                trailing_update(A, lda, n, k0, sm, cl);
             }
         }
+        if (!csync(cl, sh)) { sh.info = -1; break; }
     }
 }
 
@@ -897,16 +975,16 @@ constexpr size_t solve_smem() {
 }
 
 // x[r, l] -= sum_k Ablk[r + k lda] y[k * LP + l]  for r in [r0, r1), l < lg
-template <typename R>
-__device__ void solve_update(const cplx<R>* __restrict__ Ablk, int64_t lda, int r0, int r1, int nbk,
-                             const cplx<R>* y, int LP, int lg, cplx<R>* __restrict__ x, int64_t ldx) {
-    constexpr int LC = SolveChunk<R>::LC;
+template <typename R, int LC>
+__device__ void solve_update(const cplx<R>* Ablk, int64_t lda, int r0, int r1, int nbk,
+                             const cplx<R>* y, int LP, int lg, cplx<R>* x, int64_t ldx) {
     for (int l0 = 0; l0 < lg; l0 += LC) {
         for (int r = r0 + (int)threadIdx.x; r < r1; r += NT) {
             cplx<R> acc[LC];
 #pragma unroll
             for (int l = 0; l < LC; ++l) acc[l] = (l0 + l < lg) ? x[r + (int64_t)(l0 + l) * ldx] : czero<R>();
-#pragma unroll 8
+            // the factor's entries of 32 columns in flight: the pass is bound by the latency of L2
+#pragma unroll 32
             for (int k = 0; k < nbk; ++k) {
                 const cplx<R> a = Ablk[r + (int64_t)k * lda];
 #pragma unroll
@@ -919,10 +997,11 @@ __device__ void solve_update(const cplx<R>* __restrict__ Ablk, int64_t lda, int 
     }
 }
 
-// x <- A^{-1} x for one factored point (all J.L columns), by the NT worker threads.
+// x <- A^{-1} x for one factored point (columns l_lo .. l_hi - 1), by the NT worker threads.
 // smem: solve_smem<R>() bytes; rows/src/cnt: 2 NB + 2 NB + 1 ints of shared scratch.
 template <typename R>
-__device__ void solve_one(const DenseJob<R>& J, unsigned char* smem, int* s_rows, int* s_src, int* s_cnt) {
+__device__ void solve_one(const DenseJob<R>& J, int l_lo, int l_hi, unsigned char* smem, int* s_rows, int* s_src,
+                          int* s_cnt) {
     constexpr int LC = SolveChunk<R>::LC;
     cplx<R>* sinv = reinterpret_cast<cplx<R>*>(smem);  // (r, c) at r * NBP + c
     cplx<R>* g = sinv + NB * NBP;                      // [2 NB][LG]
@@ -930,8 +1009,12 @@ __device__ void solve_one(const DenseJob<R>& J, unsigned char* smem, int* s_rows
     const int n = J.n;
     const int np = (int)dense_panels(n);
     const int64_t lda = J.lda;
-    for (int l_begin = 0; l_begin < J.L; l_begin += LG) {
-        const int lg = min(LG, J.L - l_begin);
+    auto update = [&](const cplx<R>* Ablk, int r0, int r1, int nbk, const cplx<R>* y, int LP, int lg, cplx<R>* x) {
+        if (lg <= 2) solve_update<R, 2>(Ablk, lda, r0, r1, nbk, y, LP, lg, x, n);
+        else solve_update<R, LC>(Ablk, lda, r0, r1, nbk, y, LP, lg, x, n);
+    };
+    for (int l_begin = l_lo; l_begin < l_hi; l_begin += LG) {
+        const int lg = min(LG, l_hi - l_begin);
         const int LP = (lg + LC - 1) / LC * LC;
         cplx<R>* x = J.x + (int64_t)l_begin * n;
         for (int idx = threadIdx.x; idx < NB * LP; idx += NT) y[idx] = czero<R>();
@@ -969,7 +1052,7 @@ __device__ void solve_one(const DenseJob<R>& J, unsigned char* smem, int* s_rows
                 x[k0 + t + (int64_t)l * n] = acc;
             }
             wsync();
-            if (k0 + nbk < n) solve_update(J.a + (int64_t)k0 * lda, lda, k0 + nbk, n, nbk, y, LP, lg, x, n);
+            if (k0 + nbk < n) update(J.a + (int64_t)k0 * lda, k0 + nbk, n, nbk, y, LP, lg, x);
             wsync();
         }
         for (int p = np - 1; p >= 0; --p) {  // backward
@@ -992,7 +1075,7 @@ __device__ void solve_one(const DenseJob<R>& J, unsigned char* smem, int* s_rows
                 x[k0 + t + (int64_t)l * n] = acc;
             }
             wsync();
-            if (k0 > 0) solve_update(J.a + (int64_t)k0 * lda, lda, 0, k0, nbk, y, LP, lg, x, n);
+            if (k0 > 0) update(J.a + (int64_t)k0 * lda, 0, k0, nbk, y, LP, lg, x);
             wsync();
         }
     }
@@ -1006,6 +1089,8 @@ __device__ void solve_one(const DenseJob<R>& J, unsigned char* smem, int* s_rows
 //   and refinement X += (LU)^{-1} r while the stopping rule of the band path asks for it.
 // ------------------------------------------------------------------------------------------
 constexpr int kMaxL = 256;
+
+constexpr int kMaxCluster = 8;
 
 struct SampleShared {
     double rn2[kMaxL], xn2[kMaxL];
@@ -1022,7 +1107,8 @@ struct Slot {
     cplx<R>* inv;
     int32_t* swaps;
     double* colsum;
-    c128* tv;  // T(z_j) on the CSR pattern
+    c128* tv;      // T(z_j) on the CSR pattern
+    double* part;  // [kMaxCluster][2][L] the CTAs' shares of the residual's sums
 };
 
 __host__ __device__ inline size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -1032,11 +1118,12 @@ __host__ __device__ inline size_t slot_bytes(int n_max, int L_max, int64_t nnz_m
     const size_t np = (size_t)dense_panels(n_max);
     return align256((size_t)n_max * n_max * sizeof(cplx<R>)) + align256((size_t)n_max * L_max * sizeof(cplx<R>)) +
            align256((size_t)n_max * 4) + align256(np * 2 * NB * NB * sizeof(cplx<R>)) +
-           align256(np * kDenseSwapInts * 4) + align256((size_t)n_max * 8) + align256((size_t)nnz_max * sizeof(c128));
+           align256(np * kDenseSwapInts * 4) + align256((size_t)n_max * 8) + align256((size_t)nnz_max * sizeof(c128)) +
+           align256((size_t)kMaxCluster * 2 * L_max * sizeof(double));
 }
 
 template <typename R>
-__device__ Slot<R> slot_at(unsigned char* base, int n_max, int L_max) {
+__device__ Slot<R> slot_at(unsigned char* base, int n_max, int L_max, int64_t nnz_max) {
     const size_t np = (size_t)dense_panels(n_max);
     Slot<R> t;
     unsigned char* p = base;
@@ -1053,6 +1140,8 @@ __device__ Slot<R> slot_at(unsigned char* base, int n_max, int L_max) {
     t.colsum = reinterpret_cast<double*>(p);
     p += align256((size_t)n_max * 8);
     t.tv = reinterpret_cast<c128*>(p);
+    p += align256((size_t)nnz_max * sizeof(c128));
+    t.part = reinterpret_cast<double*>(p);
     return t;
 }
 
@@ -1068,11 +1157,12 @@ __device__ double worker_max(double v, SampleShared& ss) {
 }
 
 // r = U - T X (FP64, T's CSR values tv); x = r in precision R; per-column ||r||^2 and ||X||^2 into
-// ss.rn2 / ss.xn2.  A warp takes a row: lane = (column of a group of 8, one of 4 entries), so that no
+// ss.rn2 / ss.xn2 (this CTA's rows only).  A warp takes a row: lane = (column of a group of 8, one of 4 entries), so that no
 // lane idles; the FP64 rate bounds it (two multiply-adds a clock: 1 ms for 132000 entries and 8
 // columns, where a thread a row and T formed anew from its terms took 2.7 ms).
 template <typename R>
-__device__ void residual_one(const DenseNep& E, const c128* X, const c128* tv, cplx<R>* x, SampleShared& ss) {
+__device__ void residual_one(const DenseNep& E, const c128* X, const c128* tv, cplx<R>* x, SampleShared& ss,
+                             const Cluster& cl) {
     const int n = E.n, L = E.L, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane >> 3;
     for (int l = threadIdx.x; l < L; l += NT) ss.rn2[l] = ss.xn2[l] = 0.0;
     wsync();
@@ -1081,7 +1171,7 @@ __device__ void residual_one(const DenseNep& E, const c128* X, const c128* tv, c
         const bool on = l < L;
         const c128* Xl = X + (int64_t)(on ? l : l0) * n;
         double pr = 0.0, px = 0.0;
-        for (int r = warp; r < n; r += NW) {
+        for (int r = cl.rank * NW + warp; r < n; r += cl.size * NW) {
             const int64_t end = E.rowptr[r + 1];
             c128 acc = czero<double>();
 #pragma unroll 4
@@ -1108,18 +1198,28 @@ __device__ void residual_one(const DenseNep& E, const c128* X, const c128* tv, c
 
 template <typename R>
 __device__ void sample_one(const DenseNep& E, int j, const Slot<R>& sl, cplx<R>* sm, DShared& sh, SampleShared& ss,
-                           float* img, size_t img_b, TcShared* ts, TcPhase* ph, const DenseSampleCfg& cfg) {
+                           float* img, size_t img_b, TcShared* ts, TcPhase* ph, const DenseSampleCfg& cfg, Cluster& cl) {
     const int n = E.n, L = E.L, J = E.J;
     const int64_t nnz = E.nnz, nl = (int64_t)n * L;
+    const int gtid = cl.rank * NT + threadIdx.x, gstep = cl.size * NT;
+    const int l_lo = L * cl.rank / cl.size, l_hi = L * (cl.rank + 1) / cl.size;  // this CTA's columns
+    const int64_t x_lo = (int64_t)n * l_lo, x_hi = (int64_t)n * l_hi;
     cplx<R>* A = sl.a;
+    auto failed_wait = [&]() {  // a wait in the cluster gave up: every CTA that notices reports the point
+        if (threadIdx.x == 0) {
+            E.status[j] = -1;
+            E.sweeps[j] = 0;
+        }
+        wsync();
+    };
     // assemble T(z_j) (precision R) and its FP64 column sums
     {
         const int64_t nn = (int64_t)n * n;
-        for (int64_t idx = threadIdx.x; idx < nn; idx += NT) A[idx] = czero<R>();
-        for (int c = threadIdx.x; c < n; c += NT) sl.colsum[c] = 0.0;
-        wsync();
+        for (int64_t idx = gtid; idx < nn; idx += gstep) A[idx] = czero<R>();
+        for (int c = gtid; c < n; c += gstep) sl.colsum[c] = 0.0;
+        if (!csync(cl, sh)) return failed_wait();
         const c128* f = E.F + (int64_t)j * J;
-        for (int64_t k = threadIdx.x; k < nnz; k += NT) {
+        for (int64_t k = gtid; k < nnz; k += gstep) {
             c128 t = czero<double>();
             for (int i = 0; i < J; ++i) cfma(t, f[i], E.vals[(int64_t)i * nnz + k]);
             sl.tv[k] = t;
@@ -1127,9 +1227,10 @@ __device__ void sample_one(const DenseNep& E, int j, const Slot<R>& sl, cplx<R>*
             A[E.rowidx[k] + (int64_t)c * n] = ccast<R>(t);
             atomicAdd(&sl.colsum[c], sqrt(cnorm2(t)));
         }
-        wsync();
+        if (threadIdx.x == 0) sh.info = 0;
+        if (!csync(cl, sh)) return failed_wait();
         double m = 0.0;
-        for (int c = threadIdx.x; c < n; c += NT) m = fmax(m, sl.colsum[c]);
+        for (int c = threadIdx.x; c < n; c += NT) m = fmax(m, __ldcg(sl.colsum + c));
         m = worker_max(m, ss);
         if (threadIdx.x == 0) ss.normT = m;
     }
@@ -1142,13 +1243,12 @@ __device__ void sample_one(const DenseNep& E, int j, const Slot<R>& sl, cplx<R>*
     Jb.inv = sl.inv;
     Jb.swaps = sl.swaps;
     Jb.x = sl.x;
-    if (threadIdx.x == 0) sh.info = 0;
-    wsync();
-    factor_one(Jb, sm, sh, img, img_b, ts, ph);
+    factor_one(Jb, sm, sh, img, img_b, ts, ph, cl);
     wsync();
     const int info = sh.info;
+    if (info < 0) return failed_wait();
     if (info != 0) {
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == 0 && cl.rank == 0) {
             E.status[j] = info;
             E.sweeps[j] = 0;
         }
@@ -1156,22 +1256,32 @@ __device__ void sample_one(const DenseNep& E, int j, const Slot<R>& sl, cplx<R>*
         return;
     }
     c128* X = E.S + (int64_t)j * nl;
-    for (int64_t idx = threadIdx.x; idx < nl; idx += NT) sl.x[idx] = ccast<R>(E.U[idx]);
+    for (int64_t idx = x_lo + threadIdx.x; idx < x_hi; idx += NT) sl.x[idx] = ccast<R>(E.U[idx]);
     wsync();
     unsigned char* smb = reinterpret_cast<unsigned char*>(sm);
-    solve_one(Jb, smb, sh.rows, sh.src, &sh.cnt);
-    for (int64_t idx = threadIdx.x; idx < nl; idx += NT) X[idx] = ccast<double>(sl.x[idx]);
-    wsync();
+    solve_one(Jb, l_lo, l_hi, smb, sh.rows, sh.src, &sh.cnt);
+    for (int64_t idx = x_lo + threadIdx.x; idx < x_hi; idx += NT) X[idx] = ccast<double>(sl.x[idx]);
     double prev = 0.0;
     int sweeps = 0;
     for (;;) {
-        residual_one(E, X, sl.tv, sl.x, ss);
-        // backward error per column and the decision (one thread decides, all follow)
+        if (!csync(cl, sh)) return failed_wait();  // every column of X is there
+        residual_one(E, X, sl.tv, sl.x, ss, cl);
+        for (int l = threadIdx.x; l < L; l += NT) {
+            sl.part[(2 * cl.rank) * L + l] = ss.rn2[l];
+            sl.part[(2 * cl.rank + 1) * L + l] = ss.xn2[l];
+        }
+        if (!csync(cl, sh)) return failed_wait();
+        // backward error per column and the decision (the same in every CTA: the same sums)
         double mx = 0.0;
         int nonfinite = 0;
         for (int l = threadIdx.x; l < L; l += NT) {
-            const double e = sqrt(ss.rn2[l]) / (ss.normT * sqrt(ss.xn2[l]) + sqrt(E.un2[l]));
-            E.eta[(int64_t)j * L + l] = e;
+            double rn2 = 0.0, xn2 = 0.0;
+            for (int q = 0; q < cl.size; ++q) {
+                rn2 += __ldcg(sl.part + (2 * q) * L + l);
+                xn2 += __ldcg(sl.part + (2 * q + 1) * L + l);
+            }
+            const double e = sqrt(rn2) / (ss.normT * sqrt(xn2) + sqrt(E.un2[l]));
+            if (cl.rank == 0) E.eta[(int64_t)j * L + l] = e;
             if (!isfinite(e)) nonfinite = 1;
             mx = fmax(mx, e);
         }
@@ -1188,26 +1298,23 @@ __device__ void sample_one(const DenseNep& E, int j, const Slot<R>& sl, cplx<R>*
         wsync();
         const int action = ss.action;
         if (action != 1) {
-            if (threadIdx.x == 0) {
+            if (threadIdx.x == 0 && cl.rank == 0) {
                 E.status[j] = action;
                 E.sweeps[j] = sweeps;
             }
             break;
         }
-        solve_one(Jb, smb, sh.rows, sh.src, &sh.cnt);
-        for (int64_t idx = threadIdx.x; idx < nl; idx += NT) X[idx] = X[idx] + ccast<double>(sl.x[idx]);
-        wsync();
+        solve_one(Jb, l_lo, l_hi, smb, sh.rows, sh.src, &sh.cnt);
+        for (int64_t idx = x_lo + threadIdx.x; idx < x_hi; idx += NT) X[idx] = X[idx] + ccast<double>(sl.x[idx]);
         ++sweeps;
     }
     wsync();
 }
 
-// Complex64 launches NT + 32 threads: warps 0..7 work, warp 8 feeds the tensor cores;
-// complex128 launches NT.  CTA b uses slot b and (complex64) image block b.
 template <typename R>
 __global__ void __launch_bounds__(sizeof(R) == 4 ? NT + 32 : NT, 1)
     dense_sample_kernel(const DenseNep* __restrict__ neps, const DenseSampleJob* __restrict__ jobs, int njobs,
-                        int n_max, int L_max, unsigned char* slots, size_t slot_stride, float* img, size_t img_stride,
+                        int n_max, int L_max, int64_t nnz_max, unsigned char* slots, size_t slot_stride, float* img, size_t img_stride,
                         size_t img_b, int32_t* __restrict__ next, DenseSampleCfg cfg) {
     extern __shared__ __align__(16) unsigned char dense_smem[];
     cplx<R>* sm = reinterpret_cast<cplx<R>*>(dense_smem);
@@ -1216,6 +1323,17 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? NT + 32 : NT, 1)
     __shared__ __align__(8) TcShared ts;
     TcPhase ph;
     constexpr bool tc = sizeof(R) == 4;
+    cg::cluster_group cluster = cg::this_cluster();
+    Cluster cl;
+    cl.rank = (int)cluster.block_rank();
+    cl.size = (int)cluster.num_blocks();
+    if (threadIdx.x == 0) {
+        mbar_init(&sh.cbar, (uint32_t)cl.size);
+        ts.rank = cl.rank;
+        ts.size = cl.size;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    cluster.sync();  // the barriers exist before anyone arrives on them
     if (tc) {
         if (threadIdx.x == 0) {
             for (int i = 0; i < 7; ++i) mbar_init(&ts.bar[i], i == 3 || i == 4 ? NT / 32 : 1);
@@ -1235,15 +1353,20 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? NT + 32 : NT, 1)
         if (threadIdx.x >= NT) tc_producer(dense_smem, ts);
     }
     if (threadIdx.x < NT) {
-        const Slot<R> sl = slot_at<R>(slots + (size_t)blockIdx.x * slot_stride, n_max, L_max);
-        float* my_img = img ? img + (size_t)blockIdx.x * img_stride : nullptr;
+        const size_t slot = blockIdx.x / cl.size;
+        const Slot<R> sl = slot_at<R>(slots + slot * slot_stride, n_max, L_max, nnz_max);
+        float* my_img = img ? img + slot * img_stride : nullptr;
         for (;;) {
-            if (threadIdx.x == 0) sh.job = (tc && ts.stop) ? njobs : atomicAdd(next, 1);  // no new job after a timeout
-            wsync();
+            // CTA 0 takes the next job for the cluster (none after a timeout)
+            if (threadIdx.x == 0 && cl.rank == 0) {
+                const int jb = (tc && ts.stop) || cl.fail ? njobs : atomicAdd(next, 1);
+                for (int q = 0; q < cl.size; ++q) *cluster.map_shared_rank(&sh.job, q) = jb;
+            }
+            if (!csync(cl, sh)) break;
             const int jb = sh.job;
             if (jb >= njobs) break;
             const DenseSampleJob job = jobs[jb];
-            sample_one<R>(neps[job.nep], job.j, sl, sm, sh, ss, my_img, img_b, &ts, &ph, cfg);
+            sample_one<R>(neps[job.nep], job.j, sl, sm, sh, ss, my_img, img_b, &ts, &ph, cfg, cl);
         }
         if (tc && threadIdx.x == 0) {
             ts.cmd = 2;
@@ -1258,6 +1381,7 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? NT + 32 : NT, 1)
             asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(ts.tmem), "r"(TC_TMEM_COLS)
                          : "memory");
     }
+    cluster.sync();  // no CTA leaves while another may still arrive on its barrier
 }
 
 // Opt a kernel into its dynamic shared memory.  The attribute is per function and process-wide,
@@ -1290,7 +1414,32 @@ int sm_count() {
 
 }  // namespace
 
-int dense_sample_grid(int njobs) { return std::max(1, std::min(njobs, sm_count())); }
+// Cluster size and count for jobs of orders n (descending): the size whose greedy schedule of the
+// jobs ends first.  A point's time is taken as n^2 (s + (1 - s) / size): CTA 0's panels are serial, the
+// rest is shared; no more CTAs than the largest matrix has panels.
+void dense_plan(const std::vector<int>& n, int* size, int* count) {
+    const int nsm = sm_count();
+    double best = 0.0;
+    *size = 1;
+    *count = 1;
+    for (int c = 1; c <= kMaxCluster && (c == 1 || c * NB <= n.front()); c *= 2) {
+        const int m = std::max(1, std::min((int)n.size(), nsm / c));
+        std::priority_queue<double, std::vector<double>, std::greater<double>> busy;
+        for (int i = 0; i < m; ++i) busy.push(0.0);
+        double end = 0.0;
+        for (int x : n) {
+            const double t = busy.top() + (double)x * x * (kDenseSerial + (1.0 - kDenseSerial) / c);
+            busy.pop();
+            busy.push(t);
+            end = std::max(end, t);
+        }
+        if (c == 1 || end < 0.95 * best) {
+            best = end;
+            *size = c;
+            *count = m;
+        }
+    }
+}
 
 template <typename R>
 size_t dense_slot_bytes(int n_max, int L_max, int64_t nnz_max) {
@@ -1306,7 +1455,7 @@ size_t dense_image_bytes(int n_max) {
 
 template <typename R>
 int launch_dense_sample(const DenseNep* d_neps, const DenseSampleJob* d_jobs, int njobs, int n_max, int L_max,
-                        int64_t nnz_max, int grid, void* d_slots, void* d_img, int32_t* d_next, DenseSampleCfg cfg, cudaStream_t s) {
+                        int64_t nnz_max, int clusters, int cluster_size, void* d_slots, void* d_img, int32_t* d_next, DenseSampleCfg cfg, cudaStream_t s) {
     if (njobs <= 0) return RSRR_OK;
     if (L_max > kMaxL) return set_error(RSRR_EINVAL, "dense sampling: L above 256");
     if (sizeof(R) == 4 && !d_img) return set_error(RSRR_EINVAL, "dense sampling: operand images missing");
@@ -1316,13 +1465,21 @@ int launch_dense_sample(const DenseNep* d_neps, const DenseSampleJob* d_jobs, in
     const int threads = sizeof(R) == 4 ? NT + 32 : NT;
     const size_t img_stride = dense_image_bytes<R>(n_max) / 4;
     const size_t img_b = sizeof(R) == 4 ? (size_t)((n_max + TC_ROWS - 1) / TC_ROWS) * TC_A_FLOATS : 0;
-    {
-        dense_sample_kernel<R><<<grid, threads, sm, s>>>(d_neps, d_jobs, njobs, n_max, L_max,
-                                                         static_cast<unsigned char*>(d_slots),
-                                                         dense_slot_bytes<R>(n_max, L_max, nnz_max), static_cast<float*>(d_img),
-                                                         img_stride, img_b, d_next, cfg);
-        note_launch();
-    }
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)(clusters * cluster_size));
+    lc.blockDim = dim3((unsigned)threads);
+    lc.dynamicSmemBytes = sm;
+    lc.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cluster_size;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    RSRR_CUDA(cudaLaunchKernelEx(&lc, dense_sample_kernel<R>, d_neps, d_jobs, njobs, n_max, L_max, nnz_max,
+                                 static_cast<unsigned char*>(d_slots), dense_slot_bytes<R>(n_max, L_max, nnz_max),
+                                 static_cast<float*>(d_img), img_stride, img_b, d_next, cfg));
+    note_launch();
     RSRR_CUDA(cudaGetLastError());
     return RSRR_OK;
 }
@@ -1331,9 +1488,9 @@ template size_t dense_slot_bytes<float>(int, int, int64_t);
 template size_t dense_slot_bytes<double>(int, int, int64_t);
 template size_t dense_image_bytes<float>(int);
 template size_t dense_image_bytes<double>(int);
-template int launch_dense_sample<float>(const DenseNep*, const DenseSampleJob*, int, int, int, int64_t, int, void*, void*,
+template int launch_dense_sample<float>(const DenseNep*, const DenseSampleJob*, int, int, int, int64_t, int, int, void*, void*,
                                         int32_t*, DenseSampleCfg, cudaStream_t);
-template int launch_dense_sample<double>(const DenseNep*, const DenseSampleJob*, int, int, int, int64_t, int, void*, void*,
+template int launch_dense_sample<double>(const DenseNep*, const DenseSampleJob*, int, int, int, int64_t, int, int, void*, void*,
                                          int32_t*, DenseSampleCfg, cudaStream_t);
 
 }  // namespace rsrr

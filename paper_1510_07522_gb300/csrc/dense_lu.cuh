@@ -21,6 +21,8 @@
 //          leading dimension kDenseNB), so each block solve is one small product.
 #pragma once
 
+#include <vector>
+
 #include "common.cuh"
 
 namespace rsrr {
@@ -31,7 +33,7 @@ constexpr int kDenseSwapInts = 1 + 4 * kDenseNB;
 
 __host__ __device__ inline int64_t dense_panels(int64_t n) { return (n + kDenseNB - 1) / kDenseNB; }
 
-// The factor and solve of one point (one CTA's slot).
+// The factor and solve of one point (one cluster's slot).
 template <typename R>
 struct DenseJob {
     cplx<R>* a;              // [n][lda] column-major
@@ -45,7 +47,7 @@ struct DenseJob {
 };
 
 // ---- fused dense sampling: one persistent launch for all points of a set of NEPs --------------
-// Each CTA takes (NEP, point) jobs largest n first and, in a memory slot of its own, assembles
+// Each cluster takes (NEP, point) jobs largest n first and, in a memory slot of its own, assembles
 // T(z_j), factors it, solves T X = U, computes the FP64 residual and backward error and refines
 // until the stopping rule of the band path holds, writing X into the NEP's S_hat.
 struct DenseNep {
@@ -73,17 +75,17 @@ struct DenseSampleCfg {
     int32_t max_refine;
 };
 
-// Device bytes of one CTA's slot for n <= n_max, L <= L_max, nnz <= nnz_max.
+// Device bytes of one cluster's slot for n <= n_max, L <= L_max, nnz <= nnz_max.
 template <typename R>
 size_t dense_slot_bytes(int n_max, int L_max, int64_t nnz_max);
-// Largest CTA count worth launching for njobs jobs (one per SM at most).
-int dense_sample_grid(int njobs);
-// Device bytes of one CTA's tensor-core operand images (complex64; 0 for complex128).
+// Cluster size (CTAs per point) and number of clusters for jobs of orders n (descending).
+void dense_plan(const std::vector<int>& n, int* size, int* count);
+// Device bytes of one cluster's tensor-core operand images (complex64; 0 for complex128).
 template <typename R>
 size_t dense_image_bytes(int n_max);
-// d_slots: grid * dense_slot_bytes; d_img: grid * dense_image_bytes; d_next: one int32.
+// d_slots: clusters * dense_slot_bytes; d_img: clusters * dense_image_bytes; d_next: one int32.
 template <typename R>
 int launch_dense_sample(const DenseNep* d_neps, const DenseSampleJob* d_jobs, int njobs, int n_max, int L_max,
-                        int64_t nnz_max, int grid, void* d_slots, void* d_img, int32_t* d_next, DenseSampleCfg cfg, cudaStream_t s);
+                        int64_t nnz_max, int clusters, int cluster_size, void* d_slots, void* d_img, int32_t* d_next, DenseSampleCfg cfg, cudaStream_t s);
 
 }  // namespace rsrr

@@ -524,12 +524,17 @@ int sample_dense_set(const std::vector<rsrr_nep>& hs, const std::vector<c128*>& 
     for (int i : order)
         for (int j = 0; j < hs[i]->N; ++j) jobs.push_back(DenseSampleJob{i, j});
     const int njobs = (int)jobs.size();
-    // CTAs: one per SM at most, and no more slots than the free memory holds
+    // clusters of CTAs, one point each at a time: one CTA per SM at most, and no more slots than the free
+    // memory holds
     size_t free_b = 0, total_b = 0;
     RSRR_CUDA(cudaMemGetInfo(&free_b, &total_b));
-    const size_t per_cta = dense_slot_bytes<R>(n_max, L_max, nnz_max) + dense_image_bytes<R>(n_max);
+    const size_t per_slot = dense_slot_bytes<R>(n_max, L_max, nnz_max) + dense_image_bytes<R>(n_max);
     const size_t budget = (size_t)(0.8 * (double)free_b);
-    const int grid = (int)std::min<size_t>((size_t)dense_sample_grid(njobs), budget / per_cta);
+    std::vector<int> job_n(jobs.size());
+    for (size_t i = 0; i < jobs.size(); ++i) job_n[i] = (int)hs[jobs[i].nep]->n;
+    int csize = 1, ccount = 1;
+    dense_plan(job_n, &csize, &ccount);
+    const int grid = (int)std::min<size_t>((size_t)ccount, budget / per_slot);
     if (grid < 1) return set_error(RSRR_ENOMEM, "one dense sampling slot does not fit in device memory");
 
     std::vector<DenseNep> neps(nh);
@@ -584,7 +589,7 @@ int sample_dense_set(const std::vector<rsrr_nep>& hs, const std::vector<c128*>& 
     cfg.max_refine = max_refine;
     EvPair ev;
     ev.start(st);
-    TRYD(launch_dense_sample<R>(d_neps, d_jobs, njobs, n_max, L_max, nnz_max, grid, d_slots, d_img, d_next, cfg, st));
+    TRYD(launch_dense_sample<R>(d_neps, d_jobs, njobs, n_max, L_max, nnz_max, grid, csize, d_slots, d_img, d_next, cfg, st));
     ev.stop(st);
     bool singular = false, timeout = false, nonfinite = false, notconv = false;
     for (int i = 0; i < nh; ++i) {
