@@ -651,10 +651,12 @@ int jacobi_orthogonalize(c128* B, int mb, int k, c128* J, cudaStream_t s, int ma
     std::vector<int> order(k);
     std::vector<uint8_t> hord(ord_bytes);
     int sweep = 0;
-    for (; sweep < max_sweeps; ++sweep) {
+    auto fetch_norms = [&]() {  // queued; the next sweep sorts by them
         column_norms(curB, mb, k, mb, dnrm, s);
-        if (cudaMemcpyAsync(hn.data(), dnrm, (size_t)k * 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess) { rc = set_error(RSRR_ECUDA, "jacobi norms"); break; }
+        return cudaMemcpyAsync(hn.data(), dnrm, (size_t)k * 8, cudaMemcpyDeviceToHost, s) == cudaSuccess;
+    };
+    if (!fetch_norms() || cudaStreamSynchronize(s) != cudaSuccess) rc = set_error(RSRR_ECUDA, "jacobi norms");
+    for (; rc == RSRR_OK && sweep < max_sweeps; ++sweep) {
         for (int i = 0; i < k; ++i) order[i] = i;
         std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return hn[a] > hn[b]; });
         bool sorted = true;
@@ -704,7 +706,7 @@ int jacobi_orthogonalize(c128* B, int mb, int k, c128* J, cudaStream_t s, int ma
         }
         if (e != cudaSuccess) { rc = set_error(RSRR_ECUDA, cudaGetErrorString(e)); break; }
         JacobiCtl hc;
-        if (cudaMemcpyAsync(&hc, dctl, sizeof(hc), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        if (cudaMemcpyAsync(&hc, dctl, sizeof(hc), cudaMemcpyDeviceToHost, s) != cudaSuccess || !fetch_norms() ||
             cudaStreamSynchronize(s) != cudaSuccess) { rc = set_error(RSRR_ECUDA, "jacobi sync"); break; }
         if (hc.err) { rc = set_error(RSRR_ETIMEOUT, "a wait in the Jacobi sweep gave up"); break; }
         // the sweep's work: one complex inner product and two norms for every pair formed (16 real

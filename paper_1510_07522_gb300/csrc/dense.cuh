@@ -34,6 +34,24 @@ int zinv_batch(c128* X, int k, int batch, int32_t* info, cudaStream_t st);
 // the shapes for which zgemm() takes it.  zgemm_path: 0 = by shape, 1 = FP64 CUDA cores only,
 // 2 = tensor cores for every shape (per host thread; for tests and measurements).
 int zgemm_tc(const Zgemm& g, cudaStream_t s);
+// While one is alive (and begin() succeeded), the tensor-core ZGEMMs of this host thread do not wait
+// for their kernel: a bounded wait that gave up is recorded in one device word, which check() reads
+// after synchronising `st`.  The products must all run on `st`.  check() ends the deferral.
+class ZgemmDefer {
+  public:
+    explicit ZgemmDefer(cudaStream_t s) : st(s) {}
+    ~ZgemmDefer();
+    ZgemmDefer(const ZgemmDefer&) = delete;
+    ZgemmDefer& operator=(const ZgemmDefer&) = delete;
+    int begin();
+    int check();
+
+  private:
+    cudaStream_t st;
+    int* word = nullptr;
+    int* outer = nullptr;  // the deferral that was in force before this one
+    bool on = false;
+};
 bool zgemm_tc_fits(const Zgemm& g);
 void zgemm_set_path(int path);
 int zgemm_get_path();

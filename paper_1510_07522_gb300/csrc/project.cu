@@ -382,6 +382,8 @@ int householder_qr(c128* A, int64_t rows, int cols, int64_t lda, HqrWork& w, dou
             g3.A = w.V; g3.lda = rows; g3.B = w.W2; g3.ldb = kPB; g3.C = A + kb + (int64_t)kk * lda; g3.ldc = lda;
             RSRR_TRY(zgemm(g3, st));
         }
+        // without a stop test the panels run on and the barrier's error word is read after the last
+        if (stop_norm < 0.0 && kk < kmax) continue;
         int berr = 0;
         double tn2 = 0.0;
         if (stop_norm >= 0.0) {
@@ -544,6 +546,8 @@ int project_run(rsrr_nep h, double delta) {
     double* colnrm = nullptr;
     int *order_d = nullptr, *cols_d = nullptr;
     int rc = RSRR_OK;
+    ZgemmDefer defer(st);
+    RSRR_TRY(defer.begin());
     auto cleanup = [&]() {
         double zm, zf;
         zgemm_profile_end(&zm, &zf);
@@ -702,7 +706,7 @@ int project_run(rsrr_nep h, double delta) {
             h->d_Q = Ybuf;
             Ybuf = nullptr;
             pc.mark();
-            CUDAC(cudaStreamSynchronize(st));
+            TRYC(defer.check());
             for (int i = 0; i < 4; ++i) h->ms_project_parts[i] = pc.ms(i);
             zgemm_profile_end(&h->ms_zgemm_project, &h->zgemm_flops_project, &h->ms_zgemm_tc_project,
                               &h->zgemm_tc_flops_project);
@@ -724,7 +728,7 @@ int project_run(rsrr_nep h, double delta) {
         Ybuf = nullptr;
         pc.mark();  // projection done
     }
-    CUDAC(cudaStreamSynchronize(st));
+    TRYC(defer.check());
     for (int i = 0; i < 4; ++i) h->ms_project_parts[i] = pc.ms(i);
     zgemm_profile_end(&h->ms_zgemm_project, &h->zgemm_flops_project, &h->ms_zgemm_tc_project,
                       &h->zgemm_tc_flops_project);

@@ -387,6 +387,8 @@ int solve_run(rsrr_nep h, int N_S, int K, double tol_gap, int cap, double* lambd
             jacobi_profile_end(&h->ms_jacobi_solve, &h->jacobi_flops_solve);
         }
     } zpg{h};
+    ZgemmDefer defer(st);
+    RSRR_TRY(defer.begin());
     // J, fns: the reduced NEP's terms (T's own, or Chebyshev polynomials); the final residual
     // uses T itself (h->J, h->fns, the CSR values)
     const int k = h->kS, J = h->red_J;
@@ -764,7 +766,7 @@ int solve_run(rsrr_nep h, int N_S, int K, double tol_gap, int cap, double* lambd
         }
     }
     cudaEventRecord(ev[3], st);
-    CUDAC(cudaStreamSynchronize(st));
+    TRYC(defer.check());
     for (int i = 0; i < 3; ++i) {
         float t = 0.f;
         cudaEventElapsedTime(&t, ev[i], ev[i + 1]);

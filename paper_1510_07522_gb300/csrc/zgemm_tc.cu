@@ -608,6 +608,31 @@ bool zgemm_tc_fits(const Zgemm& g) {
     return work >= 1e8 && g.K >= 16 && std::min(g.M, g.N) > 8;
 }
 
+namespace {
+thread_local int* t_defer = nullptr;  // error word of the deferral in force on this host thread
+}
+
+ZgemmDefer::~ZgemmDefer() {
+    if (on) t_defer = outer;
+    dfree(word, st);
+}
+int ZgemmDefer::begin() {
+    RSRR_TRY(dalloc_n(&word, 1, st));
+    if (cudaMemsetAsync(word, 0, 4, st) != cudaSuccess) return set_error(RSRR_ECUDA, "memset");
+    outer = t_defer;
+    t_defer = word;
+    on = true;
+    return RSRR_OK;
+}
+int ZgemmDefer::check() {
+    if (on) t_defer = outer;
+    on = false;
+    int herr = 0;
+    RSRR_CUDA(cudaMemcpyAsync(&herr, word, 4, cudaMemcpyDeviceToHost, st));
+    RSRR_CUDA(cudaStreamSynchronize(st));
+    return herr ? set_error(RSRR_ETIMEOUT, "tensor-core ZGEMM: a bounded wait gave up") : RSRR_OK;
+}
+
 int zgemm_tc(const Zgemm& g0, cudaStream_t s) {
     Zgemm g = g0;
     // orientation: the 32-column tile side goes to the smaller output side; computing C^T =
@@ -641,20 +666,21 @@ int zgemm_tc(const Zgemm& g0, cudaStream_t s) {
 
     unsigned long long *rmax = nullptr, *cmax = nullptr;
     uint8_t *imgA = nullptr, *imgB = nullptr;
-    int* err = nullptr;
+    int* own_err = nullptr;
     int rc = RSRR_OK;
     auto release = [&]() {
-        for (void* p : {(void*)rmax, (void*)cmax, (void*)imgA, (void*)imgB, (void*)err}) dfree(p, s);
+        for (void* p : {(void*)rmax, (void*)cmax, (void*)imgA, (void*)imgB, (void*)own_err}) dfree(p, s);
     };
     const size_t bytesA = (size_t)batch * MT * nslab * OZ_A_BYTES, bytesB = (size_t)batch * NTt * nslab * OZ_B_BYTES;
     if ((rc = dalloc_n(&rmax, (size_t)batch * M, s)) || (rc = dalloc_n(&cmax, (size_t)batch * N, s)) ||
-        (rc = dalloc_n(&imgA, bytesA, s)) || (rc = dalloc_n(&imgB, bytesB, s)) || (rc = dalloc_n(&err, 1, s))) {
+        (rc = dalloc_n(&imgA, bytesA, s)) || (rc = dalloc_n(&imgB, bytesB, s)) || (!t_defer && (rc = dalloc_n(&own_err, 1, s)))) {
         release();
         return rc;
     }
     cudaMemsetAsync(rmax, 0, (size_t)batch * M * 8, s);
     cudaMemsetAsync(cmax, 0, (size_t)batch * N * 8, s);
-    cudaMemsetAsync(err, 0, 4, s);
+    int* err = t_defer ? t_defer : own_err;
+    if (own_err) cudaMemsetAsync(own_err, 0, 4, s);
     oz_max(A, lda, sA, opA, M, K, batch, rmax, s);
     // columns of op(B) are the rows of op(B)^T
     oz_max(B, ldb, sB, tr(opB), N, K, batch, cmax, s);
@@ -685,7 +711,7 @@ int zgemm_tc(const Zgemm& g0, cudaStream_t s) {
     { oz_gemm_kernel<<<G, OZ_THREADS, OZ_SMEM, s>>>(oa); note_launch(); }
     rc = cudaGetLastError() == cudaSuccess ? RSRR_OK : set_error(RSRR_ECUDA, "tensor-core ZGEMM launch");
     int herr = 0;
-    if (rc == RSRR_OK) {
+    if (rc == RSRR_OK && own_err) {
         cudaMemcpyAsync(&herr, err, 4, cudaMemcpyDeviceToHost, s);
         if (cudaStreamSynchronize(s) != cudaSuccess) rc = set_error(RSRR_ECUDA, "tensor-core ZGEMM");
         else if (herr) rc = set_error(RSRR_ETIMEOUT, "tensor-core ZGEMM: a bounded wait gave up");
