@@ -20,6 +20,7 @@
 //   4. P_i = S^H (A_i S): CSR SpMM, then ZGEMM.
 #include <algorithm>
 #include <cmath>
+#include <functional>
 #include <numeric>
 #include <vector>
 
@@ -339,16 +340,22 @@ struct HqrWork {
 };
 
 int block_norm2_est(const c128* A, int64_t lda, int r0, int r1, int c0, int c1, int iters, c128* x, c128* y,
-                    double* dn, cudaStream_t st, double* est);
+                    double* dn, cudaStream_t st, double* est, double enough = INFINITY);
 
-// stop_norm >= 0: stop after the first panel whose remaining trailing block has 2-norm at most
-// stop_norm, tested by the Frobenius norm (an upper bound) or, once that is within
-// sqrt(min(rows, cols)) of the target, by three times a power-iteration estimate.
-int householder_qr(c128* A, int64_t rows, int cols, int64_t lda, HqrWork& w, double stop_norm, int* kk_out,
+// With a stop rule: stop after the first panel whose remaining trailing block has 2-norm at most
+// the rule's level, tested by the Frobenius norm (an upper bound) or, once that is within
+// sqrt(min(rows, cols)) of the target, by three times a power-iteration estimate.  The level may need
+// the rows of R found so far (`level`, asked for once); `bound` is at least as large and known before.
+struct StopRule {
+    double bound;
+    std::function<int(int kk, double* stop)> level;
+};
+int householder_qr(c128* A, int64_t rows, int cols, int64_t lda, HqrWork& w, const StopRule* rule, int* kk_out,
                    int* npan_out) {
     cudaStream_t st = w.st;
     const int kmax = (int)std::min<int64_t>(rows, cols);
     int kk = 0, npan = 0;
+    double stop_norm = -1.0;
     for (int kb = 0; kb < kmax; kb += kPB) {
         const int bw = std::min(kPB, kmax - kb);
         // rows per CTA: a multiple of 32 (lane = row), the fewest that use every SM.  Fewer than 32
@@ -383,10 +390,10 @@ int householder_qr(c128* A, int64_t rows, int cols, int64_t lda, HqrWork& w, dou
             RSRR_TRY(zgemm(g3, st));
         }
         // without a stop test the panels run on and the barrier's error word is read after the last
-        if (stop_norm < 0.0 && kk < kmax) continue;
+        if (!rule && kk < kmax) continue;
         int berr = 0;
         double tn2 = 0.0;
-        if (stop_norm >= 0.0) {
+        if (rule) {
             RSRR_CUDA(cudaMemsetAsync(w.dnorm, 0, 8, st));
             block_norm2(A, lda, kk, (int)rows, kk, cols, w.dnorm, st);
             RSRR_CUDA(cudaMemcpyAsync(&tn2, w.dnorm, 8, cudaMemcpyDeviceToHost, st));
@@ -395,13 +402,15 @@ int householder_qr(c128* A, int64_t rows, int cols, int64_t lda, HqrWork& w, dou
         RSRR_CUDA(cudaStreamSynchronize(st));
         if (berr) return set_error(RSRR_ETIMEOUT, "grid barrier gave up in the panel kernel");
         if (!std::isfinite(tn2)) return set_error(RSRR_ENONFINITE, "non-finite QR");
-        if (stop_norm >= 0.0 && kk < kmax) {
-            const double fro = sqrt(tn2);
+        if (rule && kk < kmax) {
+            const double fro = sqrt(tn2), dimf = sqrt((double)std::min<int64_t>(rows - kk, cols - kk));
+            if (fro > rule->bound * dimf) continue;
+            if (stop_norm < 0.0) RSRR_TRY(rule->level(kk, &stop_norm));
             if (fro <= stop_norm) break;
-            const double dimf = sqrt((double)std::min<int64_t>(rows - kk, cols - kk));
             if (fro <= stop_norm * dimf) {
                 double est = 0.0;
-                RSRR_TRY(block_norm2_est(A, lda, kk, (int)rows, kk, cols, 12, w.px, w.py, w.dnorm, st, &est));
+                RSRR_TRY(block_norm2_est(A, lda, kk, (int)rows, kk, cols, 12, w.px, w.py, w.dnorm, st, &est,
+                                         stop_norm / 3.0));
                 if (3.0 * est <= stop_norm) break;
             }
         }
@@ -477,9 +486,9 @@ __global__ void seed_vec_kernel(c128* x, int n) {  // fixed pseudo-random start 
 }
 
 // Power-iteration estimate of the 2-norm of the block (a lower bound that converges from
-// below; the caller applies a safety factor).
+// below; the caller applies a safety factor).  It ends early once it is above `enough`.
 int block_norm2_est(const c128* A, int64_t lda, int r0, int r1, int c0, int c1, int iters, c128* x, c128* y,
-                    double* dn, cudaStream_t st, double* est) {
+                    double* dn, cudaStream_t st, double* est, double enough) {
     const int nr = r1 - r0, nc = c1 - c0;
     *est = 0.0;
     if (nr <= 0 || nc <= 0) return RSRR_OK;
@@ -495,7 +504,7 @@ int block_norm2_est(const c128* A, int64_t lda, int r0, int r1, int c0, int c1, 
         RSRR_CUDA(cudaStreamSynchronize(st));
         // x had unit norm (after the first step): ||A^H A x|| -> sigma_max^2
         cur = (it == 0) ? 0.0 : sqrt(sqrt(h2));
-        if (it >= 2 && cur <= 1.02 * prev) { prev = cur; break; }
+        if ((it >= 2 && cur <= 1.02 * prev) || cur > enough) { prev = cur; break; }
         prev = cur;
     }
     *est = prev;
@@ -606,13 +615,9 @@ int project_run(rsrr_nep h, double delta) {
     // ---- Householder QR with early termination -----------------------------------------------
     // stop once the trailing block's 2-norm is below 0.1 delta sigma_1 (or the noise level
     // below): dropping it moves no
-    // singular value by more than a tenth of the truncation level (Weyl).  sigma_1 is taken
-    // from a power-iteration estimate of ||S_hat||_2 (a lower bound, so the rule stays safe).
+    // singular value by more than a tenth of the truncation level (Weyl).
     HqrWork hw;
     TRYC(hw.alloc(n, m, kmax, st));
-    double s1_est = 0.0;
-    TRYC(block_norm2_est(A, n, 0, (int)n, 0, m, 30, hw.px, hw.py, hw.dnorm, st, &s1_est));
-    const double sref = std::max(smax, s1_est);
     // The stop level is raised to the rounding noise of S_hat itself when that is higher, up
     // to 0.3 delta sigma_1: in FP64 the trailing block of the QR levels off near u ||S_hat||_F
     // (measured: a plateau at 0.7-0.9e-15 sigma_1 on the damped QEP, just under 0.1 delta
@@ -621,9 +626,42 @@ int project_run(rsrr_nep h, double delta) {
     // no singular value by more than that (Weyl).
     double fro2 = 0.0;
     for (double c : cn) fro2 += c * c;
-    const double noise = std::min(8.0 * 1.1102230246251565e-16 * std::sqrt(fro2), 0.3 * delta * sref);
+    const double fro = std::sqrt(fro2);
+    auto stop_level = [&](double s1) {
+        return std::max(0.1 * delta * s1, std::min(8.0 * 1.1102230246251565e-16 * fro, 0.3 * delta * s1));
+    };
+    // sigma_1 is taken from a power-iteration estimate (a lower bound, so the rule stays safe) of the
+    // rows of R at the first panel that could be the last: there the rest is below 1e-12 sigma_1, and an
+    // iteration reads kk x m values instead of n x m (n = 40000, m = 2048: 1.4 ms an iteration).
+    // Until then ||S_hat||_F bounds it.
+    double sref = smax;
+    bool have_s1 = false;
+    auto sigma1_of_r = [&](int kk_now) -> int {
+        c128 *Rh = nullptr, *x = nullptr, *y = nullptr;
+        auto release = [&]() { for (c128* p : {Rh, x, y}) dfree(p, st); };
+        int r = dalloc_n(&Rh, (size_t)m * kk_now, st);
+        if (r == RSRR_OK) r = dalloc_n(&x, (size_t)kk_now, st);
+        if (r == RSRR_OK) r = dalloc_n(&y, (size_t)m, st);
+        double est = 0.0;
+        if (r == RSRR_OK) {
+            { rkeep_h_kernel<<<(unsigned)ceil_div((int64_t)m * kk_now, 256), 256, 0, st>>>(A, n, m, kk_now, Rh); note_launch(); }
+            r = block_norm2_est(Rh, m, 0, m, 0, kk_now, 30, x, y, hw.dnorm, st, &est);
+        }
+        release();
+        if (r == RSRR_OK) {
+            sref = std::max(smax, est);
+            have_s1 = true;
+        }
+        return r;
+    };
+    StopRule rule{stop_level(fro), [&](int kk_now, double* stop) {
+                      RSRR_TRY(sigma1_of_r(kk_now));
+                      *stop = stop_level(sref);
+                      return RSRR_OK;
+                  }};
     int kk = 0, npan = 0;
-    TRYC(householder_qr(A, n, m, n, hw, std::max(0.1 * delta * sref, noise), &kk, &npan));
+    TRYC(householder_qr(A, n, m, n, hw, &rule, &kk, &npan));
+    if (!have_s1) TRYC(sigma1_of_r(kk));
     pc.mark();  // QR done
     // ---- SVD of R_keep (kk x m) ---------------------------------------------------------------
     // R_keep^H = Q2 R2 (a second QR, only R2 kept), so R_keep = R2^H Q2^H and the left singular
@@ -638,7 +676,7 @@ int project_run(rsrr_nep h, double delta) {
         HqrWork hw2;
         TRYC(hw2.alloc(m, kk, std::min(m, kk), st));
         int kk2 = 0, np2 = 0;
-        TRYC(householder_qr(B, m, kk, m, hw2, -1.0, &kk2, &np2));
+        TRYC(householder_qr(B, m, kk, m, hw2, nullptr, &kk2, &np2));
         TRYC(dalloc_n(&X, (size_t)kk * kk, st));
         { rkeep_h_kernel<<<(unsigned)ceil_div((int64_t)kk * kk, 256), 256, 0, st>>>(B, m, kk, kk, X); note_launch(); }
     }
@@ -917,7 +955,7 @@ int jacobi_svd_preconditioned(c128* H, int D, c128* Jr, cudaStream_t st, double 
     HqrWork hw;
     TRYR(hw.alloc(D, D, D, st));
     int kk = 0, npan = 0;
-    TRYR(householder_qr(A, D, D, D, hw, -1.0, &kk, &npan));
+    TRYR(householder_qr(A, D, D, D, hw, nullptr, &kk, &npan));
     // X = R^H, then the Jacobi with the rotations accumulated into Jr (used as J here)
     { rkeep_h_kernel<<<(unsigned)ceil_div(DD, 256), 256, 0, st>>>(A, D, D, D, X); note_launch(); }
     { identity_kernel<<<(unsigned)ceil_div(DD, 256), 256, 0, st>>>(Jr, D); note_launch(); }
