@@ -6,7 +6,7 @@
 //             T_S(z_j)^{-1}: blocked Gauss-Jordan elimination with partial pivoting, batched
 //             over the points, its rank-bb updates on the ZGEMM (zinv.cu); for k_S too large
 //             for its panels, a dense LU on the band kernels (kl = ku = k_S-1) solved against I.
-//             The weighted sums are one ZGEMM.
+//             The weighted sums are one pass over the inverses (moments_kernel).
 //   winding   1/(i N_S) sum_j phi'_j tr(T_S(z_j)^{-1} T_S'(z_j))            (Eq. eq-ncs)
 //   Hankel    H, H^< from A_0..A_{2K-1}                                      (Eq. eq-HH)
 //   SVD of H  one-sided Jacobi with accumulated rotations                  (Eq. eq-svdH)
@@ -64,6 +64,71 @@ __global__ void transpose_terms_kernel(const c128* P, int k, int J, c128* Pt) {
     if (idx >= (int64_t)k * k) return;
     const int r = (int)(idx % k), c = (int)(idx / k);
     Pt[(int64_t)i * k * k + c + (int64_t)r * k] = P[(int64_t)i * k * k + idx];
+}
+
+// Moments mom_a[e] += sum_j X_j[e] W[j][a] for kThin columns a, one entry e a thread.  As a product it
+// has k^2 rows and a handful of columns: a GEMM tile spends its time on staging.  FP64-bound (0.69 ms for
+// k = 233, 500 points and 4 moments); 64 threads a CTA so that the last wave is short.
+constexpr int kThin = 4;
+constexpr int kMomThreads = 64, kMomPoints = 256;
+__global__ void __launch_bounds__(kMomThreads) moments_kernel(const c128* __restrict__ X, int64_t kk, int np,
+                                                              const c128* __restrict__ W, int64_t ldw, int na, c128* mom) {
+    __shared__ c128 w[kMomPoints][kThin];
+    const int64_t e = (int64_t)blockIdx.x * kMomThreads + threadIdx.x;
+    const int a0 = blockIdx.y * kThin;
+    c128 acc[kThin] = {czero<double>(), czero<double>(), czero<double>(), czero<double>()};
+    for (int j0 = 0; j0 < np; j0 += kMomPoints) {
+        const int nj = min(kMomPoints, np - j0);
+        __syncthreads();
+        for (int idx = threadIdx.x; idx < nj * kThin; idx += kMomThreads) {
+            const int j = idx / kThin, a = idx % kThin;
+            w[j][a] = a0 + a < na ? W[j0 + j + (int64_t)(a0 + a) * ldw] : czero<double>();
+        }
+        __syncthreads();
+        if (e < kk) {
+            const c128* x = X + (int64_t)j0 * kk + e;
+#pragma unroll 8
+            for (int j = 0; j < nj; ++j) {
+                const c128 v = x[(int64_t)j * kk];
+#pragma unroll
+                for (int a = 0; a < kThin; ++a) cfma(acc[a], v, w[j][a]);
+            }
+        }
+    }
+    if (e < kk)
+#pragma unroll
+        for (int a = 0; a < kThin; ++a)
+            if (a0 + a < na) mom[(int64_t)(a0 + a) * kk + e] = mom[(int64_t)(a0 + a) * kk + e] + acc[a];
+}
+
+// Traces tr(X_j P_i) = vec(X_j)^T vec(P_i^T) for kThin terms i, one matrix a CTA (FP64-bound as above).
+__global__ void __launch_bounds__(256) trace_kernel(const c128* __restrict__ X, int64_t kk, const c128* __restrict__ Pt,
+                                                    int J, c128* out, int64_t ldo) {
+    __shared__ c128 red[8][kThin];
+    const int i0 = blockIdx.y * kThin, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const c128* x = X + (int64_t)blockIdx.x * kk;
+    c128 acc[kThin] = {czero<double>(), czero<double>(), czero<double>(), czero<double>()};
+#pragma unroll 4
+    for (int64_t e = threadIdx.x; e < kk; e += 256) {
+        const c128 v = x[e];
+#pragma unroll
+        for (int i = 0; i < kThin; ++i)
+            if (i0 + i < J) cfma(acc[i], v, Pt[(int64_t)(i0 + i) * kk + e]);
+    }
+#pragma unroll
+    for (int i = 0; i < kThin; ++i) {
+        for (int off = 16; off; off >>= 1) {
+            acc[i].re += __shfl_xor_sync(0xffffffffu, acc[i].re, off);
+            acc[i].im += __shfl_xor_sync(0xffffffffu, acc[i].im, off);
+        }
+        if (lane == 0) red[warp][i] = acc[i];
+    }
+    __syncthreads();
+    if (threadIdx.x < kThin && i0 + (int)threadIdx.x < J) {
+        c128 s = red[0][threadIdx.x];
+        for (int w = 1; w < 8; ++w) s = s + red[w][threadIdx.x];
+        out[blockIdx.x + (int64_t)(i0 + threadIdx.x) * ldo] = s;
+    }
 }
 
 // H (or H^<) from the moments: block (r, c) = A_{r + c + shift}
@@ -508,17 +573,30 @@ int solve_run(rsrr_nep h, int N_S, int K, double tol_gap, int cap, double* lambd
         CUDAC(cudaStreamSynchronize(st));
         for (int t = 0; t < np; ++t)
             if (hinfo[t]) { cleanup(); return set_error(RSRR_ESINGULAR, "T_S(z) is singular at a quadrature point"); }
-        // moments: [k^2 x 2K] += [k^2 x np] * Wt[j0:j0+np, :]
-        Zgemm gm;
-        gm.opA = OP_N; gm.opB = OP_N; gm.M = (int)kk; gm.N = 2 * K; gm.K = np;
-        gm.A = X; gm.lda = kk; gm.B = dWt + j0; gm.ldb = N_S; gm.C = mom; gm.ldc = kk;
-        gm.beta = mk<double>(1.0, 0.0);
-        TRYC(zgemm(gm, st));
-        // traces tr(X_j P_i) = vec(X_j)^T vec(P_i^T): [np x J]
-        Zgemm gt;
-        gt.opA = OP_T; gt.opB = OP_N; gt.M = np; gt.N = J; gt.K = (int)kk;
-        gt.A = X; gt.lda = kk; gt.B = Pt; gt.ldb = kk; gt.C = trc + j0; gt.ldc = N_S;
-        TRYC(zgemm(gt, st));
+        // Both are products with a thin side.  moments_kernel needs k^2 / 64 CTAs to fill the GPU (each walks
+        // all points: 0.3 ms at k = 45, where the GEMM's K slices take 0.1) and wins by a factor of 2.6 from
+        // there on (k = 233: 0.76 ms); from 9 columns or terms on the emulated GEMM is the faster one.
+        const int64_t mctas = ceil_div(kk, kMomThreads);
+        if (2 * K <= 2 * kThin && mctas >= 2 * 152) {
+            moments_kernel<<<dim3((unsigned)mctas, (unsigned)ceil_div(2 * K, kThin)), kMomThreads, 0, st>>>(X, kk, np, dWt + j0, N_S, 2 * K, mom);
+            note_launch();
+        } else {
+            Zgemm gm;  // [k^2 x 2K] += [k^2 x np] * Wt[j0:j0+np, :]
+            gm.opA = OP_N; gm.opB = OP_N; gm.M = (int)kk; gm.N = 2 * K; gm.K = np;
+            gm.A = X; gm.lda = kk; gm.B = dWt + j0; gm.ldb = N_S; gm.C = mom; gm.ldc = kk;
+            gm.beta = mk<double>(1.0, 0.0);
+            TRYC(zgemm(gm, st));
+        }
+        if (J <= 2 * kThin) {
+            trace_kernel<<<dim3((unsigned)np, (unsigned)ceil_div(J, kThin)), 256, 0, st>>>(X, kk, Pt, J, trc + j0, N_S);
+            note_launch();
+        } else {
+            Zgemm gt;  // [np x J]
+            gt.opA = OP_T; gt.opB = OP_N; gt.M = np; gt.N = J; gt.K = (int)kk;
+            gt.A = X; gt.lda = kk; gt.B = Pt; gt.ldb = kk; gt.C = trc + j0; gt.ldc = N_S;
+            TRYC(zgemm(gt, st));
+        }
+        CUDAC(cudaGetLastError());
     }
     cudaEventRecord(ev[1], st);  // inverses, moments, traces done
     std::vector<c128> htr((size_t)N_S * J);
