@@ -30,6 +30,7 @@
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <string>
 
 #include "band_tc.cuh"
@@ -710,74 +711,86 @@ __global__ void __launch_bounds__(kFwdThreads) band_fwd_tc_kernel(SolveArgs<floa
 //                                   kv columns; x_right: the rows already solved)
 //   x_blk = inv(U11) r
 // U12 is a rectangle of the band's dense view (rows x = kv + k0 .. + 31, columns c), so it
-// arrives by TMA in chunks of 32 x 64 into a ring of nbuf shared-memory buffers; thread 0 keeps
-// the ring nbuf - 1 chunks ahead of the consumers, across panel boundaries.  Entries of a chunk
-// right of a row's band (c > row + kv) are never used.  The solved rows a panel needs (the kv
-// rows below it) stay in a circular window of shared memory (row c at c mod wrows, 16 columns).
-// U12 x_right is tiled over the threads: lane q = block row, warp w = (column group w % 4 of four
-// right-hand sides, quarter w / 4 of each chunk's 64 columns); the four quarters' partial sums are
-// added at the end of the panel.  Per step a thread loads one U entry and four window entries
-// (broadcast) for four complex multiply-adds.
-// The panels are a serial chain on few CTAs (32 to 64 of 152 SMs have one), so what bounds the
-// kernel is the issue rate of one SM and the latency between a panel's barriers, not memory.
-// So: a whole share of a chunk is a fixed-length unrolled loop whose window row is a running
-// index; inv(U11) and the block's right-hand sides of a panel are loaded while its products run
-// (inv(U11) a panel ahead, in registers, then in two alternating buffers); the product with
+// arrives by TMA in chunks of 32 x 64 into a ring of nbuf shared-memory buffers.  Warps run through
+// a panel's chunks without a block barrier: each waits for a chunk's arrival and reports its use on
+// the slot's second mbarrier, and thread 0, a chunk behind, refills the slot that all warps have
+// left (so the ring runs ahead across panels).  Entries of a chunk right of a row's band (c > row +
+// kv) are never used.  The solved rows a panel needs (the kv rows below it) stay in a circular
+// window of shared memory (row c at c mod wrows, 4 G columns).
+// U12 x_right is tiled over the threads: lane q = block row, warp w = (column group w % G of four
+// right-hand sides, share w / G of each chunk's 64 columns: 16 / G shares of 4 G); the shares'
+// partial sums are added at the end of the panel.  Per step a thread loads one U entry and four
+// window entries (broadcast) for four complex multiply-adds.  G = 1, 2 or 4, the least that holds
+// the block's right-hand sides, so that all 16 warps have work for any number of them.
+// The panels are a serial chain in one block, so what bounds the kernel is the issue rate of one
+// SM and the latency between a panel's barriers, not memory: with 16 columns, of about 20 thousand
+// cycles a panel 7 are the multiply-adds' own and 2 the panel's end.  So: a whole share is a fixed-length
+// unrolled loop; inv(U11) and the block's right-hand sides of a panel are loaded while its products
+// run (inv(U11) a panel ahead, in registers, then in two alternating buffers); the product with
 // inv(U11) has a fixed length, over the stored zeros, in two sums; and one barrier with a vote
-// closes the panel.  n = 40000, kl = 200, 32 points, 16 right-hand sides: 16.2 -> 14.0 ms a call;
-// n = 9991: 2.32 -> 1.78 ms.
+// closes the panel.
 // One CTA per (point, share of at most 16 right-hand sides).  A bounded wait that gives up marks
 // the point's solution non-finite (the caller's residual check then reports it).
+// Measured, a call: n = 9991, kv = 206, 31 points, 13 right-hand sides: 2.32 ms with a barrier a
+// chunk and a window test a column, 1.78 unrolled, 1.61 with the slots' own barriers and G = 2,
+// 1.38 with G = 1 and four CTAs a point; n = 40000, kv = 400, 64 points: 16.2 -> 14.0 unrolled,
+// the same with the slots' own barriers (16 columns a CTA: all warps had work before, too).
 // ------------------------------------------------------------------------------------------
 constexpr int kBwdThreads = 512;
 constexpr int kBwdCh = 64;                                  // U12 columns per chunk
 constexpr uint32_t kBwdChBytes = kBwdCh * NB * 8;           // 16 KB
 constexpr int kBwdMaxBuf = 8;
-constexpr int kBwdCols = 16;                                // right-hand sides per CTA
-constexpr int kBwdPartLd = 18;                              // row stride of the partial sums (16-byte rows)
+constexpr int kBwdCols = 16;                                // right-hand sides per CTA, at most
 
+template <int G>
 __global__ void __launch_bounds__(kBwdThreads)
     band_bwd_tc_kernel(const __grid_constant__ CUtensorMap umap, SolveArgs<float> a, int wrows, int nbuf) {
     extern __shared__ __align__(16) unsigned char bwd_raw[];
-    __shared__ __align__(8) uint64_t fb[kBwdMaxBuf];
+    __shared__ __align__(8) uint64_t fb[kBwdMaxBuf], eb[kBwdMaxBuf];  // chunk arrived; chunk used by every warp
+    constexpr int NW = kBwdThreads / 32, S = NW / G, W = kBwdCh / S;  // shares of a chunk, columns of a share
+    constexpr int C = 4 * G, PL = C + 2;  // window columns; row stride of the partial sums (16-byte rows)
     const BandDims d = a.d;
     const int pt = blockIdx.x / a.split, part = blockIdx.x % a.split;
     if (a.active && !a.active[pt]) return;
-    const int tid = threadIdx.x, q = tid & 31, w = tid >> 5, cg = w & 3, ks = w >> 2;
+    const int tid = threadIdx.x, q = tid & 31, w = tid >> 5, cg = w % G, ks = w / G;
     const c64* lp = a.lp + pt * a.lp_stride;
     const int c_lo = (int)((int64_t)a.L * part / a.split), c_hi = (int)((int64_t)a.L * (part + 1) / a.split);
     c64* x = a.x + pt * a.x_stride + (int64_t)c_lo * d.n;
     const int Lp = c_hi - c_lo, n = d.n, kv = d.kv;
     // [nbuf][kBwdCh][32] U12 chunks (TMA box layout), 1024-byte aligned (the size includes the slack)
     c64* ub = reinterpret_cast<c64*>(bwd_raw + ((1024u - (smem_u32(bwd_raw) & 1023u)) & 1023u));
-    c64* win = ub + (size_t)nbuf * kBwdCh * 32;         // [wrows][16]
-    c64* ui = win + (size_t)wrows * kBwdCols;           // [2][32][33] inv(U11) of this panel and the next
-    c64* pr = ui + 2 * 32 * 33;                         // [4][32][kBwdPartLd] partial sums, then r
+    c64* win = ub + (size_t)nbuf * kBwdCh * 32;         // [wrows][C]
+    c64* ui = win + (size_t)wrows * C;                  // [2][32][33] inv(U11) of this panel and the next
+    c64* pr = ui + 2 * 32 * 33;                         // [S][32][PL] partial sums, then r
     const bool grp = 4 * cg < Lp;                       // this thread's column group holds a right-hand side
     auto chunks_of = [&](int p) {
         const int k0 = p * NB, cb = k0 + min(NB, n - k0), c_end = min(n, k0 + NB + kv);
         return cb < c_end ? (c_end - cb + kBwdCh - 1) / kBwdCh : 0;
     };
     // producer state (thread 0): the next chunk to load
-    int pp = d.npanels - 1, pc = 0;
-    auto issue_next = [&](int slot) {
+    int pp = d.npanels - 1, pc = 0, issued = 0;
+    auto issue_next = [&] {
         while (pp >= 0 && pc >= chunks_of(pp)) { --pp; pc = 0; }
         if (pp < 0) return;
+        const int slot = issued++ % nbuf;
         const int k0 = pp * NB, cb = k0 + min(NB, n - k0);
         mbar_expect_tx(&fb[slot], kBwdChBytes);
         tma_load_3d(ub + (size_t)slot * kBwdCh * 32, &umap, kv + k0, cb + pc * kBwdCh, pt, &fb[slot]);
         ++pc;
     };
     if (tid == 0) {
-        for (int i = 0; i < nbuf; ++i) mbar_init(&fb[i], 1);
+        for (int i = 0; i < nbuf; ++i) {
+            mbar_init(&fb[i], 1);
+            mbar_init(&eb[i], NW);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&umap) : "memory");
     }
     // the last chunk of a panel can reach columns whose window slots were never written
-    for (int idx = tid; idx < wrows * kBwdCols; idx += kBwdThreads) win[idx] = czero<float>();
+    for (int idx = tid; idx < wrows * C; idx += kBwdThreads) win[idx] = czero<float>();
     __syncthreads();
     if (tid == 0)
-        for (int i = 0; i < nbuf; ++i) issue_next(i);
+        for (int i = 0; i < nbuf; ++i) issue_next();
     // inv(U11) of a panel is loaded into registers while the panel before it is worked on
     constexpr int kUi = NB * NB / kBwdThreads;
     c64 nui[kUi];
@@ -806,66 +819,66 @@ __global__ void __launch_bounds__(kBwdThreads)
         c64 acc[4] = {czero<float>(), czero<float>(), czero<float>(), czero<float>()};
         // this row's band ends at column row + kv (and the matrix at n - 1)
         const int c_stop = min(n, row + kv + 1);
-        int sw0 = (cb + ks * (kBwdCh / 4)) % wrows;  // window row of this share's first column
+        // Window row of this share's first column.  cb, wrows and a share are multiples of W, so a
+        // share never crosses the end of the window.
+        int sw0 = (cb + ks * W) % wrows;
         for (int ch = 0; ch < nch; ++ch, ++g) {
             const int slot = g % nbuf;
             if (!fail && !mbar_wait(&fb[slot], (uint32_t)((g / nbuf) & 1))) fail = true;
-            const c64* u = ub + (size_t)slot * kBwdCh * 32;
-            const int c0 = cb + ch * kBwdCh;
             if (grp && q < nbe && !fail) {
-                const int j0 = ks * (kBwdCh / 4), j1 = min(j0 + kBwdCh / 4, c_stop - c0);
-                const c64* uq = u + q;
-                const c64* wc = win + 4 * cg;
-                auto step = [&](int j, int sw) {
-                    const c64 uv = uq[j * 32];
-                    const float4* wp = reinterpret_cast<const float4*>(wc + (size_t)sw * kBwdCols);
+                const int j0 = ks * W, nj = c_stop - (cb + ch * kBwdCh) - j0;
+                const c64* u = ub + (size_t)slot * kBwdCh * 32 + (size_t)j0 * 32 + q;
+                const c64* wc = win + (size_t)sw0 * C + 4 * cg;
+                auto step = [&](int j) {
+                    const c64 uv = u[j * 32];
+                    const float4* wp = reinterpret_cast<const float4*>(wc + j * C);
                     const float4 w01 = wp[0], w23 = wp[1];
                     cfms(acc[0], uv, mk<float>(w01.x, w01.y));
                     cfms(acc[1], uv, mk<float>(w01.z, w01.w));
                     cfms(acc[2], uv, mk<float>(w23.x, w23.y));
                     cfms(acc[3], uv, mk<float>(w23.z, w23.w));
                 };
-                if (j1 - j0 == kBwdCh / 4 && sw0 + kBwdCh / 4 <= wrows) {  // a whole share, no wrap in the window
+                if (nj >= W) {
 #pragma unroll
-                    for (int j = 0; j < kBwdCh / 4; ++j) step(j0 + j, sw0 + j);
+                    for (int j = 0; j < W; ++j) step(j);
                 } else {
-                    int sw = sw0;
-                    for (int j = j0; j < j1; ++j) {
-                        step(j, sw);
-                        if (++sw == wrows) sw = 0;
-                    }
+                    for (int j = 0; j < nj; ++j) step(j);
                 }
             }
             sw0 += kBwdCh;
             if (sw0 >= wrows) sw0 -= wrows;
-            __syncthreads();  // the slot is free again
-            if (tid == 0 && !fail) issue_next(slot);
+            __syncwarp();
+            if (q == 0) mbar_arrive(&eb[slot]);
+            // refill the slot of the chunk before this one: the other warps are seldom behind it
+            if (tid == 0 && !fail && g > 0) {
+                if (mbar_wait(&eb[(g - 1) % nbuf], (uint32_t)(((g - 1) / nbuf) & 1))) issue_next();
+                else fail = true;
+            }
         }
         {
-            float4* pp4 = reinterpret_cast<float4*>(pr + ((size_t)ks * 32 + q) * kBwdPartLd + 4 * cg);
+            float4* pp4 = reinterpret_cast<float4*>(pr + ((size_t)ks * 32 + q) * PL + 4 * cg);
             pp4[0] = make_float4(acc[0].re, acc[0].im, acc[1].re, acc[1].im);
             pp4[1] = make_float4(acc[2].re, acc[2].im, acc[3].re, acc[3].im);
         }
         __syncthreads();
-        // r = x_blk - sum of the quarters (thread: row q, right-hand side w)
-        if (w < Lp && q < nbe) {
+        // r = x_blk - sum of the shares (thread: row q, right-hand side w)
+        if (w < Lp) {
             c64 r = xb;
-            for (int s2 = 0; s2 < 4; ++s2) r = r + pr[((size_t)s2 * 32 + q) * kBwdPartLd + w];
-            pr[(size_t)q * kBwdPartLd + w] = r;
-        } else if (q >= nbe) {
-            pr[(size_t)q * kBwdPartLd + w] = czero<float>();  // meets zeros of inv(U11)
+#pragma unroll
+            for (int s2 = 0; s2 < S; ++s2) r = r + pr[((size_t)s2 * 32 + q) * PL + w];
+            pr[(size_t)q * PL + w] = q < nbe ? r : czero<float>();  // rows past the block meet zeros of inv(U11)
         }
         __syncthreads();
         if (w < Lp && q < nbe) {
             c64 s0 = czero<float>(), s1 = czero<float>();
 #pragma unroll
             for (int j = 0; j < NB; j += 2) {  // inv(U11) is stored with its zeros
-                cfma(s0, uip[q * 33 + j], pr[(size_t)j * kBwdPartLd + w]);
-                cfma(s1, uip[q * 33 + j + 1], pr[(size_t)(j + 1) * kBwdPartLd + w]);
+                cfma(s0, uip[q * 33 + j], pr[(size_t)j * PL + w]);
+                cfma(s1, uip[q * 33 + j + 1], pr[(size_t)(j + 1) * PL + w]);
             }
             const c64 sacc = s0 + s1;
             x[row + (int64_t)w * n] = sacc;
-            win[(size_t)(row % wrows) * kBwdCols + w] = sacc;
+            win[(size_t)(row % wrows) * C + w] = sacc;
         }
         // one barrier for the window, the partial sums and the common decision to stop
         if (__syncthreads_or(fail)) { stop = true; break; }
@@ -874,7 +887,7 @@ __global__ void __launch_bounds__(kBwdThreads)
         // let the loads in flight land (bounded) before the block's shared memory is released,
         // then mark this share of the solution non-finite
         if (tid == 0)
-            for (int i = 0; i < nbuf; ++i) mbar_wait(&fb[(g + i) % nbuf], (uint32_t)(((g + i) / nbuf) & 1), 1u << 16);
+            for (int i = g; i < issued; ++i) mbar_wait(&fb[i % nbuf], (uint32_t)((i / nbuf) & 1), 1u << 16);
         const float nan = __int_as_float(0x7fc00000);
         for (int64_t idx = tid; idx < (int64_t)Lp * n; idx += kBwdThreads) x[idx] = mk<float>(nan, nan);
     }
@@ -981,38 +994,48 @@ int launch_factor_tc(const FactorArgs<float>& a, int npts, cudaStream_t s) {
 
 namespace {
 int bwd_window_rows(const BandDims& d) { return (d.kv + 2 * NB + 31) / 32 * 32; }  // >= kv + 64 solved rows
-size_t bwd_smem(const BandDims& d, int nbuf) {
-    return (size_t)nbuf * kBwdChBytes + (size_t)bwd_window_rows(d) * kBwdCols * sizeof(c64) +
-           (size_t)2 * 32 * 33 * sizeof(c64) + (size_t)4 * 32 * kBwdPartLd * sizeof(c64) + 1024;
+size_t bwd_smem(const BandDims& d, int nbuf, int G) {
+    return (size_t)nbuf * kBwdChBytes + (size_t)bwd_window_rows(d) * 4 * G * sizeof(c64) +
+           (size_t)2 * 32 * 33 * sizeof(c64) + (size_t)(kBwdThreads / 32 / G) * 32 * (4 * G + 2) * sizeof(c64) + 1024;
 }
 constexpr size_t kBwdSmemMax = 224 * 1024;
-int bwd_nbuf(const BandDims& d) {
-    for (int nb : {kBwdMaxBuf, 4, 2})
-        if (bwd_smem(d, nb) <= kBwdSmemMax) return nb;
+int bwd_nbuf(const BandDims& d, int G) {
+    for (int nb = kBwdMaxBuf; nb >= 2; --nb)
+        if (bwd_smem(d, nb, G) <= kBwdSmemMax) return nb;
     return 0;
 }
-}  // namespace
-
-bool band_bwd_tc_fits(const BandDims& d) { return bwd_nbuf(d) > 0; }
-
-int launch_bwd_tc(const SolveArgs<float>& a, int npts, cudaStream_t s) {
-    if (a.L > 64) return set_error(RSRR_EINVAL, "launch_bwd_tc: at most 64 right-hand sides");
-    const int nbuf = bwd_nbuf(a.d);
+template <int G>
+int launch_bwd_tc_groups(const CUtensorMap& map, const SolveArgs<float>& b, int npts, cudaStream_t s) {
+    const int nbuf = bwd_nbuf(b.d, G);
     if (!nbuf) return set_error(RSRR_EINVAL, "launch_bwd_tc: band too wide for the solved-row window");
-    if ((a.d.kv & 1) || (a.ab_stride & 1) || (reinterpret_cast<uintptr_t>(a.ab) & 15))
-        return set_error(RSRR_EINVAL, "launch_bwd_tc: band layout not prepared for TMA");
-    const int wrows = bwd_window_rows(a.d);
-    const size_t sm = bwd_smem(a.d, nbuf);
-    CUtensorMap map;
-    RSRR_TRY(band_tensor_map(&map, a.ab, a.ab_stride, npts, a.d, NB, kBwdCh));
-    RSRR_TRY(set_smem_max(band_bwd_tc_kernel, sm, "band_bwd_tc_kernel"));
-    SolveArgs<float> b = a;
-    b.split = a.L > kBwdCols ? 2 : solve_split_tc(npts, a.L);
-    if ((a.L + b.split - 1) / b.split > kBwdCols) b.split = (a.L + kBwdCols - 1) / kBwdCols;
-    band_bwd_tc_kernel<<<npts * b.split, kBwdThreads, sm, s>>>(map, b, wrows, nbuf);
+    const size_t sm = bwd_smem(b.d, nbuf, G);
+    RSRR_TRY(set_smem_max(band_bwd_tc_kernel<G>, sm, "band_bwd_tc_kernel"));
+    band_bwd_tc_kernel<G><<<npts * b.split, kBwdThreads, sm, s>>>(map, b, bwd_window_rows(b.d), nbuf);
     note_launch();
     RSRR_CUDA(cudaGetLastError());
     return RSRR_OK;
+}
+}  // namespace
+
+bool band_bwd_tc_fits(const BandDims& d) { return bwd_nbuf(d, kBwdCols / 4) > 0; }
+
+int launch_bwd_tc(const SolveArgs<float>& a, int npts, cudaStream_t s) {
+    if (a.L > 64) return set_error(RSRR_EINVAL, "launch_bwd_tc: at most 64 right-hand sides");
+    if ((a.d.kv & 1) || (a.ab_stride & 1) || (reinterpret_cast<uintptr_t>(a.ab) & 15))
+        return set_error(RSRR_EINVAL, "launch_bwd_tc: band layout not prepared for TMA");
+    CUtensorMap map;
+    RSRR_TRY(band_tensor_map(&map, a.ab, a.ab_stride, npts, a.d, NB, kBwdCh));
+    SolveArgs<float> b = a;
+    // CTAs a point: as many as fill the SMs once, with at least four right-hand sides each (31 points,
+    // 13 right-hand sides: two CTAs a point 1.61 ms, four 1.38 ms)
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    b.split = std::max((a.L + kBwdCols - 1) / kBwdCols, std::min(nsm / std::max(npts, 1), (a.L + 3) / 4));
+    const int cols = (a.L + b.split - 1) / b.split;
+    if (cols <= 4) return launch_bwd_tc_groups<1>(map, b, npts, s);
+    if (cols <= 8) return launch_bwd_tc_groups<2>(map, b, npts, s);
+    return launch_bwd_tc_groups<4>(map, b, npts, s);
 }
 
 int launch_fwd_tc(const SolveArgs<float>& a, int npts, cudaStream_t s) {

@@ -33,10 +33,10 @@ int launch_factor_tc(const FactorArgs<float>& a, int npts, cudaStream_t s);
 // Solves take at most 64 right-hand sides per launch (EINVAL beyond).
 int launch_fwd_tc(const SolveArgs<float>& a, int npts, cudaStream_t s);
 // Backward solve with U in the band and the stored inv(U11) blocks.  Its shared memory holds a
-// window of kv + 64 solved rows (16 right-hand sides) and a ring of TMA-loaded U12 chunks (8
-// buffers up to kv ~ 480, 4 up to ~990, 2 up to ~1250: band_bwd_tc_fits); beyond that the
+// window of kv + 64 solved rows (4, 8 or 16 right-hand sides) and a ring of TMA-loaded U12 chunks
+// (with 16: 8 buffers up to kv ~ 416, 4 up to ~ 928, 2 up to ~ 1184: band_bwd_tc_fits); beyond that the
 // CUDA-core backward solve (band.cuh) takes the same storage.  (The sampler sends bands with
-// ku > 768 to the dense LU, so it uses the eight- and four-buffer plans.)
+// ku > 768 to the dense LU, so it uses the plans of three to eight buffers.)
 bool band_bwd_tc_fits(const BandDims& d);
 int launch_bwd_tc(const SolveArgs<float>& a, int npts, cudaStream_t s);
 

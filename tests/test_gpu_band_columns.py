@@ -1,0 +1,26 @@
+"""The backward solve of the tensor-core band path gives a thread block 4, 8 or 16 right-hand sides,
+by the number of points and columns of a batch: the shares of a chunk, the window and the partial
+sums differ with it.  80 points keep every column of a point in one block (3, 7 and 14 columns: the
+three forms, ragged); 20 columns take two blocks of 10; 6 points spread 18 columns over five blocks.
+
+A0 has rows of modulus sum below 130 off the diagonal and 200 on it, so cond(T) < 6 and a solution
+with backward error 2e-15 is within 1.2e-14 of the exact one; the bound leaves three digits for norms."""
+import numpy as np
+import pytest
+
+import oracle
+from gpu_util import rel_err_cols
+from test_gpu_band_tc import banded_problem, rs, run  # noqa: F401  (rs is the module's fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("N,L", [(80, 1), (80, 3), (80, 7), (80, 14), (80, 20), (6, 18)])
+def test_backward_solve_column_groups(rs, N, L):  # noqa: F811
+    prob = banded_problem(450, 40, 37, seed=N + L, N=N, L=L, shift=200.0)
+    X, eta, info = run(rs, prob, rs.RSRR_C64_IR | rs.RSRR_REFINE_FULL, 1e-10)
+    assert info["band_lu_tc"] == 1 and info["dense_lu"] == 0
+    ref, infos, _ = oracle.sample(prob)
+    assert np.all(infos == 0)
+    assert eta.max() <= 2e-15
+    assert rel_err_cols(X, ref).max() < 1e-11
