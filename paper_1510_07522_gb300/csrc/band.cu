@@ -12,6 +12,7 @@
 // The forward solve reuses step B verbatim on the right-hand-side columns; the backward
 // solve runs the same routine in reversed row order with a non-unit diagonal.
 #include <cooperative_groups.h>
+#include <algorithm>
 
 #include "band.cuh"
 
@@ -593,13 +594,16 @@ int set_smem(K kernel, size_t sm, const char* name) {
 }
 }  // namespace
 
-// CTAs per point for the solves: two when the doubled grid still fits one wave, so the
-// right-hand-side columns of a point are shared by two SMs.
+// CTAs per point for the solves: as many as fill the SMs once, with a right-hand side each at
+// least.  A block's columns are a warp each, so fewer of them a CTA share its FP64 (or shared-memory)
+// rate.  32 points, two CTAs a point and four: FP64, a 64 x 60 grid, 16 columns, forward 4.9 and
+// 3.0 ms, backward 6.2 and 3.9 ms; complex64, a 240 x 250 grid, 24 columns, forward 13.2 and 11.5 ms,
+// backward 33.7 and 29.6 ms.
 int solve_split(int npts, int L) {
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    return (L >= 2 && 2 * npts <= nsm) ? 2 : 1;
+    return std::max(1, std::min(nsm / std::max(npts, 1), L));
 }
 
 template <typename R>

@@ -24,3 +24,22 @@ def test_backward_solve_column_groups(rs, N, L):  # noqa: F811
     assert np.all(infos == 0)
     assert eta.max() <= 2e-15
     assert rel_err_cols(X, ref).max() < 1e-11
+
+
+@pytest.mark.parametrize("N,L,kl,ku", [(6, 7, 40, 37), (40, 5, 12, 15), (60, 17, 3, 1), (80, 4, 40, 37)])
+@pytest.mark.parametrize("fp64", [True, False])
+def test_cuda_core_solves_column_split(rs, N, L, kl, ku, fp64):  # noqa: F811
+    """The CUDA-core solves spread a point's columns over as many blocks as fill the device: one
+    column each, uneven shares, more columns than a block has warps, and one block.  FP64 has no
+    refinement: a backward error of a few (kl + ku + 2) u, below 1e-13, times cond < 6 stays below
+    1e-11 too."""
+    prob = banded_problem(450, kl, ku, seed=N + L, N=N, L=L, shift=200.0)
+    if fp64:
+        X, eta, info = run(rs, prob, rs.RSRR_FP64, 1e-10)
+    else:
+        X, eta, info = run(rs, prob, rs.RSRR_C64_IR | rs.RSRR_REFINE_FULL, 1e-10, flags=rs.RSRR_BAND_CUDA_CORES)
+    assert info["band_lu_tc"] == 0 and info["dense_lu"] == 0
+    ref, infos, _ = oracle.sample(prob)
+    assert np.all(infos == 0)
+    assert eta.max() <= 1e-13
+    assert rel_err_cols(X, ref).max() < 1e-11
