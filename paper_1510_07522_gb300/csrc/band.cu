@@ -351,25 +351,36 @@ __global__ void __launch_bounds__(kLuThreads) band_factor_kernel(FactorArgs<R> a
 }
 
 // ------------------------------------------------------------------------------------------
-// Cluster variant: two CTAs (one thread-block cluster) per sampling point, so a batch of N
-// points keeps 2N SMs busy.
-//   CTA 0: panel team (warps 0..3) + update team (warps 4..15), exactly as above; its update
-//          warps do the lead tasks (columns of the next panel) and a share of the rest.
-//   CTA 1: 16 update warps; at the start of each step it copies the finished panel block and
-//          its permutation from CTA 0's shared memory (distributed shared memory), then does
-//          the remaining share of the trailing columns.
-// Each step ends with a cluster barrier (release/acquire), which also orders both CTAs'
-// updates of the band in global memory before the next step reads them.  Every thread of
-// both CTAs reaches it exactly once per step and once after the prologue.
+// Cluster variant: C = 2 to 4 CTAs (one thread-block cluster) per sampling point, so a batch of N
+// points keeps C N SMs busy.
+//   CTA 0:  panel team (warps 0..3) + update team (warps 4..15)
+//   others: 16 update warps; at the start of each step each copies the finished panel block and
+//           its permutation from CTA 0's shared memory (distributed shared memory).
+// The next panel waits for the lead tasks (its own columns).  CTA 0's update team does them if it
+// has a warp for each; more of them go round the CTAs.  Then CTA 0's panel team factors it while all update warps share the other columns.  CTA 0's
+// share of those is by warps, and smaller where that would leave it with more work than the others:
+// the next panel counts as nb / (2 CG) tasks, by its multiply-adds.
+// A step has two cluster barriers (release/acquire), passed once by every thread of all CTAs: the
+// first, arrived at after the lead tasks and waited for only before the panel, hands the lead
+// columns to the panel team; the second ends the step and orders the CTAs' updates of the band in
+// global memory before the next step reads them.
+// 32 points, two CTAs a point and four: FP64, a 64 x 60 grid (16 lead tasks, 60 in all) 53.8 and
+// 34.6 ms (37.0 with the lead tasks on CTA 0 alone); complex64, a 240 x 250 grid (8 lead tasks, 120 in
+// all) 255.7 and 209 ms (219 with the lead tasks on all CTAs, which wait for their copy of the panel).
+// What remains is the panel's chain of columns.
 // ------------------------------------------------------------------------------------------
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
 template <typename R>
 __global__ void __launch_bounds__(kLuThreads) band_factor_cluster_kernel(FactorArgs<R> a) {
     namespace cg = cooperative_groups;
-    constexpr int CG = BandTraits<R>::CG, CH = BandTraits<R>::CH;
+    constexpr int CG = BandTraits<R>::CG, CH = BandTraits<R>::CH, NW = kLuThreads / 32;
     cg::cluster_group cluster = cg::this_cluster();
     const unsigned rank = cluster.block_rank();
+    const int C = (int)cluster.num_blocks();
     const BandDims d = a.d;
-    const int pt = blockIdx.x / 2;
+    const int pt = blockIdx.x / C;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     cplx<R>* ab = a.ab + pt * a.ab_stride;
     cplx<R>* lp = a.lp + pt * a.lp_stride;
@@ -399,35 +410,41 @@ __global__ void __launch_bounds__(kLuThreads) band_factor_cluster_kernel(FactorA
         const int ntask = max(0, (ce - cb + CG - 1) / CG);
         const bool has_next = p + 1 < d.npanels;
         const int nlead = has_next ? min(ntask, (nb + CG - 1) / CG) : 0;
-        const int rest = ntask - nlead;
-        const int n1 = (rest * 3) / 5;  // CTA 1's share of the non-lead columns
+        const int LC = nlead > kUpdateWarps ? C : 1;  // CTAs of the lead tasks
+        // CTA 0's share of the other columns: by warps, and at most what levels the work
+        const int rest = ntask - nlead, panel = nb / (2 * CG);
+        const int r0 = min(rest * kUpdateWarps / (kUpdateWarps + (C - 1) * NW),
+                           max(0, (ntask + panel) / C - (nlead + LC - 1) / LC - panel));
+        const int n1 = rest - r0;
         cplx<R>* Pb = P + (size_t)buf * blk;
         int* pb = psm + (size_t)buf * ldp;
-        if (rank == 1) {
-            // copy panel p (block and permutation) from CTA 0's shared memory
-            const cplx<R>* rP = cluster.map_shared_rank(Pb, 0);
-            const int* rpb = cluster.map_shared_rank(pb, 0);
-            for (int idx = tid; idx < blk; idx += kLuThreads) Pb[idx] = rP[idx];
-            for (int q = tid; q < ldp; q += kLuThreads) pb[q] = rpb[q];
-            __syncthreads();
-            for (int task = nlead + warp; task < nlead + n1; task += kLuThreads / 32) {
-                TrailingCols<R, CG> acc{ab, ldab, kv, k0, cb + task * CG, ce};
-                apply_block<R, CG, CH, true>(Pb, ldp, nbe, m, pb, nullptr, ust + warp * 32 * CG, acc, lane);
+        auto run = [&](int task, int uw) {
+            TrailingCols<R, CG> acc{ab, ldab, kv, k0, cb + task * CG, ce};
+            apply_block<R, CG, CH, true>(Pb, ldp, nbe, m, pb, nullptr, ust + uw * 32 * CG, acc, lane);
+        };
+        if (rank > 0) {
+            if (ntask > 0) {  // copy panel p (block and permutation) from CTA 0's shared memory
+                const cplx<R>* rP = cluster.map_shared_rank(Pb, 0);
+                const int* rpb = cluster.map_shared_rank(pb, 0);
+                for (int idx = tid; idx < blk; idx += kLuThreads) Pb[idx] = rP[idx];
+                for (int q = tid; q < ldp; q += kLuThreads) pb[q] = rpb[q];
+                __syncthreads();
             }
+            if (LC > 1)
+                for (int task = (int)rank + C * warp; task < nlead; task += C * NW) run(task, warp);
+            cluster_arrive();
+            const int t0 = nlead + n1 * ((int)rank - 1) / (C - 1), t1 = nlead + n1 * (int)rank / (C - 1);
+            for (int task = t0 + warp; task < t1; task += NW) run(task, warp);
+            cluster_wait();
         } else if (warp >= kPanelWarps) {
             const int uw = warp - kPanelWarps;
-            for (int task = uw; task < nlead; task += kUpdateWarps) {
-                TrailingCols<R, CG> acc{ab, ldab, kv, k0, cb + task * CG, ce};
-                apply_block<R, CG, CH, true>(Pb, ldp, nbe, m, pb, nullptr, ust + uw * 32 * CG, acc, lane);
-            }
-            __threadfence_block();
-            lead_arrive();
-            for (int task = nlead + n1 + uw; task < ntask; task += kUpdateWarps) {
-                TrailingCols<R, CG> acc{ab, ldab, kv, k0, cb + task * CG, ce};
-                apply_block<R, CG, CH, true>(Pb, ldp, nbe, m, pb, nullptr, ust + uw * 32 * CG, acc, lane);
-            }
+            for (int task = LC * uw; task < nlead; task += LC * kUpdateWarps) run(task, uw);
+            cluster_arrive();
+            for (int task = nlead + n1 + uw; task < ntask; task += kUpdateWarps) run(task, uw);
+            cluster_wait();
         } else {
-            lead_wait();
+            cluster_arrive();
+            cluster_wait();
             if (has_next)
                 factor_panel<R>(a, ab, lp, permg, ipiv, p + 1, P + (size_t)(buf ^ 1) * blk, psm + (size_t)(buf ^ 1) * ldp,
                                 &s_piv, &s_pval, &s_info);
@@ -612,20 +629,33 @@ int launch_factor(const FactorArgs<R>& a, int npts, cudaStream_t s) {
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (2 * npts <= nsm) {  // few points: two SMs per point
+    if (2 * npts <= nsm) {  // few points: several SMs per point
         RSRR_TRY(set_smem(band_factor_cluster_kernel<R>, sm, "band_factor_cluster_kernel"));
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(2 * npts, 1, 1);
         cfg.blockDim = dim3(kLuThreads, 1, 1);
         cfg.dynamicSmemBytes = sm;
         cfg.stream = s;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2;
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
+        // Cluster size: up to four, if all points' clusters run at once and every CTA beside CTA 0
+        // has a task for each warp (kv columns less the next panel's, in groups of CG).  Two
+        // otherwise.
+        constexpr int CG = BandTraits<R>::CG;
+        const int rest = std::max(0, (std::min(a.d.kv, a.d.n) + CG - 1) / CG - (a.d.nb + CG - 1) / CG);
+        int C = std::max(2, std::min({4, nsm / npts, 1 + (rest + kLuThreads / 32 - 1) / (kLuThreads / 32)}));
+        for (; C > 2; --C) {
+            attr[0].val.clusterDim.x = C;
+            cfg.gridDim = dim3(C * npts, 1, 1);
+            int fit = 0;
+            if (cudaOccupancyMaxActiveClusters(&fit, band_factor_cluster_kernel<R>, &cfg) == cudaSuccess && fit >= npts) break;
+            cudaGetLastError();
+        }
+        attr[0].val.clusterDim.x = C;
+        cfg.gridDim = dim3(C * npts, 1, 1);
         RSRR_CUDA(cudaLaunchKernelEx(&cfg, band_factor_cluster_kernel<R>, a));
         note_launch();
         return RSRR_OK;

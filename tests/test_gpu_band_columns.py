@@ -43,3 +43,31 @@ def test_cuda_core_solves_column_split(rs, N, L, kl, ku, fp64):  # noqa: F811
     assert np.all(infos == 0)
     assert eta.max() <= 1e-13
     assert rel_err_cols(X, ref).max() < 1e-11
+
+
+@pytest.mark.parametrize("N", [6, 45, 60])
+@pytest.mark.parametrize("fp64,kl,ku", [(True, 70, 70), (True, 90, 5), (True, 3, 40), (False, 70, 70), (False, 5, 90)])
+def test_cuda_core_factor_cluster_sizes(rs, N, fp64, kl, ku):  # noqa: F811
+    """The CUDA-core factorisation gives a point a cluster of 4, 3 or 2 blocks by the number of points,
+    and fewer where the band has few trailing columns.  The shifted band is diagonally dominant
+    (row sums off the diagonal below 240, 330 on it): cond < 7, bounds as above."""
+    prob = banded_problem(601, kl, ku, seed=N + kl, N=N, L=3, shift=330.0)
+    if fp64:
+        X, eta, info = run(rs, prob, rs.RSRR_FP64, 1e-10)
+    else:
+        X, eta, info = run(rs, prob, rs.RSRR_C64_IR | rs.RSRR_REFINE_FULL, 1e-10, flags=rs.RSRR_BAND_CUDA_CORES)
+    assert info["band_lu_tc"] == 0 and info["dense_lu"] == 0
+    ref, infos, _ = oracle.sample(prob)
+    assert np.all(infos == 0)
+    assert eta.max() <= 1e-13
+    assert rel_err_cols(X, ref).max() < 1e-11
+
+
+def test_cuda_core_factor_cluster_pivoting(rs):  # noqa: F811
+    """Rows move at nearly every column (no shift) under a cluster of four blocks: the solutions'
+    backward error.  The entries of L are at most 1 and those of U grow at most by some tens here, so eta stays below
+    100 (kl + ku + 2) u = 3e-12."""
+    prob = banded_problem(601, 60, 50, seed=5, N=6, L=3)
+    X, eta, info = run(rs, prob, rs.RSRR_FP64, 1e-10)
+    assert info["band_lu_tc"] == 0 and info["dense_lu"] == 0
+    assert eta.max() <= 3e-12
