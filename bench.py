@@ -336,9 +336,9 @@ def run_ours(args):
                 "achieved": jac_tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                 "frac": (jac_tf / FP64_PEAK_TFLOPS) if jac_tf else None, "traffic": None,
                 "peak_source": "nominal FP64 rate of GB300 (1.25 TFLOP/s)",
-                "algorithmic": "per sweep: 4 mb k for the column norms, 8 mb per pair whose inner product is "
-                               "formed, 32 mb + 24 k per rotated pair (rotation of B and of the k-row J, new "
-                               "norms); pairs and rotations counted by the kernel", "ms_per_step": jac_ms}
+                "algorithmic": "16 mb per pair formed (norms and inner product), 24 mb per rotated pair, "
+                               "+ 24 k where the k-row J is accumulated; pairs and rotations counted by the "
+                               "kernel", "ms_per_step": jac_ms}
     # the SVD stages against a fixed count that does not grow with the sweeps: a bidiagonalising
     # SVD with both vector sets, ~4 (4 m n^2 + 8 n^3) real flops for a complex m x n (m >= n):
     # the projection's SVD of R^H (N L x rows kept) and the Hankel SVD (K k_S square)

@@ -357,8 +357,8 @@ typedef struct {
     double ms_zgemm_tc;         /* the part of ms_zgemm spent in the tensor-core emulation       */
     double zgemm_tc_gflop;      /* and its algorithmic work (8 M N K per product), GFLOP        */
     double ms_jacobi;           /* device time of the one-sided Jacobi sweeps (project + solve)  */
-    double jacobi_gflop;        /* their algorithmic work: per sweep and column pair of an mb-row
-                                   matrix, 40 mb real flops (+ 24 k for the accumulated rotations) */
+    double jacobi_gflop;        /* their algorithmic work, columns of mb rows: 16 mb real flops for
+                                   a pair formed, 24 mb (+ 24 k with the k-row J) for one rotated */
     int32_t band_lu_tc;         /* 1 if the last rsrr_sample ran the complex64 band LU with its
                                    trailing updates on the tensor cores (kl in [32, 224])     */
     int32_t tune_strategy;      /* RSRR_AUTOTUNE's choice: 0 band LU (tensor cores), 1 band LU
