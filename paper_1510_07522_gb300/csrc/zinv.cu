@@ -36,7 +36,12 @@ constexpr int kZiWarps = kZiThreads / 32;
 constexpr unsigned FULLM = 0xffffffffu;
 constexpr size_t kZiSmemMax = 225 * 1024;
 
-size_t panel_smem(int rows, int bb) { return (size_t)rows * bb * sizeof(c128) + (size_t)2 * 32 * 33 * sizeof(c128); }
+// The two triangular inverses take the panel's place once it has been used, so they cost no block
+// width: 32 columns up to k = 450 (with a place of their own up to 384: at k = 404, 500 matrices,
+// 16-column blocks took 156 ms, 32-column ones take 105).
+size_t panel_smem(int rows, int bb) {
+    return std::max((size_t)rows * bb, (size_t)2 * 32 * 33) * sizeof(c128);
+}
 
 __global__ void __launch_bounds__(kZiThreads) zinv_panel_kernel(c128* X, int k, int jb, int bb, int b, int32_t* piv,
                                                                c128* E, c128* Dv, int32_t* info) {
@@ -53,8 +58,8 @@ __global__ void __launch_bounds__(kZiThreads) zinv_panel_kernel(c128* X, int k, 
     c128* Dt = Dv + (int64_t)t * b * b;
     const int rows = k - jb;
     c128* P = reinterpret_cast<c128*>(zi_raw);  // [bb][rows], column-major
-    c128* Ui = P + (size_t)rows * bb;           // [32][33] U11^{-1}, column-major
-    c128* Li = Ui + 32 * 33;                    // [32][33] L11^{-1}
+    c128* Ui = P;             // [32][33] U11^{-1}, column-major, over the panel
+    c128* Li = Ui + 32 * 33;  // [32][33] L11^{-1}
     if (tid == 0) s_sing = 0;
     for (int idx = tid; idx < rows * bb; idx += kZiThreads) {
         const int r = idx % rows, c = idx / rows;
@@ -138,10 +143,19 @@ __global__ void __launch_bounds__(kZiThreads) zinv_panel_kernel(c128* X, int k, 
     // Both triangular inverses grow from blocks of one column: [A, B; 0, C]^{-1} has -A^{-1} B C^{-1}
     // off the diagonal (and its mirror image for L).  At level w there are 16 w such entries a factor;
     // threads 0..255 take U's, threads 256..511 L's.
-    for (int idx = tid; idx < 32 * 32; idx += kZiThreads) {
-        const int r = idx % 32, c = idx / 32;
+    constexpr int kTri = 32 * 32 / kZiThreads;
+    c128 tri[kTri];
+#pragma unroll
+    for (int q = 0; q < kTri; ++q) {
+        const int idx = tid + q * kZiThreads, r = idx % 32, c = idx / 32;
+        tri[q] = r < bb && c < bb ? P[r + (int64_t)c * rows] : czero<double>();
+    }
+    __syncthreads();  // the panel has been read
+#pragma unroll
+    for (int q = 0; q < kTri; ++q) {
+        const int idx = tid + q * kZiThreads, r = idx % 32, c = idx / 32;
         const bool in = r < bb && c < bb;
-        const c128 v = in ? P[r + (int64_t)c * rows] : czero<double>();
+        const c128 v = tri[q];
         Ui[r + 33 * c] = r == c ? (in ? s_inv[c] : czero<double>()) : r < c ? v : czero<double>();
         Li[r + 33 * c] = r == c ? mk<double>(in ? 1.0 : 0.0, 0.0) : r > c ? v : czero<double>();
     }
