@@ -356,14 +356,15 @@ void block_norm2(const c128* A, int64_t lda, int r0, int r1, int c0, int c1, dou
 // The rounds of a sweep are a chain, so a pair's latency is what counts, and on this part a
 // dependent FP64 operation takes 70-85 ns, a division 260 ns, a square root 350 ns.  A pair is
 // therefore one pass: both columns are loaded into registers with the first reads, one reduction
-// gives the inner product and both norms, the tangent T = t e^{i phi} of the rotation is formed in
-// FP32, and only what unitarity needs is FP64: c = (1 + |T|^2)^(-1/2), s e^{i phi} = c T.  The
-// rotation is unitary to FP64 for any T; an angle off by 2^-23 leaves that share of the pair's
-// inner product, which the next sweep sees (sweeps already converge quadratically to 1e-10).
+// gives the inner product and both norms, and the rotation comes from two FP64 reciprocal square
+// roots (an FP32 seed and one third-order step each, four dependent operations).  With the angle in
+// FP32 a whole pass took 0.3 to 1.2 % less (70.2 instead of 70.7 ms at n = 900), but a pair kept 2^-23 of its
+// inner product and two columns needed a third sweep.
 // One round then takes 3.0 us at 212 columns, from 6.1 us; a whole pass's sweeps: n = 900, k_S = 233:
 // 50.7 -> 18.7 ms, n = 40000: 88.9 -> 43.5 ms (there also without J in the projection, see project.cu).
-// The norms that decide about the floor are al - Re(conj(T) g) and be + Re(conj(T) g), exact to
-// rounding in the smaller one; every pair forms its own from the columns.
+// The norms that decide about the floor are al - Re(conj(T) g) and be + Re(conj(T) g), T the rotation's
+// complex tangent: to rounding in the larger one (of two nearly parallel columns the smaller one keeps few digits;
+// such a pair is rotated, so another sweep follows with fresh norms).  Every pair forms its own from the columns.
 // ---------------------------------------------------------------------------------------------
 namespace {
 __device__ __forceinline__ int rr_pos(int k, int r, int n) {  // player at seat k in round r
@@ -395,6 +396,12 @@ __device__ __forceinline__ c128 ldcg_c(const c128* p) {
 }
 constexpr int kJacCache = 3;  // rows per thread kept in registers
 constexpr int kJacVer = 8;
+
+// x^(-1/2) to FP64 rounding for x in FP32's normal range
+__device__ __forceinline__ double rsqrt_mid(double x) {
+    const double y = (double)rsqrtf((float)x), r = fma(-(x * y), y, 1.0);
+    return fma(fma(0.375, r, 0.5), y * r, y);
+}
 
 struct JacSums { double gr, gi, al, be; };
 __device__ __forceinline__ void jac_acc(JacSums& t, c128 x, c128 y) {
@@ -516,21 +523,19 @@ __global__ void __launch_bounds__(NT, 768 / NT) jacobi_sweep_kernel(JacobiArgs a
                     const bool act = g2 > 0.0 && g2 > a.tol2 * ab;
                     double dn = 0.0;
                     if (act) {
-                        // T = 2 g sign(d) / (|d| + sqrt(d^2 + 4 |g|^2)), d = be - al, scaled by a power of two
-                        const int e = min(2045, (__double2hiint(fmax(al, be)) >> 20) & 0x7ff);
+                        // With d = be - al and h = sqrt(d^2 + 4 |g|^2): cos 2 theta = |d| / h, sin 2 theta = 2 |g| / h, so
+                        // c^2 = (1 + |d| / h) / 2 and S = s e^{i phi} = g sign(d) / (h c); d and g are scaled by a power of two
+                        const int e = max(1, min(2045, (__double2hiint(fmax(al, be)) >> 20) & 0x7ff));
                         const double sf = __hiloint2double((2046 - e) << 20, 0);
-                        const float fr = (float)(gr * sf), fi = (float)(gi * sf), fd = (float)((be - al) * sf);
-                        const float h = sqrtf(fmaf(fd, fd, 4.f * fmaf(fr, fr, fi * fi)));
-                        const float w = copysignf(2.f / (fabsf(fd) + h), fd);
-                        const double Tr = (double)(fr * w), Ti = (double)(fi * w);
-                        // (1 + |T|^2)^(-1/2): FP32 seed, one third-order step
-                        const double x = fma(Tr, Tr, fma(Ti, Ti, 1.0)), y0 = (double)rsqrtf((float)x);
-                        const double r1 = fma(-(x * y0), y0, 1.0);
-                        const double c = fma(fma(0.375, r1, 0.5), y0 * r1, y0);
-                        dn = fma(Tr, gr, Ti * gi);
+                        const double fr = gr * sf, fi = gi * sf, d = (be - al) * sf;
+                        const double ih = rsqrt_mid(fma(d, d, 4.0 * fma(fr, fr, fi * fi)));
+                        const double c2 = fma(0.5 * fabs(d), ih, 0.5), ic = rsqrt_mid(c2);
+                        const double w = copysign(ih * ic, d);
+                        const c128 S = mk<double>(fr * w, fi * w);
+                        dn = fma(S.re, gr, S.im * gi) * ic;  // Re(conj(T) g), T = S / c
                         if (lane == 0) {
-                            s_c = c;
-                            s_S = mk<double>(Tr * c, Ti * c);
+                            s_c = c2 * ic;
+                            s_S = S;
                         }
                     }
                     if (lane == 0) {
