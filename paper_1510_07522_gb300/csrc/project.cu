@@ -16,7 +16,7 @@
 //      on the columns of R2^H gives R2^H J = U Sigma, and the left singular vectors of
 //      R_keep = R2^H Q2^H are the columns of U.
 //   3. S = Q [U(:, 1:k_S); 0] by applying the panels' reflectors in reverse, after one
-//      Newton-Schulz step on U(:, 1:k_S).
+//      Newton-Schulz step on U(:, 1:k_S) (a QR if the sweeps left them far from orthogonal).
 //   4. P_i = S^H (A_i S): CSR SpMM, then ZGEMM.
 #include <algorithm>
 #include <cmath>
@@ -250,10 +250,11 @@ __global__ void init_y_kernel(const c128* X, int kk, const int* cols, const doub
     Y[idx] = (r < kk) ? cscale(X[r + (int64_t)cols[c] * kk], 1.0 / nrm[cols[c]]) : czero<double>();
 }
 
-__global__ void identity_kernel(c128* J, int k) {
+// the first k columns of the identity of order m
+__global__ void identity_cols_kernel(c128* J, int m, int k) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)k * k) return;
-    J[idx] = (idx % k == idx / k) ? mk<double>(1.0, 0.0) : czero<double>();
+    if (idx >= (int64_t)m * k) return;
+    J[idx] = (idx % m == idx / m) ? mk<double>(1.0, 0.0) : czero<double>();
 }
 
 // Y_i = A_i X for every term (CSR of the union pattern with the term's values).  Products with a real
@@ -716,28 +717,48 @@ int project_run(rsrr_nep h, double delta) {
         CUDAC(cudaMemcpyAsync(cols_d, idx.data(), kS * 4, cudaMemcpyHostToDevice, st));
         TRYC(dalloc_n(&Ybuf, (size_t)n * kS, st));
         { init_y_kernel<<<(unsigned)ceil_div(n * kS, 256), 256, 0, st>>>(X, kk, cols_d, colnrm, kS, n, Ybuf); note_launch(); }
-        // The columns are orthogonal to 1e-10 (the sweeps' stopping level).  One Newton-Schulz step,
-        // U <- U (I - E / 2) with E = U^H U - I, makes them orthonormal to O(|E|^2) and leaves their
-        // span unchanged.
+        // The columns are orthogonal to 1e-10 (the sweeps' stopping level) unless the sweeps ran out or the
+        // matrix is so small (columns below 1e-77) that squared inner products underflow.  So E = U^H U - I
+        // is measured.  Small, one Newton-Schulz step, U <- U (I - E / 2), makes the columns orthonormal to
+        // O(|E|^2) and leaves their span unchanged; else they go through another QR.
         TRYC(dalloc_n(&Eg, (size_t)kS * kS, st));
-        { identity_kernel<<<(unsigned)ceil_div((int64_t)kS * kS, 256), 256, 0, st>>>(Eg, kS); note_launch(); }
+        { identity_cols_kernel<<<(unsigned)ceil_div((int64_t)kS * kS, 256), 256, 0, st>>>(Eg, kS, kS); note_launch(); }
         Zgemm ge;
         ge.opA = OP_C; ge.opB = OP_N; ge.M = kS; ge.N = kS; ge.K = kk;
         ge.beta = mk<double>(-1.0, 0.0);
         ge.A = Ybuf; ge.lda = n; ge.B = Ybuf; ge.ldb = n; ge.C = Eg; ge.ldc = kS;
         TRYC(zgemm(ge, st));
+        double e2 = 0.0;
+        CUDAC(cudaMemsetAsync(hw.dnorm, 0, 8, st));
+        block_norm2(Eg, kS, 0, kS, 0, kS, hw.dnorm, st);
+        CUDAC(cudaMemcpyAsync(&e2, hw.dnorm, 8, cudaMemcpyDeviceToHost, st));
+        CUDAC(cudaStreamSynchronize(st));
+        TRYC(dalloc_n(&Z, (size_t)kPB * kS, st));
+        TRYC(dalloc_n(&Z2, (size_t)kPB * kS, st));
         TRYC(dalloc_n(&Jn, (size_t)kk * kS, st));
         CUDAC(cudaMemcpy2DAsync(Jn, (size_t)kk * sizeof(c128), Ybuf, (size_t)n * sizeof(c128), (size_t)kk * sizeof(c128),
                                 kS, cudaMemcpyDeviceToDevice, st));
-        Zgemm gn;
-        gn.M = kk; gn.N = kS; gn.K = kS;
-        gn.alpha = mk<double>(-0.5, 0.0); gn.beta = mk<double>(1.0, 0.0);
-        gn.A = Ybuf; gn.lda = n; gn.B = Eg; gn.ldb = kS; gn.C = Jn; gn.ldc = kk;
-        TRYC(zgemm(gn, st));
+        if (e2 <= 1e-15) {
+            Zgemm gn;
+            gn.M = kk; gn.N = kS; gn.K = kS;
+            gn.alpha = mk<double>(-0.5, 0.0); gn.beta = mk<double>(1.0, 0.0);
+            gn.A = Ybuf; gn.lda = n; gn.B = Eg; gn.ldb = kS; gn.C = Jn; gn.ldc = kk;
+            TRYC(zgemm(gn, st));
+        } else {
+            HqrWork hu;
+            TRYC(hu.alloc(kk, kS, kS, st));
+            int ku = 0, nu = 0;
+            TRYC(householder_qr(Jn, kk, kS, kk, hu, nullptr, &ku, &nu));
+            c128* Qu = nullptr;  // kk x kS
+            TRYC(dalloc_n(&Qu, (size_t)kk * kS, st));
+            { identity_cols_kernel<<<(unsigned)ceil_div((int64_t)kk * kS, 256), 256, 0, st>>>(Qu, kk, kS); note_launch(); }
+            rc = apply_q(Jn, kk, nu, ku, hu, Qu, kS, Z, Z2, st);
+            std::swap(Jn, Qu);
+            dfree(Qu, st);
+            TRYC(rc);
+        }
         CUDAC(cudaMemcpy2DAsync(Ybuf, (size_t)n * sizeof(c128), Jn, (size_t)kk * sizeof(c128), (size_t)kk * sizeof(c128),
                                 kS, cudaMemcpyDeviceToDevice, st));
-        TRYC(dalloc_n(&Z, (size_t)kPB * kS, st));
-        TRYC(dalloc_n(&Z2, (size_t)kPB * kS, st));
         TRYC(apply_q(A, n, npan, kmax, hw, Ybuf, kS, Z, Z2, st));
         pc.mark();  // basis done
         if (h->tz) {  // no A_i: rsrr_project_chebyshev forms the reduced NEP from T(x_k)
@@ -958,7 +979,7 @@ int jacobi_svd_preconditioned(c128* H, int D, c128* Jr, cudaStream_t st, double 
     TRYR(householder_qr(A, D, D, D, hw, nullptr, &kk, &npan));
     // X = R^H, then the Jacobi with the rotations accumulated into Jr (used as J here)
     { rkeep_h_kernel<<<(unsigned)ceil_div(DD, 256), 256, 0, st>>>(A, D, D, D, X); note_launch(); }
-    { identity_kernel<<<(unsigned)ceil_div(DD, 256), 256, 0, st>>>(Jr, D); note_launch(); }
+    { identity_cols_kernel<<<(unsigned)ceil_div(DD, 256), 256, 0, st>>>(Jr, D, D); note_launch(); }
     TRYR(jacobi_orthogonalize(X, D, D, Jr, st, 40, sweeps, floor, conv));
     // left singular vectors Q J (in place of J), sigma_j = |W_j|, right vectors P W Sigma^{-1}
     TRYR(apply_q(A, D, npan, kk, hw, Jr, D, Z, Z2, st));
