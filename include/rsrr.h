@@ -420,6 +420,9 @@ int rsrr_band_solve_noalloc(int64_t n, int32_t kl, int32_t ku, double* ab_reim, 
  *   kind 1  an mbarrier wait on a phase that nothing arrives at: returns RSRR_ETIMEOUT
  *   kind 2  the same grid barrier over the CTAs there are: returns RSRR_OK
  *   kind 3  the same mbarrier wait after its one expected arrival: returns RSRR_OK
+ *   kind 4  no wait: a step fails with RSRR_ESINGULAR after the host has marked an earlier product
+ *           of the same call as given up: returns RSRR_ETIMEOUT
+ *   kind 5  the same step with no product marked: returns RSRR_ESINGULAR
  *   stream  cudaStream_t for the work (NULL = default); returns after it completes.
  * The device context stays usable after every kind.  Errors: EINVAL (kind), ENOMEM, ECUDA. */
 int rsrr_selftest_bounded_wait(int32_t kind, void* stream);

@@ -343,7 +343,8 @@ def rsrr_band_solve_noalloc(n, kl, ku, ab_ptr, L, b_ptr, stream=None):
 
 def rsrr_selftest_bounded_wait(kind, stream=None):
     """Run one bounded device wait made to run out (kind 0: grid barrier, 1: mbarrier) or to
-    complete (2, 3); raises RsrrError('ETIMEOUT') when the wait gave up."""
+    complete (2, 3); raises RsrrError('ETIMEOUT') when the wait gave up.  Kinds 4 and 5: a failing step
+    after a product that gave up (ETIMEOUT) or did not (ESINGULAR)."""
     _check(lib().rsrr_selftest_bounded_wait(int(kind), ctypes.c_void_p(stream) if stream else None))
 
 

@@ -24,7 +24,10 @@ int tz_values(rsrr_nep_s* h, const std::vector<zd>& z, c128** d_vals) {
         zr[2 * k] = z[k].real();
         zr[2 * k + 1] = z[k].imag();
     }
-    h->tz(h->tz_user, m, zr.data(), raw.data());
+    {
+        ZgemmNoDefer user_code;
+        h->tz(h->tz_user, m, zr.data(), raw.data());
+    }
     std::vector<c128> pv((size_t)m * nnz);
     for (int64_t k = 0; k < m; ++k)
         for (int64_t e = 0; e < nnz; ++e) {

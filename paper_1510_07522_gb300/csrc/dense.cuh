@@ -36,7 +36,9 @@ int zinv_batch(c128* X, int k, int batch, int32_t* info, cudaStream_t st);
 int zgemm_tc(const Zgemm& g, cudaStream_t s);
 // While one is alive (and begin() succeeded), the tensor-core ZGEMMs of this host thread do not wait
 // for their kernel: a bounded wait that gave up is recorded in one device word, which check() reads
-// after synchronising `st`.  The products must all run on `st`.  check() ends the deferral.
+// after synchronising `st`.  The products must all run on `st`.  check() ends the deferral.  A call that
+// fails before its check() passes its status through failed(): what it met may be a product that was
+// never written, so a recorded timeout takes the status's place.
 class ZgemmDefer {
   public:
     explicit ZgemmDefer(cudaStream_t s) : st(s) {}
@@ -45,12 +47,26 @@ class ZgemmDefer {
     ZgemmDefer& operator=(const ZgemmDefer&) = delete;
     int begin();
     int check();
+    int failed(int rc);
+    int* device_word() const { return word; }
 
   private:
     cudaStream_t st;
     int* word = nullptr;
     int* outer = nullptr;  // the deferral that was in force before this one
     bool on = false;
+};
+// Suspends the deferral while user code runs on this host thread: products that a callback asks for have
+// their own stream and wait for themselves.
+class ZgemmNoDefer {
+  public:
+    ZgemmNoDefer();
+    ~ZgemmNoDefer();
+    ZgemmNoDefer(const ZgemmNoDefer&) = delete;
+    ZgemmNoDefer& operator=(const ZgemmNoDefer&) = delete;
+
+  private:
+    int* outer;
 };
 bool zgemm_tc_fits(const Zgemm& g);
 void zgemm_set_path(int path);

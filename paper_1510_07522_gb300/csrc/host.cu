@@ -7,6 +7,7 @@
 #include <numeric>
 #include <queue>
 
+#include "dense.cuh"
 #include "internal.h"
 
 namespace rsrr {
@@ -101,6 +102,7 @@ void eval_fn(const rsrr_fn& f, zd z, zd* val, zd* deriv) {
         case RSRR_F_CALLBACK: {
             const double zr[2] = {z.real(), z.imag()};
             double fr[2] = {0.0, 0.0}, dr[2] = {0.0, 0.0};
+            ZgemmNoDefer user_code;
             f.cb(f.user, 1, zr, fr, dr);
             *val = zd(fr[0], fr[1]);
             *deriv = zd(dr[0], dr[1]);

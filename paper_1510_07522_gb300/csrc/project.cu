@@ -532,7 +532,8 @@ struct PhaseClock {  // device time between successive marks on one stream
 };
 }  // namespace
 
-int project_run(rsrr_nep h, double delta) {
+namespace {
+int project_body(rsrr_nep h, double delta, ZgemmDefer& defer) {
     cudaStream_t st = h->stream;
     PhaseClock pc(st);
     pc.mark();
@@ -556,8 +557,6 @@ int project_run(rsrr_nep h, double delta) {
     double* colnrm = nullptr;
     int *order_d = nullptr, *cols_d = nullptr;
     int rc = RSRR_OK;
-    ZgemmDefer defer(st);
-    RSRR_TRY(defer.begin());
     auto cleanup = [&]() {
         double zm, zf;
         zgemm_profile_end(&zm, &zf);
@@ -796,6 +795,14 @@ int project_run(rsrr_nep h, double delta) {
 #undef TRYC
 #undef CUDAC
     return RSRR_OK;
+}
+}  // namespace
+
+int project_run(rsrr_nep h, double delta) {
+    ZgemmDefer defer(h->stream);
+    RSRR_TRY(defer.begin());
+    const int rc = project_body(h, delta, defer);
+    return rc == RSRR_OK ? rc : defer.failed(rc);
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -435,8 +435,9 @@ int alloc_zero(c128** p, size_t n, cudaStream_t s) {
 
 }  // namespace
 
-int solve_run(rsrr_nep h, int N_S, int K, double tol_gap, int cap, double* lambda_reim, double* V_reim,
-              double* resid, int32_t* nC_out) {
+namespace {
+int solve_body(rsrr_nep h, int N_S, int K, double tol_gap, int cap, double* lambda_reim, double* V_reim,
+               double* resid, int32_t* nC_out, ZgemmDefer& defer) {
     cudaStream_t st = h->stream;
     cudaEvent_t ev[4];
     for (auto& e : ev) cudaEventCreate(&e);
@@ -452,8 +453,6 @@ int solve_run(rsrr_nep h, int N_S, int K, double tol_gap, int cap, double* lambd
             jacobi_profile_end(&h->ms_jacobi_solve, &h->jacobi_flops_solve);
         }
     } zpg{h};
-    ZgemmDefer defer(st);
-    RSRR_TRY(defer.begin());
     // J, fns: the reduced NEP's terms (T's own, or Chebyshev polynomials); the final residual
     // uses T itself (h->J, h->fns, the CSR values)
     const int k = h->kS, J = h->red_J;
@@ -829,7 +828,7 @@ int solve_run(rsrr_nep h, int N_S, int K, double tol_gap, int cap, double* lambd
             hv.resize((size_t)n * nk);
             CUDAC(cudaMemcpyAsync(hv.data(), Vfull, hv.size() * sizeof(c128), cudaMemcpyDeviceToHost, st));
         }
-        CUDAC(cudaStreamSynchronize(st));
+        TRYC(defer.check());  // no product follows; nothing has reached the caller's arrays yet
         for (int t = 0; t < nk; ++t) {
             lambda_reim[2 * t] = lk[t].real();
             lambda_reim[2 * t + 1] = lk[t].imag();
@@ -843,8 +842,9 @@ int solve_run(rsrr_nep h, int N_S, int K, double tol_gap, int cap, double* lambd
                 }
         }
     }
+    if (nk == 0) TRYC(defer.check());
     cudaEventRecord(ev[3], st);
-    TRYC(defer.check());
+    CUDAC(cudaEventSynchronize(ev[3]));
     for (int i = 0; i < 3; ++i) {
         float t = 0.f;
         cudaEventElapsedTime(&t, ev[i], ev[i + 1]);
@@ -854,6 +854,18 @@ int solve_run(rsrr_nep h, int N_S, int K, double tol_gap, int cap, double* lambd
 #undef TRYC
 #undef CUDAC
     return RSRR_OK;
+}
+
+}  // namespace
+
+int solve_run(rsrr_nep h, int N_S, int K, double tol_gap, int cap, double* lambda_reim, double* V_reim,
+              double* resid, int32_t* nC_out) {
+    ZgemmDefer defer(h->stream);
+    RSRR_TRY(defer.begin());
+    int rc = solve_body(h, N_S, K, tol_gap, cap, lambda_reim, V_reim, resid, nC_out, defer);
+    if (rc != RSRR_OK) rc = defer.failed(rc);
+    if (rc == RSRR_ETIMEOUT) *nC_out = 0;
+    return rc;
 }
 
 }  // namespace rsrr

@@ -41,8 +41,15 @@ __global__ void selftest_mbar_kernel(int arrive, uint32_t limit, int* result) {
 using namespace rsrr;
 
 extern "C" int rsrr_selftest_bounded_wait(int32_t kind, void* stream) {
-    if (kind < 0 || kind > 3) return set_error(RSRR_EINVAL, "rsrr_selftest_bounded_wait: kind is 0..3");
+    if (kind < 0 || kind > 5) return set_error(RSRR_EINVAL, "rsrr_selftest_bounded_wait: kind is 0..5");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (kind >= 4) {  // a call that fails while its products' error word is set, or is clear
+        ZgemmDefer defer(st);
+        RSRR_TRY(defer.begin());
+        if (kind == 4 && cudaMemsetAsync(defer.device_word(), 1, 4, st) != cudaSuccess)
+            return set_error(RSRR_ECUDA, "rsrr_selftest_bounded_wait: memset");
+        return defer.failed(set_error(RSRR_ESINGULAR, "rsrr_selftest_bounded_wait: the failing step"));
+    }
     constexpr int kCtas = 2;
     unsigned* bar = nullptr;
     int* result = nullptr;

@@ -632,6 +632,18 @@ int ZgemmDefer::check() {
     RSRR_CUDA(cudaStreamSynchronize(st));
     return herr ? set_error(RSRR_ETIMEOUT, "tensor-core ZGEMM: a bounded wait gave up") : RSRR_OK;
 }
+int ZgemmDefer::failed(int rc) {
+    if (!on) return rc;  // check() has spoken
+    t_defer = outer;
+    on = false;
+    int herr = 0;
+    if (cudaMemcpyAsync(&herr, word, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess || !herr)
+        return rc;
+    return set_error(RSRR_ETIMEOUT, "tensor-core ZGEMM: a bounded wait gave up");
+}
+ZgemmNoDefer::ZgemmNoDefer() : outer(t_defer) { t_defer = nullptr; }
+ZgemmNoDefer::~ZgemmNoDefer() { t_defer = outer; }
 
 int zgemm_tc(const Zgemm& g0, cudaStream_t s) {
     Zgemm g = g0;
