@@ -86,6 +86,7 @@ constexpr size_t factor_smem() {
 struct DShared {
     uint64_t cbar;      // the cluster's barrier: one arrival per CTA
     int cok;
+    int cabort;         // a CTA of the cluster has given up
     double2 u12[32 * 32];  // U12 of the panel's left leaf (32 x 32, complex64 or complex128)
     int piv[NB];        // panel pivots, relative to the panel's first row
     int rows[2 * NB];   // composed interchanges: row rows[e] receives row src[e]
@@ -104,12 +105,20 @@ struct Cluster {
     int rank = 0, size = 1;
     uint32_t phase = 0;
     bool fail = false;
+    unsigned long long polls = 0;  // of one wait (dense_wait_polls)
 };
+
+// The CTA gives up: the others of the cluster leave their waits too.
+__device__ __forceinline__ void cluster_fail(Cluster& c, DShared& sh) {
+    if (!c.fail && (int)threadIdx.x < c.size) *(volatile int*)cg::this_cluster().map_shared_rank(&sh.cabort, threadIdx.x) = 1;
+    c.fail = true;
+}
 
 // Barrier of all workers of the cluster, ordering their global and shared memory accesses.  The
 // hardware cluster barrier counts every thread, and the tensor-core producer warp takes no part, so the
-// CTAs arrive on one another's mbarrier.  Bounded: when a wait gives up, `fail` is set and no
-// later one is entered (the other CTAs then run out of arrivals and give up too).
+// CTAs arrive on one another's mbarrier.  Bounded by what another CTA may do in between
+// (dense_wait_polls): when a wait gives up, `fail` is set here, no later one is entered, and the other CTAs'
+// waits end at once.
 __device__ __forceinline__ bool csync(Cluster& c, DShared& sh) {
     wsync();
     if (c.size == 1 || c.fail) return !c.fail;
@@ -121,17 +130,20 @@ __device__ __forceinline__ bool csync(Cluster& c, DShared& sh) {
     }
     if (threadIdx.x == 0) {
         uint32_t done = 0;
-        for (uint32_t it = 0; it < (1u << 21) && !done; ++it) {
+        for (unsigned long long it = 0; it < c.polls && !done; ++it) {
             asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
                          " selp.u32 %0, 1, 0, p;\n}\n" : "=r"(done) : "r"(smem_u32(&sh.cbar)), "r"(c.phase) : "memory");
-            if (!done && it > 4096) __nanosleep(64);
+            if (!done && it > 4096) {
+                __nanosleep(64);
+                if ((it & 63) == 0 && *(volatile int*)&sh.cabort) break;
+            }
         }
         __threadfence();
         sh.cok = (int)done;
     }
     wsync();
     c.phase ^= 1;
-    if (!sh.cok) c.fail = true;
+    if (!sh.cok) cluster_fail(c, sh);
     return !c.fail;
 }
 
@@ -947,7 +959,7 @@ __device__ void factor_one(const DenseJob<R>& J, cplx<R>* sm, DShared& sh, float
                 trailing_update_tc(A, lda, n, k0, img, img + img_b, *ts, *ph);
                 if (ts->stop) {  // uniform: written by thread 0 between two worker barriers
                     sh.info = -1;
-                    cl.fail = true;
+                    cluster_fail(cl, sh);
                     break;
                 }
             } else {
@@ -1327,8 +1339,10 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? NT + 32 : NT, 1)
     Cluster cl;
     cl.rank = (int)cluster.block_rank();
     cl.size = (int)cluster.num_blocks();
+    cl.polls = dense_wait_polls(n_max, (L_max + cl.size - 1) / cl.size);
     if (threadIdx.x == 0) {
         mbar_init(&sh.cbar, (uint32_t)cl.size);
+        sh.cabort = 0;
         ts.rank = cl.rank;
         ts.size = cl.size;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");

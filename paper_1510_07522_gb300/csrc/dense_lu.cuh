@@ -33,6 +33,16 @@ constexpr int kDenseSwapInts = 1 + 4 * kDenseNB;
 
 __host__ __device__ inline int64_t dense_panels(int64_t n) { return (n + kDenseNB - 1) / kDenseNB; }
 
+// Polls after which a CTA that waits for the others of its cluster gives up.  A poll that fails takes
+// 3.8 us (the hardware suspends the thread; 1 us is counted on).  Between two barriers one CTA may do what the
+// others wait for: a triangular solve of `cols` columns (n^2 entries, 1.1 ns an entry and column at the
+// FP64 rate), or the 64 columns of a panel too tall for shared memory (3 us a row).  The limit is a floor
+// of 2^21 (8 s) and about eight times that work; the floor alone would end a healthy FP64 solve of 8
+// columns a CTA from n = 30000 on.
+__host__ __device__ inline unsigned long long dense_wait_polls(int64_t n, int64_t cols) {
+    return (1ull << 21) + (unsigned long long)(n * n / 128 * cols + 32 * n);
+}
+
 // The factor and solve of one point (one cluster's slot).
 template <typename R>
 struct DenseJob {
