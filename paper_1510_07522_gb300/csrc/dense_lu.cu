@@ -1119,7 +1119,7 @@ struct Slot {
     cplx<R>* inv;
     int32_t* swaps;
     double* colsum;
-    c128* tv;      // T(z_j) on the CSR pattern
+    c128* tv;      // T(z_j) on the CSR pattern, or null
     double* part;  // [kMaxCluster][2][L] the CTAs' shares of the residual's sums
 };
 
@@ -1151,7 +1151,7 @@ __device__ Slot<R> slot_at(unsigned char* base, int n_max, int L_max, int64_t nn
     p += align256(np * kDenseSwapInts * 4);
     t.colsum = reinterpret_cast<double*>(p);
     p += align256((size_t)n_max * 8);
-    t.tv = reinterpret_cast<c128*>(p);
+    t.tv = nnz_max > 0 ? reinterpret_cast<c128*>(p) : nullptr;
     p += align256((size_t)nnz_max * sizeof(c128));
     t.part = reinterpret_cast<double*>(p);
     return t;
@@ -1168,12 +1168,12 @@ __device__ double worker_max(double v, SampleShared& ss) {
     return m;
 }
 
-// r = U - T X (FP64, T's CSR values tv); x = r in precision R; per-column ||r||^2 and ||X||^2 into
+// r = U - T X (FP64, T's CSR values tv if KEPT, else formed from the terms); x = r in precision R; per-column ||r||^2 and ||X||^2 into
 // ss.rn2 / ss.xn2 (this CTA's rows only).  A warp takes a row: lane = (column of a group of 8, one of 4 entries), so that no
 // lane idles; the FP64 rate bounds it (two multiply-adds a clock: 1 ms for 132000 entries and 8
 // columns, where a thread a row and T formed anew from its terms took 2.7 ms).
-template <typename R>
-__device__ void residual_one(const DenseNep& E, const c128* X, const c128* tv, cplx<R>* x, SampleShared& ss,
+template <typename R, bool KEPT>
+__device__ void residual_one(const DenseNep& E, int j, const c128* X, const c128* tv, cplx<R>* x, SampleShared& ss,
                              const Cluster& cl) {
     const int n = E.n, L = E.L, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane >> 3;
     for (int l = threadIdx.x; l < L; l += NT) ss.rn2[l] = ss.xn2[l] = 0.0;
@@ -1186,8 +1186,17 @@ __device__ void residual_one(const DenseNep& E, const c128* X, const c128* tv, c
         for (int r = cl.rank * NW + warp; r < n; r += cl.size * NW) {
             const int64_t end = E.rowptr[r + 1];
             c128 acc = czero<double>();
+            if constexpr (KEPT) {
 #pragma unroll 4
-            for (int64_t k = E.rowptr[r] + sub; k < end; k += 4) cfma(acc, tv[k], Xl[E.colind[k]]);
+                for (int64_t k = E.rowptr[r] + sub; k < end; k += 4) cfma(acc, tv[k], Xl[E.colind[k]]);
+            } else {
+                const c128* f = E.F + (int64_t)j * E.J;
+                for (int64_t k = E.rowptr[r] + sub; k < end; k += 4) {
+                    c128 t = czero<double>();
+                    for (int i = 0; i < E.J; ++i) cfma(t, f[i], E.vals[(int64_t)i * E.nnz + k]);
+                    cfma(acc, t, Xl[E.colind[k]]);
+                }
+            }
 #pragma unroll
             for (int off = 8; off <= 16; off <<= 1) {
                 acc.re += __shfl_xor_sync(FULL, acc.re, off);
@@ -1208,7 +1217,7 @@ __device__ void residual_one(const DenseNep& E, const c128* X, const c128* tv, c
     wsync();
 }
 
-template <typename R>
+template <typename R, bool KEPT>
 __device__ void sample_one(const DenseNep& E, int j, const Slot<R>& sl, cplx<R>* sm, DShared& sh, SampleShared& ss,
                            float* img, size_t img_b, TcShared* ts, TcPhase* ph, const DenseSampleCfg& cfg, Cluster& cl) {
     const int n = E.n, L = E.L, J = E.J;
@@ -1234,7 +1243,7 @@ __device__ void sample_one(const DenseNep& E, int j, const Slot<R>& sl, cplx<R>*
         for (int64_t k = gtid; k < nnz; k += gstep) {
             c128 t = czero<double>();
             for (int i = 0; i < J; ++i) cfma(t, f[i], E.vals[(int64_t)i * nnz + k]);
-            sl.tv[k] = t;
+            if constexpr (KEPT) sl.tv[k] = t;
             const int c = E.colind[k];
             A[E.rowidx[k] + (int64_t)c * n] = ccast<R>(t);
             atomicAdd(&sl.colsum[c], sqrt(cnorm2(t)));
@@ -1277,7 +1286,7 @@ __device__ void sample_one(const DenseNep& E, int j, const Slot<R>& sl, cplx<R>*
     int sweeps = 0;
     for (;;) {
         if (!csync(cl, sh)) return failed_wait();  // every column of X is there
-        residual_one(E, X, sl.tv, sl.x, ss, cl);
+        residual_one<R, KEPT>(E, j, X, sl.tv, sl.x, ss, cl);
         for (int l = threadIdx.x; l < L; l += NT) {
             sl.part[(2 * cl.rank) * L + l] = ss.rn2[l];
             sl.part[(2 * cl.rank + 1) * L + l] = ss.xn2[l];
@@ -1323,7 +1332,8 @@ __device__ void sample_one(const DenseNep& E, int j, const Slot<R>& sl, cplx<R>*
     wsync();
 }
 
-template <typename R>
+// KEPT: the slots hold T's values (a kernel of its own: as a branch, the other residual cost a batch 1 to 2 %)
+template <typename R, bool KEPT>
 __global__ void __launch_bounds__(sizeof(R) == 4 ? NT + 32 : NT, 1)
     dense_sample_kernel(const DenseNep* __restrict__ neps, const DenseSampleJob* __restrict__ jobs, int njobs,
                         int n_max, int L_max, int64_t nnz_max, unsigned char* slots, size_t slot_stride, float* img, size_t img_stride,
@@ -1380,7 +1390,7 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? NT + 32 : NT, 1)
             const int jb = sh.job;
             if (jb >= njobs) break;
             const DenseSampleJob job = jobs[jb];
-            sample_one<R>(neps[job.nep], job.j, sl, sm, sh, ss, my_img, img_b, &ts, &ph, cfg, cl);
+            sample_one<R, KEPT>(neps[job.nep], job.j, sl, sm, sh, ss, my_img, img_b, &ts, &ph, cfg, cl);
         }
         if (tc && threadIdx.x == 0) {
             ts.cmd = 2;
@@ -1428,16 +1438,43 @@ int sm_count() {
 
 }  // namespace
 
+namespace {
+template <typename R>
+cudaLaunchConfig_t sample_config(int clusters, int cluster_size, cudaLaunchAttribute* at, cudaStream_t s) {
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)(clusters * cluster_size));
+    lc.blockDim = dim3((unsigned)(sizeof(R) == 4 ? NT + 32 : NT));
+    lc.dynamicSmemBytes = std::max(factor_smem<R>(), solve_smem<R>());
+    lc.stream = s;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = (unsigned)cluster_size;
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    return lc;
+}
+}  // namespace
+
 // Cluster size and count for jobs of orders n (descending): the size whose greedy schedule of the
 // jobs ends first.  A point's time is taken as n^2 (s + (1 - s) / size): CTA 0's panels are serial, the
-// rest is shared; no more CTAs than the largest matrix has panels.
-void dense_plan(const std::vector<int>& n, int* size, int* count) {
-    const int nsm = sm_count();
+// rest is shared; no more CTAs than the largest matrix has panels, and no more clusters than there are
+// slots or than the device holds at once (of 4 CTAs with 200 KB each 36 fit, of 8 CTAs 15).
+template <typename R>
+int dense_plan(const std::vector<int>& n, int slots, int* size, int* count) {
+    RSRR_TRY(set_smem(dense_sample_kernel<R, true>, std::max(factor_smem<R>(), solve_smem<R>()), "dense_sample_kernel"));
     double best = 0.0;
     *size = 1;
     *count = 1;
     for (int c = 1; c <= kMaxCluster && (c == 1 || c * NB <= n.front()); c *= 2) {
-        const int m = std::max(1, std::min((int)n.size(), nsm / c));
+        int fit = sm_count();
+        if (c > 1) {
+            cudaLaunchAttribute at[1];
+            const cudaLaunchConfig_t lc = sample_config<R>(1, c, at, nullptr);
+            if (cudaOccupancyMaxActiveClusters(&fit, dense_sample_kernel<R, true>, &lc) != cudaSuccess) fit = 0;
+            cudaGetLastError();
+            if (fit < 1) break;
+        }
+        const int m = std::max(1, std::min({(int)n.size(), fit, slots}));
         std::priority_queue<double, std::vector<double>, std::greater<double>> busy;
         for (int i = 0; i < m; ++i) busy.push(0.0);
         double end = 0.0;
@@ -1453,6 +1490,7 @@ void dense_plan(const std::vector<int>& n, int* size, int* count) {
             *count = m;
         }
     }
+    return RSRR_OK;
 }
 
 template <typename R>
@@ -1474,23 +1512,14 @@ int launch_dense_sample(const DenseNep* d_neps, const DenseSampleJob* d_jobs, in
     if (L_max > kMaxL) return set_error(RSRR_EINVAL, "dense sampling: L above 256");
     if (sizeof(R) == 4 && !d_img) return set_error(RSRR_EINVAL, "dense sampling: operand images missing");
     const size_t sm = std::max(factor_smem<R>(), solve_smem<R>());
-    RSRR_TRY(set_smem(dense_sample_kernel<R>, sm, "dense_sample_kernel"));
+    auto kernel = nnz_max > 0 ? dense_sample_kernel<R, true> : dense_sample_kernel<R, false>;
+    RSRR_TRY(set_smem(kernel, sm, "dense_sample_kernel"));
     RSRR_CUDA(cudaMemsetAsync(d_next, 0, sizeof(int32_t), s));
-    const int threads = sizeof(R) == 4 ? NT + 32 : NT;
     const size_t img_stride = dense_image_bytes<R>(n_max) / 4;
     const size_t img_b = sizeof(R) == 4 ? (size_t)((n_max + TC_ROWS - 1) / TC_ROWS) * TC_A_FLOATS : 0;
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3((unsigned)(clusters * cluster_size));
-    lc.blockDim = dim3((unsigned)threads);
-    lc.dynamicSmemBytes = sm;
-    lc.stream = s;
     cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)cluster_size;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    lc.attrs = at;
-    lc.numAttrs = 1;
-    RSRR_CUDA(cudaLaunchKernelEx(&lc, dense_sample_kernel<R>, d_neps, d_jobs, njobs, n_max, L_max, nnz_max,
+    const cudaLaunchConfig_t lc = sample_config<R>(clusters, cluster_size, at, s);
+    RSRR_CUDA(cudaLaunchKernelEx(&lc, kernel, d_neps, d_jobs, njobs, n_max, L_max, nnz_max,
                                  static_cast<unsigned char*>(d_slots), dense_slot_bytes<R>(n_max, L_max, nnz_max),
                                  static_cast<float*>(d_img), img_stride, img_b, d_next, cfg));
     note_launch();
@@ -1498,6 +1527,8 @@ int launch_dense_sample(const DenseNep* d_neps, const DenseSampleJob* d_jobs, in
     return RSRR_OK;
 }
 
+template int dense_plan<float>(const std::vector<int>&, int, int*, int*);
+template int dense_plan<double>(const std::vector<int>&, int, int*, int*);
 template size_t dense_slot_bytes<float>(int, int, int64_t);
 template size_t dense_slot_bytes<double>(int, int, int64_t);
 template size_t dense_image_bytes<float>(int);

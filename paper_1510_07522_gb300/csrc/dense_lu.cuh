@@ -85,11 +85,13 @@ struct DenseSampleCfg {
     int32_t max_refine;
 };
 
-// Device bytes of one cluster's slot for n <= n_max, L <= L_max, nnz <= nnz_max.
+// Device bytes of one cluster's slot for n <= n_max, L <= L_max, nnz <= nnz_max; with nnz_max = 0 it does not
+// keep T's values and the residuals form T from its terms.
 template <typename R>
 size_t dense_slot_bytes(int n_max, int L_max, int64_t nnz_max);
-// Cluster size (CTAs per point) and number of clusters for jobs of orders n (descending).
-void dense_plan(const std::vector<int>& n, int* size, int* count);
+// Cluster size (CTAs per point) and number of clusters, `slots` at most, for jobs of orders n (descending).
+template <typename R>
+int dense_plan(const std::vector<int>& n, int slots, int* size, int* count);
 // Device bytes of one cluster's tensor-core operand images (complex64; 0 for complex128).
 template <typename R>
 size_t dense_image_bytes(int n_max);

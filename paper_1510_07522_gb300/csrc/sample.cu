@@ -528,14 +528,18 @@ int sample_dense_set(const std::vector<rsrr_nep>& hs, const std::vector<c128*>& 
     // memory holds
     size_t free_b = 0, total_b = 0;
     RSRR_CUDA(cudaMemGetInfo(&free_b, &total_b));
-    const size_t per_slot = dense_slot_bytes<R>(n_max, L_max, nnz_max) + dense_image_bytes<R>(n_max);
     const size_t budget = (size_t)(0.8 * (double)free_b);
+    auto slots_of = [&](int64_t nnz) {
+        return (int)std::min<size_t>((size_t)njobs, budget / (dense_slot_bytes<R>(n_max, L_max, nnz) + dense_image_bytes<R>(n_max)));
+    };
+    if (slots_of(0) < 1) return set_error(RSRR_ENOMEM, "one dense sampling slot does not fit in device memory");
     std::vector<int> job_n(jobs.size());
     for (size_t i = 0; i < jobs.size(); ++i) job_n[i] = (int)hs[jobs[i].nep]->n;
-    int csize = 1, ccount = 1;
-    dense_plan(job_n, &csize, &ccount);
-    const int grid = (int)std::min<size_t>((size_t)ccount, budget / per_slot);
-    if (grid < 1) return set_error(RSRR_ENOMEM, "one dense sampling slot does not fit in device memory");
+    int csize = 1, grid = 1;
+    RSRR_TRY(dense_plan<R>(job_n, slots_of(0), &csize, &grid));
+    // A slot keeps T's values for the residuals (a full pattern makes it three times as large) only where that
+    // costs no cluster.
+    if (slots_of(nnz_max) < grid) nnz_max = 0;
 
     std::vector<DenseNep> neps(nh);
     std::vector<double*> un2(nh, nullptr);
