@@ -648,7 +648,8 @@ int launch_factor(const FactorArgs<R>& a, int npts, cudaStream_t s) {
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (2 * npts <= nsm) {  // few points: several SMs per point
+    const int pts = std::max(npts, a.plan);
+    if (2 * pts <= nsm) {  // few points: several SMs per point
         RSRR_TRY(set_smem(band_factor_cluster_kernel<R>, sm, "band_factor_cluster_kernel"));
         cudaLaunchConfig_t cfg = {};
         cfg.blockDim = dim3(kLuThreads, 1, 1);
@@ -665,12 +666,12 @@ int launch_factor(const FactorArgs<R>& a, int npts, cudaStream_t s) {
         // otherwise.
         constexpr int CG = BandTraits<R>::CG;
         const int rest = std::max(0, (std::min(a.d.kv, a.d.n) + CG - 1) / CG - (a.d.nb + CG - 1) / CG);
-        int C = std::max(2, std::min({4, nsm / npts, 1 + (rest + kLuThreads / 32 - 1) / (kLuThreads / 32)}));
+        int C = std::max(2, std::min({4, nsm / pts, 1 + (rest + kLuThreads / 32 - 1) / (kLuThreads / 32)}));
         for (; C > 2; --C) {
             attr[0].val.clusterDim.x = C;
-            cfg.gridDim = dim3(C * npts, 1, 1);
+            cfg.gridDim = dim3(C * pts, 1, 1);
             int fit = 0;
-            if (cudaOccupancyMaxActiveClusters(&fit, band_factor_cluster_kernel<R>, &cfg) == cudaSuccess && fit >= npts) break;
+            if (cudaOccupancyMaxActiveClusters(&fit, band_factor_cluster_kernel<R>, &cfg) == cudaSuccess && fit >= pts) break;
             cudaGetLastError();
         }
         attr[0].val.clusterDim.x = C;
@@ -690,7 +691,7 @@ int launch_fwd(const SolveArgs<R>& a, int npts, cudaStream_t s) {
     const size_t sm = fwd_smem_bytes<R>(a.d, a.d.fwd_nbuf);
     RSRR_TRY(set_smem(band_fwd_kernel<R>, sm, "band_fwd_kernel"));
     SolveArgs<R> b = a;
-    b.split = solve_split(npts, a.L);
+    b.split = solve_split(std::max(npts, a.plan), a.L);
     { band_fwd_kernel<R><<<npts * b.split, kSolveThreads, sm, s>>>(b); note_launch(); }
     RSRR_CUDA(cudaGetLastError());
     return RSRR_OK;
@@ -701,7 +702,7 @@ int launch_bwd(const SolveArgs<R>& a, int npts, cudaStream_t s) {
     const size_t sm = bwd_smem_bytes<R>(a.d, a.d.bwd_nbuf);
     RSRR_TRY(set_smem(band_bwd_kernel<R>, sm, "band_bwd_kernel"));
     SolveArgs<R> b = a;
-    b.split = solve_split(npts, a.L);
+    b.split = solve_split(std::max(npts, a.plan), a.L);
     { band_bwd_kernel<R><<<npts * b.split, kSolveThreads, sm, s>>>(b); note_launch(); }
     RSRR_CUDA(cudaGetLastError());
     return RSRR_OK;

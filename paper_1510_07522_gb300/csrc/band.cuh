@@ -39,6 +39,7 @@ struct FactorArgs {
     int64_t perm_stride;
     int32_t* ipiv;   // [pts][n]
     int32_t* info;   // [pts] first zero pivot column (1-based), 0 if none
+    int plan = 0;    // CTAs a point are chosen as for this many points, where that is more than the launch's
 };
 
 template <typename R>
@@ -55,6 +56,7 @@ struct SolveArgs {
     int L;
     const int32_t* active;  // [pts] 0 = skip this point (already converged); may be null
     int split = 1;          // CTAs per point; CTA r of a point takes a contiguous share of the columns
+    int plan = 0;           // as in FactorArgs
 };
 
 template <typename R> struct BandTraits;

@@ -1031,7 +1031,7 @@ int launch_bwd_tc(const SolveArgs<float>& a, int npts, cudaStream_t s) {
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    b.split = std::max((a.L + kBwdCols - 1) / kBwdCols, std::min(nsm / std::max(npts, 1), (a.L + 3) / 4));
+    b.split = std::max((a.L + kBwdCols - 1) / kBwdCols, std::min(nsm / std::max({npts, a.plan, 1}), (a.L + 3) / 4));
     const int cols = (a.L + b.split - 1) / b.split;
     if (cols <= 4) return launch_bwd_tc_groups<1>(map, b, npts, s);
     if (cols <= 8) return launch_bwd_tc_groups<2>(map, b, npts, s);
@@ -1043,7 +1043,7 @@ int launch_fwd_tc(const SolveArgs<float>& a, int npts, cudaStream_t s) {
     const size_t sm = (size_t)2 * P_BYTES + (size_t)2 * NB * 32 * sizeof(c64) + (size_t)2 * LDP * 4;
     RSRR_TRY(set_smem_max(band_fwd_tc_kernel, sm, "band_fwd_tc_kernel"));
     SolveArgs<float> b = a;
-    b.split = a.L > 32 ? 2 : solve_split_tc(npts, a.L);
+    b.split = a.L > 32 ? 2 : solve_split_tc(std::max(npts, a.plan), a.L);
     if ((a.L + b.split - 1) / b.split > 32) return set_error(RSRR_EINVAL, "launch_fwd_tc: too many columns per CTA");
     band_fwd_tc_kernel<<<npts * b.split, kFwdThreads, sm, s>>>(b);
     note_launch();

@@ -389,7 +389,6 @@ __device__ void compose_swaps(int nbk, const int* piv, DShared& sh) {
 // to the panel's other columns, and the columns right of it get their U rows and the rank-lw update.
 // The panel's columns cross L2 twice a leaf and column to its right (96 column passes for 64 columns),
 // against 1024 when every column of a 32-column leaf updated the others in global memory.
-constexpr double kDenseSerial = 0.25;  // share of a point's time in its panels (dense_plan)
 constexpr int kLeafMax = 16;
 template <typename R>
 __device__ void panel_factor_tall(cplx<R>* P, int64_t ld, int m, int nbk, int lw, int col_base, cplx<R>* sm,
@@ -1456,8 +1455,7 @@ cudaLaunchConfig_t sample_config(int clusters, int cluster_size, cudaLaunchAttri
 }  // namespace
 
 // Cluster size and count for jobs of orders n (descending): the size whose greedy schedule of the
-// jobs ends first.  A point's time is taken as n^2 (s + (1 - s) / size): CTA 0's panels are serial, the
-// rest is shared; no more CTAs than the largest matrix has panels, and no more clusters than there are
+// jobs ends first.  A point's time is taken as n^2 dense_time_share(size); no more CTAs than the largest matrix has panels, and no more clusters than there are
 // slots or than the device holds at once (of 4 CTAs with 200 KB each 36 fit, of 8 CTAs 15).
 template <typename R>
 int dense_plan(const std::vector<int>& n, int slots, int* size, int* count) {
@@ -1479,7 +1477,7 @@ int dense_plan(const std::vector<int>& n, int slots, int* size, int* count) {
         for (int i = 0; i < m; ++i) busy.push(0.0);
         double end = 0.0;
         for (int x : n) {
-            const double t = busy.top() + (double)x * x * (kDenseSerial + (1.0 - kDenseSerial) / c);
+            const double t = busy.top() + (double)x * x * dense_time_share(c);
             busy.pop();
             busy.push(t);
             end = std::max(end, t);

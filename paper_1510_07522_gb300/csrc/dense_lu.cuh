@@ -92,6 +92,8 @@ size_t dense_slot_bytes(int n_max, int L_max, int64_t nnz_max);
 // Cluster size (CTAs per point) and number of clusters, `slots` at most, for jobs of orders n (descending).
 template <typename R>
 int dense_plan(const std::vector<int>& n, int slots, int* size, int* count);
+// Time of a point on a cluster of `size` CTAs against one CTA's: the panels (a quarter of it) are one CTA's work.
+inline double dense_time_share(int size) { return 0.25 + 0.75 / size; }
 // Device bytes of one cluster's tensor-core operand images (complex64; 0 for complex128).
 template <typename R>
 size_t dense_image_bytes(int n_max);

@@ -67,6 +67,7 @@ struct rsrr_nep_s {
     bool autotune = false;         // RSRR_AUTOTUNE: the sampler strategy is timed and chosen
     bool tuned = false, tune_cached = false;
     int tune_strategy = -1, tune_band = -1;
+    int plan_points = 0;           // > 0 during a trial: launches are laid out as for this many points
     int32_t precond_band = -1;     // >= 0: factor only |i - j| <= precond_band of T(z_j) and iterate
     bool dense_used = false;       // the last rsrr_sample factored densely
     bool band_tc_used = false;     // the last rsrr_sample ran the tensor-core band LU

@@ -302,6 +302,7 @@ int sample_impl(rsrr_nep h, const std::vector<c128>& F, int max_refine) {
     const size_t budget = (size_t)(0.8 * (double)free_b);
     int chunk = (int)std::min<int64_t>(N, std::max<int64_t>(1, budget / per_pt));
     if ((size_t)chunk * per_pt > budget) return set_error(RSRR_ENOMEM, "one sampling point does not fit in device memory");
+    const int plan = (int)std::min<int64_t>(h->plan_points, std::max<int64_t>(1, budget / per_pt));
 
     c128* dF = nullptr;
     RSRR_TRY(dalloc_n(&dF, F.size(), st));
@@ -358,6 +359,7 @@ int sample_impl(rsrr_nep h, const std::vector<c128>& F, int max_refine) {
         }
         FactorArgs<R> fa{d, ab, (int64_t)(ab_b / es), lp, (int64_t)(lp_b / es), perm,
                          (int64_t)d.npanels * d.ldp, ipiv, info};
+        fa.plan = plan;
         evf.start(st);
         TRYC(factor_any<R>(tc, fa, np, st));
         evf.stop(st);
@@ -378,6 +380,7 @@ int sample_impl(rsrr_nep h, const std::vector<c128>& F, int max_refine) {
         if (singular) break;
         SolveArgs<R> sa{d, ab, (int64_t)(ab_b / es), lp, (int64_t)(lp_b / es), perm,
                         (int64_t)d.npanels * d.ldp, B, nl, L, nullptr};
+        sa.plan = plan;
         {
             dim3 g((unsigned)ceil_div(nl, 256), np);
             { broadcast_rhs_kernel<R><<<g, 256, 0, st>>>(h->d_U, nl, B); note_launch(); }
@@ -529,17 +532,18 @@ int sample_dense_set(const std::vector<rsrr_nep>& hs, const std::vector<c128*>& 
     size_t free_b = 0, total_b = 0;
     RSRR_CUDA(cudaMemGetInfo(&free_b, &total_b));
     const size_t budget = (size_t)(0.8 * (double)free_b);
+    std::vector<int> job_n;
+    for (int i : order) job_n.insert(job_n.end(), std::max(hs[i]->N, hs[i]->plan_points), (int)hs[i]->n);
     auto slots_of = [&](int64_t nnz) {
-        return (int)std::min<size_t>((size_t)njobs, budget / (dense_slot_bytes<R>(n_max, L_max, nnz) + dense_image_bytes<R>(n_max)));
+        return (int)std::min<size_t>(job_n.size(), budget / (dense_slot_bytes<R>(n_max, L_max, nnz) + dense_image_bytes<R>(n_max)));
     };
     if (slots_of(0) < 1) return set_error(RSRR_ENOMEM, "one dense sampling slot does not fit in device memory");
-    std::vector<int> job_n(jobs.size());
-    for (size_t i = 0; i < jobs.size(); ++i) job_n[i] = (int)hs[jobs[i].nep]->n;
     int csize = 1, grid = 1;
     RSRR_TRY(dense_plan<R>(job_n, slots_of(0), &csize, &grid));
     // A slot keeps T's values for the residuals (a full pattern makes it three times as large) only where that
     // costs no cluster.
     if (slots_of(nnz_max) < grid) nnz_max = 0;
+    grid = std::min(grid, njobs);
 
     std::vector<DenseNep> neps(nh);
     std::vector<double*> un2(nh, nullptr);
@@ -720,20 +724,25 @@ int dense_run(const std::vector<rsrr_nep>& hs, const std::vector<std::vector<c12
 //   band LU on the tensor cores (when the band suits them), band LU on the CUDA cores, the dense
 //   LU, and the iterative sampler (flexible GMRES preconditioned by the factor of a band part,
 //   the half-width p holding all but 1e-12 of the Frobenius weight of T(z_0)).
-// A dense point is timed only for n <= 2048; above that its time is extrapolated with n^3 from
-// the last dense measurement.  Decisions are cached process-wide per size bucket (n, kl, ku in
-// steps of 25 %, J, precision, ordering), so a batch of similar NEPs tunes once.
+// The trial runs one point, laid out as in the call it decides about: few points get several CTAs
+// each, many get one, and a point alone would favour the dense LU, which spreads furthest (n = 600,
+// kl = 80, 64 points: 7.9 ms dense, 5.5 ms on the band; alone the dense point is the faster one).
+// A dense point is timed only for n <= 2048; above that its time is extrapolated with n^3 and the
+// cluster's share (dense_time_share) from the last dense measurement.  Decisions are cached process-wide
+// per size bucket (n, kl, ku, points in steps of 25 %, J, precision, ordering), so a batch of similar NEPs
+// tunes once.
 // ---------------------------------------------------------------------------------------------
 namespace {
 struct TuneKey {
-    int nb, klb, kub, J, prec, natural;
+    int nb, klb, kub, J, prec, natural, ptb, dptb;
     bool operator<(const TuneKey& o) const {
-        return std::tie(nb, klb, kub, J, prec, natural) < std::tie(o.nb, o.klb, o.kub, o.J, o.prec, o.natural);
+        return std::tie(nb, klb, kub, J, prec, natural, ptb, dptb) <
+               std::tie(o.nb, o.klb, o.kub, o.J, o.prec, o.natural, o.ptb, o.dptb);
     }
 };
 std::mutex g_tune_mx;
 std::map<TuneKey, std::pair<int, int>> g_tune;   // -> (strategy, band)
-double g_dense_ms_per_n3 = 0.0;                  // last dense trial: ms / n^3
+double g_dense_ms_per_n3 = 0.0;                  // last dense trial: ms / (n^3 dense_time_share)
 
 int size_bucket(int64_t x) { return x <= 0 ? -1 : (int)std::floor(std::log((double)x) / std::log(1.25)); }
 
@@ -791,12 +800,14 @@ void apply_strategy(rsrr_nep h, int strategy, int band) {
     h->force_dense = strategy == TUNE_DENSE;
 }
 
-// Time of one sampling point (z_0) with a strategy, in ms; +inf if it fails or does not converge.
-double trial_ms(rsrr_nep h, const std::vector<c128>& F0, int strategy, int band, int max_refine) {
+// Time of one sampling point (z_0) of a call with `points` of them with a strategy, in ms; +inf if it fails or
+// does not converge.
+double trial_ms(rsrr_nep h, const std::vector<c128>& F0, int strategy, int band, int max_refine, int points) {
     const int N0 = h->N, pb = h->precond_band;
     const bool cc = h->band_cuda_cores, fd = h->force_dense;
     apply_strategy(h, strategy, band);
     h->N = 1;
+    h->plan_points = points;
     cudaEvent_t a = nullptr, b = nullptr;
     cudaEventCreate(&a);
     cudaEventCreate(&b);
@@ -816,17 +827,28 @@ double trial_ms(rsrr_nep h, const std::vector<c128>& F0, int strategy, int band,
     cudaEventDestroy(a);
     cudaEventDestroy(b);
     h->N = N0;
+    h->plan_points = 0;
     h->precond_band = pb;
     h->band_cuda_cores = cc;
     h->force_dense = fd;
     return rc == RSRR_OK ? (double)ms : INFINITY;
 }
 
-int autotune(rsrr_nep h, const std::vector<c128>& F, int max_refine) {
+// CTAs' share of a dense point's time in a call with `points` points of order n (0: no plan).
+double dense_share(rsrr_nep h, int64_t n, int points) {
+    int size = 1, count = 1;
+    const std::vector<int> job_n((size_t)points, (int)n);
+    const int rc = h->precision == RSRR_FP64 ? dense_plan<double>(job_n, points, &size, &count)
+                                             : dense_plan<float>(job_n, points, &size, &count);
+    return rc == RSRR_OK ? dense_time_share(size) : 0.0;
+}
+
+// dense_points: points that share the call's dense launch (all of a batch); the band paths run one NEP at a time
+int autotune(rsrr_nep h, const std::vector<c128>& F, int max_refine, int dense_points) {
     if (!h->autotune || h->tuned || h->tz) return RSRR_OK;
     const int64_t n = h->n, kl = h->ord.kl, ku = h->ord.ku;
     const TuneKey key{size_bucket(n), size_bucket(kl), size_bucket(ku), h->J, h->precision | (h->refine_full ? 0x100 : 0),
-                      h->ord.natural ? 1 : 0};
+                      h->ord.natural ? 1 : 0, size_bucket(h->N), size_bucket(dense_points)};
     {
         std::lock_guard<std::mutex> lk(g_tune_mx);
         auto it = g_tune.find(key);
@@ -850,22 +872,23 @@ int autotune(rsrr_nep h, const std::vector<c128>& F, int max_refine) {
     const bool band_ok = kl <= 2048 && ku <= 2048;
     if (band_ok) {
         if (h->precision != RSRR_FP64 && band_tc_eligible(n, kl, ku))
-            consider(TUNE_BAND_TC, -1, trial_ms(h, F0, TUNE_BAND_TC, -1, max_refine));
-        consider(TUNE_BAND_CC, -1, trial_ms(h, F0, TUNE_BAND_CC, -1, max_refine));
+            consider(TUNE_BAND_TC, -1, trial_ms(h, F0, TUNE_BAND_TC, -1, max_refine, h->N));
+        consider(TUNE_BAND_CC, -1, trial_ms(h, F0, TUNE_BAND_CC, -1, max_refine, h->N));
     }
     if (n <= 2048) {
-        const double ms = trial_ms(h, F0, TUNE_DENSE, -1, max_refine);
-        if (std::isfinite(ms)) g_dense_ms_per_n3 = ms / ((double)n * n * n);
+        const double ms = trial_ms(h, F0, TUNE_DENSE, -1, max_refine, dense_points);
+        const double share = dense_share(h, n, dense_points);
+        if (std::isfinite(ms) && share > 0.0) g_dense_ms_per_n3 = ms / ((double)n * n * n * share);
         consider(TUNE_DENSE, -1, ms);
     } else if (g_dense_ms_per_n3 > 0.0) {
-        consider(TUNE_DENSE, -1, g_dense_ms_per_n3 * (double)n * n * n);
+        consider(TUNE_DENSE, -1, g_dense_ms_per_n3 * (double)n * n * n * dense_share(h, n, dense_points));
     } else if (!band_ok) {
         consider(TUNE_DENSE, -1, 1e30);  // the only direct option left
     }
     int64_t p = 0;
     RSRR_TRY(dominant_band(h, F0.data(), 1e-12, &p));
     if (p < std::min(kl, ku) && p < n - 1)
-        consider(TUNE_ITER, (int)p, trial_ms(h, F0, TUNE_ITER, (int)p, max_refine));
+        consider(TUNE_ITER, (int)p, trial_ms(h, F0, TUNE_ITER, (int)p, max_refine, h->N));
     if (best_s < 0) best_s = band_ok ? TUNE_BAND_CC : TUNE_DENSE;
     apply_strategy(h, best_s, best_band);
     h->tuned = true;
@@ -881,7 +904,7 @@ int autotune(rsrr_nep h, const std::vector<c128>& F, int max_refine) {
 int sample_run(rsrr_nep h, const double* U_reim, int max_refine) {
     std::vector<std::vector<c128>> F(1);
     RSRR_TRY(sample_prepare(h, U_reim, &F[0]));
-    RSRR_TRY(autotune(h, F[0], max_refine));
+    RSRR_TRY(autotune(h, F[0], max_refine, h->N));
     h->dense_used = use_dense(h);
     if (h->dense_used) {
         std::vector<rsrr_nep> hs{h};
@@ -896,7 +919,9 @@ int sample_run(rsrr_nep h, const double* U_reim, int max_refine) {
 int sample_batch_run(const std::vector<rsrr_nep>& hs, const std::vector<const double*>& U, int max_refine) {
     std::vector<std::vector<c128>> F(hs.size());
     for (size_t i = 0; i < hs.size(); ++i) RSRR_TRY(sample_prepare(hs[i], U[i], &F[i]));
-    for (size_t i = 0; i < hs.size(); ++i) RSRR_TRY(autotune(hs[i], F[i], max_refine));
+    int points = 0;
+    for (rsrr_nep h : hs) points += h->N;
+    for (size_t i = 0; i < hs.size(); ++i) RSRR_TRY(autotune(hs[i], F[i], max_refine, points));
     std::vector<rsrr_nep> dh;
     std::vector<std::vector<c128>> dFs;
     for (size_t i = 0; i < hs.size(); ++i) {
