@@ -127,4 +127,12 @@ int dalloc_n(T** p, size_t count, cudaStream_t s) {
 
 inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
+// SMs of the current device
+inline int sm_count() {
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    return nsm;
+}
+
 }  // namespace rsrr

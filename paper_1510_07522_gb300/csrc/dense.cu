@@ -17,11 +17,12 @@ namespace rsrr {
 // sub-partitions, not the operand traffic: a 16 x 16 tile reads one byte a clock.  The tiles are
 // therefore small (256 outputs for 128 threads, four warps, two outputs a thread), and K is cut
 // over the up to eight CTAs of a cluster, which add their partial tiles through distributed shared
-// memory in a fixed order (no atomics, no workspace, the same bits on every run).  The
+// memory in a fixed order (no atomics, the same bits on every run).  A product of few tiles and long K
+// (32 x 8 x 100000) gives a tile several clusters, whose sums meet in a workspace (zgemm_fold_kernel).  The
 // FP64 products of one pass (projection and reduced solve), before with 32 x 32 tiles of two warps
 // and no K split below 512, and now: n = 9991, k_S = 133: 18.8 -> 3.1 ms; n = 900, moment scheme,
 // k_S = 45: 18.5 -> 1.0 ms; n = 5000, k_S = 48, K = 8: 29.7 -> 3.8 ms.
-// A tile is 16 x 16, or 64 x 4 for the products with a handful of columns (moments, traces).
+// A tile is 16 x 16, or 32 x 8 and 64 x 4 (8 x 32, 4 x 64) for the products with a handful of columns (rows).
 // ---------------------------------------------------------------------------------------------
 namespace {
 constexpr int BK = 16;          // K terms per shared-memory stage
@@ -38,8 +39,9 @@ struct ZgArgs {
     ZgOperand A, B;  // B's "row" is the output column
     c128* C;
     int64_t ldc, sC;
-    int M, N, K, tm, tn, split, kper;
+    int M, N, K, tm, tn, split, outer, kper;
     c128 alpha, beta;
+    c128* ws;  // outer > 1: [outer][batch][N][M] sums of the clusters' K ranges
 };
 
 __device__ __forceinline__ c128 zg_fetch(const ZgOperand& o, const c128* base, int r, int R, int k, int k_end) {
@@ -55,19 +57,19 @@ template <int BM, int BN>
 __global__ void __launch_bounds__(kZgThreads) zgemm_kernel(ZgArgs g) {
     static_assert(BM * BN == kZgTile, "two outputs a thread");
     constexpr int TX = BN / 2;  // threads across the columns; a thread owns columns tx and tx + TX
-    constexpr int NA = BM * BK / kZgThreads, NB = (BN * BK + kZgThreads - 1) / kZgThreads;
+    constexpr int NA = (BM * BK + kZgThreads - 1) / kZgThreads, NB = (BN * BK + kZgThreads - 1) / kZgThreads;
     __shared__ c128 As[BK][BM + 1];
     __shared__ c128 Bs[BK][BN + 1];
     __shared__ c128 part[kZgTile];
     const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
-    // the CTAs of a cluster are the K slices of one tile
-    const int64_t tile = blockIdx.x / g.split;
-    const int ks = (int)(blockIdx.x % g.split);
+    // the CTAs of a cluster are neighbouring K slices of one tile
+    const int64_t cl = blockIdx.x / g.split, tile = cl / g.outer;
+    const int ks = (int)(blockIdx.x % g.split), o = (int)(cl % g.outer);
     const int bm = (int)(tile % g.tm) * BM, bn = (int)((tile / g.tm) % g.tn) * BN;
     const int64_t b = tile / ((int64_t)g.tm * g.tn);
     const c128* Ab = g.A.p + b * g.A.sb;
     const c128* Bb = g.B.p + b * g.B.sb;
-    const int k_begin = min(g.K, ks * g.kper), k_end = min(g.K, k_begin + g.kper);
+    const int k_begin = (int)min((int64_t)g.K, ((int64_t)o * g.split + ks) * g.kper), k_end = min(g.K, k_begin + g.kper);
     // consecutive threads follow whichever index is contiguous in memory
     const bool a_rows = g.A.sr == 1, b_rows = g.B.sr == 1;
     c128 ra[NA], rb[NB];
@@ -75,8 +77,10 @@ __global__ void __launch_bounds__(kZgThreads) zgemm_kernel(ZgArgs g) {
 #pragma unroll
         for (int u = 0; u < NA; ++u) {
             const int idx = tid + kZgThreads * u;
-            const int i = a_rows ? idx % BM : idx / BK, k = a_rows ? idx / BM : idx % BK;
-            ra[u] = zg_fetch(g.A, Ab, bm + i, g.M, k0 + k, k_end);
+            if (idx < BM * BK) {
+                const int i = a_rows ? idx % BM : idx / BK, k = a_rows ? idx / BM : idx % BK;
+                ra[u] = zg_fetch(g.A, Ab, bm + i, g.M, k0 + k, k_end);
+            }
         }
 #pragma unroll
         for (int u = 0; u < NB; ++u) {
@@ -94,8 +98,10 @@ __global__ void __launch_bounds__(kZgThreads) zgemm_kernel(ZgArgs g) {
 #pragma unroll
         for (int u = 0; u < NA; ++u) {
             const int idx = tid + kZgThreads * u;
-            const int i = a_rows ? idx % BM : idx / BK, k = a_rows ? idx / BM : idx % BK;
-            As[k][i] = ra[u];
+            if (idx < BM * BK) {
+                const int i = a_rows ? idx % BM : idx / BK, k = a_rows ? idx / BM : idx % BK;
+                As[k][i] = ra[u];
+            }
         }
 #pragma unroll
         for (int u = 0; u < NB; ++u) {
@@ -118,6 +124,11 @@ __global__ void __launch_bounds__(kZgThreads) zgemm_kernel(ZgArgs g) {
     auto store = [&](int i, int j, c128 v) {
         const int gi = bm + i, gj = bn + j;
         if (gi >= g.M || gj >= g.N) return;
+        if (g.outer > 1) {
+            const int64_t batch = gridDim.x / ((int64_t)g.tm * g.tn * g.outer * g.split);
+            g.ws[((o * batch + b) * g.N + gj) * g.M + gi] = v;
+            return;
+        }
         c128* c = g.C + b * g.sC + gi + (int64_t)gj * g.ldc;
         v = g.alpha * v;
         *c = (g.beta.re == 0.0 && g.beta.im == 0.0) ? v : v + g.beta * (*c);
@@ -138,6 +149,18 @@ __global__ void __launch_bounds__(kZgThreads) zgemm_kernel(ZgArgs g) {
         store(e % BM, e / BM, v);
     }
     cluster.sync();  // no CTA leaves while its partial tile may still be read
+}
+
+// C = alpha sum_o ws[o] + beta C
+__global__ void zgemm_fold_kernel(ZgArgs g, int64_t per_batch, int64_t total) {
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= total) return;
+    c128 v = czero<double>();
+    for (int o = 0; o < g.outer; ++o) v = v + g.ws[o * total + idx];
+    const int64_t e = idx % per_batch;
+    c128* c = g.C + idx / per_batch * g.sC + e % g.M + e / g.M * g.ldc;
+    v = g.alpha * v;
+    *c = (g.beta.re == 0.0 && g.beta.im == 0.0) ? v : v + g.beta * (*c);
 }
 
 __global__ void scale_kernel(c128* C, int M, int N, int64_t ldc, int64_t sC, c128 beta) {
@@ -167,15 +190,23 @@ int zgemm_fp64(const Zgemm& g, cudaStream_t s) {
     a.tm = (int)ceil_div(g.M, BM);
     a.tn = (int)ceil_div(g.N, BN);
     a.alpha = g.alpha; a.beta = g.beta;
-    // K slices until every SM has two CTAs, but none shorter than one stage
-    const int64_t tiles = (int64_t)a.tm * a.tn * g.batch;
+    // K slices until every SM has two CTAs, but none shorter than one stage.  A cluster's eight slices are
+    // followed by a second level, which costs a launch and a pass over the sums: slices of 64 terms (17 us)
+    // at least to fill the SMs, of 512 to level their last wave (8 CTAs an SM).
+    const int64_t tiles = (int64_t)a.tm * a.tn * g.batch, nsm = sm_count();
     int split = 1;
-    while (split < kZgMaxSplit && tiles * split < 2 * 152 && g.K >= 2 * split * BK) split *= 2;
+    while (split < kZgMaxSplit && tiles * split < 2 * nsm && g.K >= 2 * split * BK) split *= 2;
+    auto clusters = [&](int64_t ctas, int64_t terms) { return std::min(ctas / (tiles * split), g.K / (split * terms)); };
+    const int64_t outer = split < kZgMaxSplit ? 1 : std::max({(int64_t)1, clusters(2 * nsm, 64), clusters(8 * nsm, 512)});
     a.split = split;
-    a.kper = (int)ceil_div(g.K, split);
-    if (tiles * split > INT32_MAX) return set_error(RSRR_EINVAL, "zgemm: too many tiles");
+    a.outer = (int)outer;
+    a.kper = (int)ceil_div(g.K, split * outer);
+    if (tiles * split * outer > INT32_MAX) return set_error(RSRR_EINVAL, "zgemm: too many tiles");
+    const int64_t per_batch = (int64_t)g.M * g.N, total = per_batch * g.batch;
+    a.ws = nullptr;
+    if (outer > 1) RSRR_TRY(dalloc_n(&a.ws, (size_t)(outer * total), s));
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(tiles * split));
+    cfg.gridDim = dim3((unsigned)(tiles * split * outer));
     cfg.blockDim = dim3(kZgThreads);
     cfg.stream = s;
     cudaLaunchAttribute at[1];
@@ -184,9 +215,16 @@ int zgemm_fp64(const Zgemm& g, cudaStream_t s) {
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    RSRR_CUDA(cudaLaunchKernelEx(&cfg, zgemm_kernel<BM, BN>, a));
+    cudaError_t e = cudaLaunchKernelEx(&cfg, zgemm_kernel<BM, BN>, a);
     note_launch();
-    return RSRR_OK;
+    if (outer > 1) {
+        if (e == cudaSuccess) {
+            { zgemm_fold_kernel<<<(unsigned)ceil_div(total, 256), 256, 0, s>>>(a, per_batch, total); note_launch(); }
+            e = cudaGetLastError();
+        }
+        dfree(a.ws, s);
+    }
+    return e == cudaSuccess ? RSRR_OK : set_error(RSRR_ECUDA, std::string("zgemm: ") + cudaGetErrorString(e));
 }
 }  // namespace
 
@@ -292,7 +330,10 @@ static int zgemm_dispatch(const Zgemm& g0, cudaStream_t s) {
         return RSRR_OK;
     }
     if (!g.fp64 && (g_zpath == 2 || (g_zpath == 0 && zgemm_tc_fits(g)))) return zgemm_tc(g, s);
-    return g.N <= 8 ? zgemm_fp64<64, 4>(g, s) : zgemm_fp64<16, 16>(g, s);
+    if (g.N <= 4) return zgemm_fp64<64, 4>(g, s);
+    if (g.N <= 8) return zgemm_fp64<32, 8>(g, s);
+    if (g.M <= 4) return zgemm_fp64<4, 64>(g, s);
+    return g.M <= 8 ? zgemm_fp64<8, 32>(g, s) : zgemm_fp64<16, 16>(g, s);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -342,7 +383,7 @@ void column_norms(const c128* B, int mb, int k, int64_t ld, double* out, cudaStr
 void block_norm2(const c128* A, int64_t lda, int r0, int r1, int c0, int c1, double* out, cudaStream_t s) {
     if (r1 <= r0 || c1 <= c0) return;
     const int64_t total = (int64_t)(r1 - r0) * (c1 - c0);
-    const int blocks = (int)std::min<int64_t>(4 * 152, ceil_div(total, 256));
+    const int blocks = (int)std::min<int64_t>(4 * sm_count(), ceil_div(total, 256));
     { blocknorm_kernel<<<blocks, 256, 0, s>>>(A, lda, r0, r1, c0, c1, out); note_launch(); }
 }
 

@@ -1428,13 +1428,6 @@ int set_smem(K kernel, size_t bytes, const char* name) {
     return RSRR_OK;
 }
 
-int sm_count() {
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    return nsm > 0 ? nsm : 1;
-}
-
 }  // namespace
 
 namespace {

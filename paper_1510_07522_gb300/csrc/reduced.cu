@@ -576,7 +576,7 @@ int solve_body(rsrr_nep h, int N_S, int K, double tol_gap, int cap, double* lamb
         // all points: 0.3 ms at k = 45, where the GEMM's K slices take 0.1) and wins by a factor of 2.6 from
         // there on (k = 233: 0.76 ms); from 9 columns or terms on the emulated GEMM is the faster one.
         const int64_t mctas = ceil_div(kk, kMomThreads);
-        if (2 * K <= 2 * kThin && mctas >= 2 * 152) {
+        if (2 * K <= 2 * kThin && mctas >= 2 * sm_count()) {
             moments_kernel<<<dim3((unsigned)mctas, (unsigned)ceil_div(2 * K, kThin)), kMomThreads, 0, st>>>(X, kk, np, dWt + j0, N_S, 2 * K, mom);
             note_launch();
         } else {

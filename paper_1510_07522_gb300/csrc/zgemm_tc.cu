@@ -600,12 +600,16 @@ static int oz_max(const c128* X, int64_t ld, int64_t sb, int op, int U, int V, i
 }
 
 // Worth it when the FP64 GEMM would take a while: from 0.1 GFLOP (100 us there) the emulation's
-// fixed costs (five launches, one host wait) are paid.  With at most 8 columns (or rows) the FP64
-// kernel wins at every size: the digit images cost 144 bytes of traffic for every operand entry,
-// which is then used a few times only, and a 32-column tile is mostly padding.
+// launches are paid.  With at most 8 columns (or rows) a 32-column tile is mostly padding and an operand's
+// digit images (144 bytes of traffic an entry) are used a few times only: 37 ps an operand entry, 100 where K is
+// not the contiguous index, against 6.4 to 8 ps a multiply-add on the FP64 cores.  So up to 4 columns the FP64
+// kernel always wins, up to 8 unless the other side is long and so is K, contiguous (600 x 8 x 100000: FP64 3.8 ms,
+// emulated 2.3; 600 x 8 x 10000: 0.52 and 0.39; 32 x 8 x 100000: 0.28 and 0.48; 100000 x 8 x 633, K strided: 3.6 and 6.5).
 bool zgemm_tc_fits(const Zgemm& g) {
     const double work = 8.0 * g.M * (double)g.N * g.K * g.batch;
-    return work >= 1e8 && g.K >= 16 && std::min(g.M, g.N) > 8;
+    const int thin = std::min(g.M, g.N), wide = std::max(g.M, g.N);
+    const bool k_contiguous = g.M >= g.N ? g.opA != OP_N : g.opB == OP_N;  // of the wide operand
+    return work >= 1e8 && g.K >= 16 && (thin > 8 || (thin > 4 && wide > 32 && g.K > 2048 && k_contiguous));
 }
 
 namespace {
@@ -672,7 +676,7 @@ int zgemm_tc(const Zgemm& g0, cudaStream_t s) {
     const int MT = (int)ceil_div(M, OZ_CROWS), NTt = (int)ceil_div(N, OZ_COLS);
     const int64_t tiles = (int64_t)MT * NTt * batch;
     int ksplit = 1;
-    if (tiles < 2 * 152) ksplit = (int)std::min<int64_t>(nchunk, ceil_div(2 * 152, tiles));
+    if (tiles < 2 * sm_count()) ksplit = (int)std::min<int64_t>(nchunk, ceil_div(2 * sm_count(), tiles));
     const int cper = (int)ceil_div(nchunk, ksplit);
     ksplit = (int)ceil_div(nchunk, cper);
 
