@@ -257,12 +257,22 @@ __global__ void identity_cols_kernel(c128* J, int m, int k) {
     J[idx] = (idx % m == idx / m) ? mk<double>(1.0, 0.0) : czero<double>();
 }
 
-// Y_i = A_i X for every term (CSR of the union pattern with the term's values).  Products with a real
-// entry are rounded before they are added: the coefficients of a stencil are small multiples of one
-// another, so an entry of X carries the same relative rounding into every row that uses it and the
-// nearly cancelling sum is exact; the error is A applied to a perturbation of X.  With fused
-// multiply-adds it is noise of u |A| |X|, which on the 1D acoustic problem moves the eigenvalues by
-// 1.1e-9 instead of 1e-10.  (Real entries also cost half the operations: the zero part is skipped.)
+// s + c += a x with the rounding errors of product and sum kept in c (Ogita, Rump and Oishi's Dot2)
+__device__ __forceinline__ void dot2_acc(double& s, double& c, double a, double x) {
+    const double p = __dmul_rn(a, x), e = fma(a, x, -p), t = s + p, z = t - s;
+    c += ((s - (t - z)) + (p - z)) + e;
+    s = t;
+}
+
+// Y_i = A_i X for every term (CSR of the union pattern with the term's values).  On a smooth basis a
+// stencil's sum nearly cancels, and S^H A S sees whatever was rounded at the size of |A| |X|: with fused
+// multiply-adds that moved the eigenvalues of the 1D acoustic problem by 1.1e-9, with rounded products by 1e-10,
+// at 10 to 20 % more noise in general rows.  Compensated sums carry their result's own rounding only: 0.42 u of
+// a random row's norm, against 0.6 (3 entries) to 1.6 (27) fused.  They take ten FP64 operations a product (fused:
+// two), which bound the kernel, so zeros are skipped (a term has few of the union pattern's entries), and rows
+// of more than 32 entries, no stencils, stay fused: with 80 entries a row and n = 1600 a pass took 39.8 ms
+// compensated, 39.2 fused.
+constexpr int kDot2Row = 32;
 __global__ void spmm_terms_kernel(const int64_t* rowptr, const int32_t* colind, const c128* vals, int64_t nnz,
                                   int64_t n, const c128* X, int k, c128* Y) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -270,17 +280,29 @@ __global__ void spmm_terms_kernel(const int64_t* rowptr, const int32_t* colind, 
     if (idx >= n * k) return;
     const int64_t r = idx % n, c = idx / n;
     const c128* v = vals + (int64_t)term * nnz;
-    c128 acc = czero<double>();
-    for (int64_t e = rowptr[r]; e < rowptr[r + 1]; ++e) {
-        const c128 a = v[e], x = X[colind[e] + c * n];
-        if (a.im == 0.0) {
-            acc.re = __dadd_rn(acc.re, __dmul_rn(a.re, x.re));
-            acc.im = __dadd_rn(acc.im, __dmul_rn(a.re, x.im));
-        } else {
-            cfma(acc, a, x);
+    const int64_t e0 = rowptr[r], e1 = rowptr[r + 1];
+    c128 acc = czero<double>(), low = czero<double>();
+    if (e1 - e0 > kDot2Row) {
+        for (int64_t e = e0; e < e1; ++e) {
+            const c128 a = v[e];
+            if (!cis_zero(a)) cfma(acc, a, X[colind[e] + c * n]);
+        }
+    } else {
+        for (int64_t e = e0; e < e1; ++e) {
+            const c128 a = v[e];
+            if (cis_zero(a)) continue;
+            const c128 x = X[colind[e] + c * n];
+            if (a.re != 0.0) {
+                dot2_acc(acc.re, low.re, a.re, x.re);
+                dot2_acc(acc.im, low.im, a.re, x.im);
+            }
+            if (a.im != 0.0) {
+                dot2_acc(acc.re, low.re, -a.im, x.im);
+                dot2_acc(acc.im, low.im, a.im, x.re);
+            }
         }
     }
-    Y[(int64_t)term * n * k + idx] = acc;
+    Y[(int64_t)term * n * k + idx] = acc + low;
 }
 
 std::vector<int> bit_reversed_order(int N) {
