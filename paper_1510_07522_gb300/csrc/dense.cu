@@ -20,8 +20,8 @@ namespace rsrr {
 // memory in a fixed order (no atomics, the same bits on every run).  A product of few tiles and long K
 // (32 x 8 x 100000) gives a tile several clusters, whose sums meet in a workspace (zgemm_fold_kernel).  The
 // FP64 products of one pass (projection and reduced solve), before with 32 x 32 tiles of two warps
-// and no K split below 512, and now: n = 9991, k_S = 133: 18.8 -> 3.1 ms; n = 900, moment scheme,
-// k_S = 45: 18.5 -> 1.0 ms; n = 5000, k_S = 48, K = 8: 29.7 -> 3.8 ms.
+// and no K split below 512, and now: n = 9991, k_S = 133: 18.8 -> 5.0 ms (with the inverses' W, which joined
+// them since); n = 900, moment scheme, k_S = 45: 18.5 -> 1.4 ms; n = 5000, k_S = 48, K = 8: 29.7 -> 3.5 ms.
 // A tile is 16 x 16, or 32 x 8 and 64 x 4 (8 x 32, 4 x 64) for the products with a handful of columns (rows).
 // ---------------------------------------------------------------------------------------------
 namespace {
@@ -401,8 +401,9 @@ void block_norm2(const c128* A, int64_t lda, int r0, int r1, int c0, int c1, dou
 // roots (an FP32 seed and one third-order step each, four dependent operations).  With the angle in
 // FP32 a whole pass took 0.3 to 1.2 % less (70.2 instead of 70.7 ms at n = 900), but a pair kept 2^-23 of its
 // inner product and two columns needed a third sweep.
-// One round then takes 3.0 us at 212 columns, from 6.1 us; a whole pass's sweeps: n = 900, k_S = 233:
-// 50.7 -> 18.7 ms, n = 40000: 88.9 -> 43.5 ms (there also without J in the projection, see project.cu).
+// One round took 3.0 us at 212 columns, from 6.1 us (with the angle still in FP32); a whole pass's sweeps: n = 900,
+// k_S = 233: 50.7 -> 18.7 ms, n = 40000: 88.9 -> 43.5 ms (there also without J in the projection, see project.cu), and
+// with the rounds over the columns above the floor only, in FP64: 11.9 and 20.9 ms.
 // The norms that decide about the floor are al - Re(conj(T) g) and be + Re(conj(T) g), T the rotation's
 // complex tangent: to rounding in the larger one (of two nearly parallel columns the smaller one keeps few digits;
 // such a pair is rotated, so another sweep follows with fresh norms).  Every pair forms its own from the columns.

@@ -1093,10 +1093,10 @@ __device__ void solve_one(const DenseJob<R>& J, int l_lo, int l_hi, unsigned cha
 }
 
 // ------------------------------------------------------------------------------------------
-// Fused dense sampling.  Per job (point j of NEP E), in the CTA's slot:
+// Fused dense sampling.  Per job (point j of NEP E), in the cluster's slot:
 //   zero the matrix, scatter T(z_j) = sum_i f_i(z_j) A_i (precision R) and the FP64 column
 //   sums |T| (for ||T||_1); factor; x = U; solve; X = x in S_hat (FP64); then
-//   r = U - T X in FP64 from the CSR values (T recomputed from the f_i), eta per column,
+//   r = U - T X in FP64 from T's CSR values (kept from the assembly, or recomputed), eta per column,
 //   and refinement X += (LU)^{-1} r while the stopping rule of the band path asks for it.
 // ------------------------------------------------------------------------------------------
 constexpr int kMaxL = 256;

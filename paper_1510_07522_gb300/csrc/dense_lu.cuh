@@ -3,9 +3,9 @@
 // dense or with a band as wide as n, e.g. the time-delay NEPs whose delay term is a random
 // sparse matrix).
 //
-// One CTA owns one sampling point for the whole factorisation: a persistent launch hands out
-// points largest-first from a device counter, so a batch of uneven problems (many NEPs of
-// different n, all their points) runs in one launch without cross-CTA synchronisation.
+// One thread-block cluster (1, 2, 4 or 8 CTAs) owns one sampling point from assembly to refinement: a
+// persistent launch hands out points largest-first from a device counter, so a batch of uneven problems
+// (many NEPs of different n, all their points) runs in one launch, synchronised within clusters only.
 //
 // Storage of one point:
 //   a      n x n column-major, leading dimension lda.  On exit the upper triangle holds U and

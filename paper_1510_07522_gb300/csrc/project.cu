@@ -320,9 +320,9 @@ std::vector<int> bit_reversed_order(int N) {
 }
 
 // Householder QR of A (rows x cols, ld lda) in place: R in the upper triangle, the
-// reflectors below it, T factors of each panel in Tall.  When stop2 >= 0 the factorisation
-// stops after the first panel whose remaining trailing block has squared Frobenius norm
-// <= stop2.  Returns the number of rows of R produced in *kk and panels in *npan.
+// reflectors below it, T factors of each panel in Tall.  With a stop rule (below) the factorisation
+// ends at the first panel that meets it.  Returns the number of rows of R produced in *kk and
+// panels in *npan.
 struct HqrWork {
     c128 *V = nullptr, *W = nullptr, *W2 = nullptr, *tau = nullptr, *Tall = nullptr, *row = nullptr;
     double *part = nullptr, *dnorm = nullptr;
